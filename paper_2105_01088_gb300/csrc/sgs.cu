@@ -653,6 +653,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
         CUDA_TRY(c, cudaMemcpyAsync(I.gamma, o.gamma0, M * nn * sizeof(double), cudaMemcpyHostToDevice, st));
     CUDA_TRY(c, cudaMemsetAsync(I.dgamma, 0, M * nn * sizeof(double), st));
     CUDA_TRY(c, cudaMemsetAsync(I.sq, 0, M * sizeof(int), st));
+    CUDA_TRY(c, cudaMemsetAsync(I.eigscratch, 0, (6 * (size_t)(2 * M) * (2 * M) + 8 * 2 * M) * sizeof(double), st));
     if (P > 0) {
         CUDA_TRY(c, cudaMemcpyAsync(I.pa, pa.data(), P * sizeof(int), cudaMemcpyHostToDevice, st));
         CUDA_TRY(c, cudaMemcpyAsync(I.pb, pb.data(), P * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -832,6 +833,7 @@ void set_kernel_attributes() {
     raise_smem_limit(gj_panel_kernel, optin);
     raise_smem_limit(pf_panel_kernel, optin);
     raise_smem_limit(renyi_pf_kernel, optin);
+    raise_smem_limit(amp_solve_kernel, optin);
     raise_smem_limit(gemm_tma_kernel<TC_TF32>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_BF16>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_3XTF32>, optin);
@@ -1121,7 +1123,7 @@ cudaError_t pair_products(sgs_ctx* c, Instance& I, cudaStream_t st) {
 // amplitude solve (A6) on the instance's G, h; E -> Eout
 cudaError_t amplitudes(Instance& I, double* Eout, cudaStream_t st) {
     AmpArgs aa{I.M, I.Gm, I.hm, I.eigscratch, Eout, I.lam, I.lt, I.coef, I.cmode, 1e-12, I.err};
-    amp_solve_kernel<<<1, 256, 0, st>>>(aa);
+    amp_solve_kernel<<<1, AMP_THREADS, amp_smem(I.M), st>>>(aa);
     counted();
     return cudaGetLastError();
 }
@@ -1880,7 +1882,7 @@ sgs_status sgs_health(sgs_ctx* c, int instance, double* out) {
     cudaStream_t st = c->stream;
     CUDA_TRY(c, cudaStreamSynchronize(st));
     // Gamma_mu^2 -> s0, then max |Gamma^2 + 1|, non-finite entries of Gamma, and the extreme eigenvalues of G
-    // of the last amplitude solve (diagonal of its Jacobi result)
+    // of the last amplitude solve (the diagonal of a Jacobi result: that solve's, or gram_eig_kernel's)
     GemmBatch g = gb_basic(n, n, n, I.p_gamma, n, I.p_gamma, n, I.p_s[0], n, M);
     const bool prof = c->prof;
     c->prof = false;
@@ -1894,6 +1896,8 @@ sgs_status sgs_health(sgs_ctx* c, int instance, double* out) {
         if (!I.corr_scratch) { c->err = "device allocation failed"; return SGS_ENOMEM; }
         I.corr_cap = 8;
     }
+    gram_eig_kernel<<<1, AMP_THREADS, 0, st>>>(I.eigscratch, M);
+    counted();
     health_kernel<<<1, 1024, 0, st>>>(I.s[0], I.gamma, M * nn, n, I.eigscratch, 2 * M, I.Ecur, I.corr_scratch);
     counted();
     CUDA_TRY(c, cudaMemcpyAsync(out, I.corr_scratch, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
