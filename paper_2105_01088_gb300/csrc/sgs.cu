@@ -832,6 +832,8 @@ void set_kernel_attributes() {
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     raise_smem_limit(gj_panel_kernel, optin);
     raise_smem_limit(pf_panel_kernel, optin);
+    raise_smem_limit(gj_cluster_kernel, optin);
+    raise_smem_limit(pf_cluster_kernel, optin);
     raise_smem_limit(renyi_pf_kernel, optin);
     raise_smem_limit(amp_solve_kernel, optin);
     raise_smem_limit(gemm_tma_kernel<TC_TF32>, optin);
@@ -845,6 +847,79 @@ void set_kernel_attributes() {
 }
 
 inline cudaError_t tma_product(const TmaBatch& t, int kind, cudaStream_t st) { return gemm_tma(t, kind, st); }
+
+// A launch with clusters of C CTAs along x.
+template <class... KArgs, class... Args>
+cudaError_t launch_cluster(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem, int C, cudaStream_t st,
+                           Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// threads of a cluster panel's CTA of ch rows (four or eight warps of rows, one more), and threads per
+// row: a power of two up to 8 that gives each of the SM's four FP64 units a warp or two
+int cluster_threads(int ch) { return ch > 128 ? 288 : 160; }
+int threads_per_row(int ch) {             // the power's exponent
+    int lg = 0;
+    while (lg < 3 && (ch << (lg + 1)) <= 128) lg++;
+    return lg;
+}
+
+// CTAs per matrix of the panels' cluster forms (0: the one-CTA form).  One CTA per matrix leaves SMs idle
+// below a few hundred matrices and pays one SM's FP64 pipe per column; more CTAs than SMs (152) only
+// share them.  Panels of 16 columns, one-CTA form against the best C, us: n = 64, 6 matrices 53 / 32
+// (C = 8); n = 164, 15: 59 / 36 (8); n = 244, 60: 65 / 47 (4); n = 388, 45: 90 / 53 (8); n = 804, 60:
+// 151 / 90 (4, 8); n = 2000, 14 (12 columns): 237 / 61 (8); at n = 512, 248 in a step, where another
+// stream shares the SMs, the one-CTA form stays ahead.
+int gj_cluster(int n, int batch, int bb) {
+    for (int C = 8; C >= 2; C /= 2)
+        if (batch * C <= 320 && n >= 8 * C && gjc_smem(bb, C, (n + C - 1) / C) <= 200 * 1024) return C;
+    return 0;
+}
+// 16 steps on `live` rows, one-CTA form against the best C, us: 64 rows, 3 matrices 153 / 80 (4); 164, 10:
+// 186 / 93 (8); 244, 105: 258 / 184 (4); 388, 36: 400 / 143 (8); 804, 105: 794 / 625 (4); 420, 105: 432 / 280;
+// 2000, 21: 1588 / 436 (8); 512, 465: 1295 / 1238 (4), within the noise of a step.
+int pf_cluster(int live, int batch, int bs) {
+    for (int C = 8; C >= 2; C /= 2)
+        if (batch * C <= 500 && live >= 4 * C && pfc_smem(bs, C, (live + C - 1) / C) <= 220 * 1024) return C;
+    return 0;
+}
+
+// the Gauss-Jordan panel of columns a.k0 .. a.k0 + a.bb - 1
+cudaError_t gj_panel(const GJPanelArgs& a, int batch, cudaStream_t st) {
+    counted();
+    const int C = gj_cluster(a.n, batch, a.bb);
+    if (C > 0) {
+        const int ch = (a.n + C - 1) / C;
+        return launch_cluster(gj_cluster_kernel, batch * C, cluster_threads(ch), gjc_smem(a.bb, C, ch), C, st, a, C, ch,
+                              threads_per_row(ch));
+    }
+    gj_panel_kernel<<<batch, 512, (size_t)a.n * (a.bb + 1) * sizeof(double) + a.bb * sizeof(double), st>>>(a);
+    return cudaGetLastError();
+}
+
+// the Pfaffian panel of elimination steps a.k0 / 2 .. a.k0 / 2 + a.bs - 1
+cudaError_t pf_panel(const PfPanelArgs& a, int batch, cudaStream_t st) {
+    counted();
+    const int C = pf_cluster(a.n - a.k0, batch, a.bs);
+    if (C > 0) {
+        const int ch = (a.n - a.k0 + C - 1) / C;
+        return launch_cluster(pf_cluster_kernel, batch * C, cluster_threads(ch), pfc_smem(a.bs, C, ch), C, st, a, C, ch,
+                              threads_per_row(ch));
+    }
+    pf_panel_kernel<<<batch, PF_PANEL_THREADS, (4 * (size_t)a.n + 4 * a.bsmax) * sizeof(double), st>>>(a);
+    return cudaGetLastError();
+}
 
 // every FP64 product of the library goes through here; flops = algorithmic work of
 // the launch (antisymmetric outputs count half), < 0 = not profiled.  With slice
@@ -954,10 +1029,7 @@ cudaError_t gj_recurse(sgs_ctx* c, int n, int batch, int leaf, int c0, int c1, d
                        const OzBuf* oz) {
     if (c1 - c0 <= leaf) {
         const int bb = c1 - c0;
-        GJPanelArgs a{W, T, piv, logdet, dsign, err, n, c0, bb, tiny};
-        gj_panel_kernel<<<batch, 512, (size_t)n * (bb + 1) * sizeof(double) + bb * sizeof(double), st>>>(a);
-        counted();
-        return cudaGetLastError();
+        return gj_panel({W, nullptr, piv, logdet, dsign, err, n, c0, bb, tiny}, batch, st);
     }
     const int leaves = (c1 - c0 + leaf - 1) / leaf;
     const int m = c0 + ((leaves + 1) / 2) * leaf;
@@ -980,7 +1052,6 @@ cudaError_t launch_gj_recursive(sgs_ctx* c, int n, int batch, int leaf, double**
 cudaError_t launch_pf(sgs_ctx* c, int n, int batch, int bsmax, double** Y, double** TU, double** PK, double** upA,
                       double** upB, double** upC, double* logabs, double* phase, int* err, cudaStream_t st,
                       const OzBuf* oz = nullptr) {
-    const size_t smem = (4 * (size_t)n + 4 * bsmax) * sizeof(double);
     set_kernel_attributes();
     for (int k0 = 0; k0 < n; k0 += 2 * bsmax) {
         const int bs = std::min(bsmax, (n - k0) / 2);
@@ -994,8 +1065,8 @@ cudaError_t launch_pf(sgs_ctx* c, int n, int batch, int bsmax, double** Y, doubl
             const OzLayout L = oz_layout(g.m, g.n, g.k, *oz, g.batch);
             a.sa = L.as; a.sb = L.bs; a.ea = L.ea; a.eb = L.eb; a.mp = L.mp; a.np = L.np;
         }
-        pf_panel_kernel<<<batch, PF_PANEL_THREADS, smem, st>>>(a);
-        counted();
+        const cudaError_t pe = pf_panel(a, batch, st);
+        if (pe != cudaSuccess) return pe;
         if (e0 >= n) break;
         g.offA = (long long)e0 * 4 * bs;
         g.offB = (long long)e0 * 4 * bs;
