@@ -518,6 +518,41 @@ __global__ void __launch_bounds__(256) gj_update_slice_kernel(double* const* W, 
     }
 }
 
+// A delayed Gauss-Jordan update of small work on the FP64 pipe, in place: columns t0 .. t0 + w - 1 of every
+// W take W[:, t] += W[:, p0 .. p0 + K - 1] T with T = their rows p0 .. p0 + K - 1 before the update, which
+// are replaced by the product.  A CTA takes WT columns whole (so no other CTA reads the rows it replaces):
+// T in shared memory, a thread per row.  Grid (ceil(w / WT), batch); K <= GJ_SMALL_K.  One launch, where
+// the emulated form takes a slicing launch and a product tile's fixed time.
+#define GJ_SMALL_K 64
+template <int WT>
+__global__ void __launch_bounds__(256) gj_update_small_kernel(double* const* W, int n, int p0, int K, int t0, int w) {
+    __shared__ double T[GJ_SMALL_K][WT];
+    double* a = W[blockIdx.y];
+    const int c0 = t0 + blockIdx.x * WT, cn = min(WT, t0 + w - c0);
+    for (int e = threadIdx.x; e < K * WT; e += blockDim.x) {
+        const int k = e / WT, q = e % WT;
+        T[k][q] = q < cn ? a[(size_t)(p0 + k) * n + c0 + q] : 0.0;
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+        const double* x = a + (size_t)r * n + p0;
+        double* y = a + (size_t)r * n + c0;
+        const bool pivot = r >= p0 && r < p0 + K;
+        double acc[WT];
+#pragma unroll
+        for (int q = 0; q < WT; q++) acc[q] = (pivot || q >= cn) ? 0.0 : y[q];
+#pragma unroll 8
+        for (int k = 0; k < K; k++) {
+            const double v = x[k];
+#pragma unroll
+            for (int q = 0; q < WT; q++) acc[q] = fma(v, T[k][q], acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < WT; q++)
+            if (q < cn) y[q] = acc[q];
+    }
+}
+
 // Undo the row interchanges of Gauss-Jordan: inverse = X P, i.e. the column
 // interchanges applied in reverse order.  perm[c] = source column of column c.
 // One block per matrix: the pivots and the permutation in shared memory (2 n ints of dynamic

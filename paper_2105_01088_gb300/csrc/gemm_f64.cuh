@@ -230,6 +230,121 @@ inline cudaError_t gemm_f64(const GemmBatch& g, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// The same product for small work: a 16 x 8 output tile per CTA, one element per thread, K in slabs of 32
+// (the next slab's loads in flight while one is multiplied).  A warp's FMA occupies its quarter of the SM
+// for 64 clocks and the SM takes one per 19, so four warps of one accumulator each keep the FP64 pipe
+// full, and small tiles spread little work over all SMs.  Bound by the FP64 pipe.
+#define GSM 16
+#define GSN 8
+#define GSK 32
+template <int TA, int TB>
+__global__ void __launch_bounds__(128) gemm_f64_small_kernel(GemmBatch g) {
+    __shared__ double As[2][GSK][GSM + 1], Bs[2][GSK][GSN + 1];
+    const int b = blockIdx.y, ntn = (g.n + GSN - 1) / GSN;
+    const int m0 = (blockIdx.x / ntn) * GSM, n0 = (blockIdx.x % ntn) * GSN, tid = threadIdx.x;
+    const bool skew = g.mode == GEMM_SKEW;
+    if (skew && m0 + GSM <= n0) return;                 // above the diagonal: written as a mirror
+    const bool active = (g.active_flag == nullptr) || (g.active_flag[b] > g.active_cmp);
+    const int rr = tid >> 3, cc = tid & 7, r = m0 + rr, c = n0 + cc;
+    double acc = 0.0;
+    if (active && g.k > 0) {
+        const double* Ab = g.A[b] + g.offA;
+        const double* A2b = g.A2 ? g.A2[b] + g.offA : nullptr;
+        const double* Bb = g.B[b] + g.offB;
+        const double* B2b = g.B2 ? g.B2[b] + g.offB : nullptr;
+        double ra[4], rb[2];
+        // loads run along the operand's contiguous index
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int x = tid + 128 * e, kk = TA ? x >> 4 : x & 31, i = TA ? x & 15 : x >> 5;
+                const int gr = m0 + i, gk = k0 + kk;
+                ra[e] = 0.0;
+                if (gr < g.m && gk < g.k) {
+                    const long long off = TA ? (long long)gk * g.lda + gr : (long long)gr * g.lda + gk;
+                    ra[e] = A2b ? fma(g.sA2, A2b[off], Ab[off]) : Ab[off];
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const int x = tid + 128 * e, kk = TB ? x & 31 : x >> 3, j = TB ? x >> 5 : x & 7;
+                const int gc = n0 + j, gk = k0 + kk;
+                rb[e] = 0.0;
+                if (gc < g.n && gk < g.k) {
+                    const long long off = TB ? (long long)gc * g.ldb + gk : (long long)gk * g.ldb + gc;
+                    rb[e] = B2b ? fma(g.sB2, B2b[off], Bb[off]) : Bb[off];
+                }
+            }
+        };
+        auto store = [&](int s) {
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int x = tid + 128 * e;
+                As[s][TA ? x >> 4 : x & 31][TA ? x & 15 : x >> 5] = ra[e];
+            }
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const int x = tid + 128 * e;
+                Bs[s][TB ? x & 31 : x >> 3][TB ? x >> 5 : x & 7] = rb[e];
+            }
+        };
+        load(0);
+        store(0);
+        __syncthreads();
+        for (int k0 = 0, s = 0; k0 < g.k; k0 += GSK, s ^= 1) {
+            const bool more = k0 + GSK < g.k;
+            if (more) load(k0 + GSK);
+            const int kn = min(GSK, g.k - k0);
+            if (kn == GSK) {
+#pragma unroll 8
+                for (int kk = 0; kk < GSK; kk++) acc = fma(As[s][kk][rr], Bs[s][kk][cc], acc);
+            } else {
+                for (int kk = 0; kk < kn; kk++) acc = fma(As[s][kk][rr], Bs[s][kk][cc], acc);
+            }
+            if (more) store(s ^ 1);
+            __syncthreads();
+        }
+    }
+    if (r >= g.m || c >= g.n || (skew && r < c)) return;
+    const double* Cinb = g.Cin ? g.Cin[b] + g.offCin : nullptr;
+    const double* Cin2b = g.Cin2 ? g.Cin2[b] + g.offCin : nullptr;
+    double* Cb = g.C[b] + g.offC;
+    const long long ci = g.cin_trans ? (long long)c * g.ldcin + r : (long long)r * g.ldcin + c;
+    double v;
+    if (!active) {
+        v = Cinb ? Cinb[ci] : 0.0;
+    } else {
+        const double alpha = g.alpha * (g.alpha_b ? g.alpha_b[b] : 1.0);
+        v = alpha * acc;
+        if (Cinb && g.beta != 0.0 && !(g.mode == GEMM_GJ && !g.gj_acc && r >= g.gj_k0 && r < g.gj_k0 + g.gj_b))
+            v = fma(g.beta, Cinb[ci], v);
+        if (Cin2b) v = fma(g.beta2, Cin2b[(long long)r * g.ldcin + c], v);
+        if (r == c) v += g.diag;
+    }
+    if (skew) {
+        if (r == c) v = 0.0;
+        Cb[(long long)r * g.ldc + c] = v;
+        if (r != c) Cb[(long long)c * g.ldc + r] = -v;
+    } else if (g.mode != GEMM_GJ || !g.gj_cols || c < g.gj_k0 || c >= g.gj_k0 + g.gj_b) {
+        Cb[(long long)r * g.ldc + c] = v;
+    }
+}
+
+inline cudaError_t gemm_f64_small(const GemmBatch& g, cudaStream_t st) {
+    if (g.batch <= 0 || g.m <= 0 || g.n <= 0) return cudaSuccess;
+    const dim3 grid((unsigned)(((g.m + GSM - 1) / GSM) * ((g.n + GSN - 1) / GSN)), g.batch);
+    if (!g.transA && !g.transB) gemm_f64_small_kernel<0, 0><<<grid, 128, 0, st>>>(g);
+    else if (!g.transA && g.transB) gemm_f64_small_kernel<0, 1><<<grid, 128, 0, st>>>(g);
+    else if (g.transA && !g.transB) gemm_f64_small_kernel<1, 0><<<grid, 128, 0, st>>>(g);
+    else gemm_f64_small_kernel<1, 1><<<grid, 128, 0, st>>>(g);
+    return cudaGetLastError();
+}
+
+// FMAs of a product (an antisymmetric result: its lower half)
+inline double gemm_fmas(const GemmBatch& g) {
+    return (double)g.batch * g.m * g.n * g.k * (g.mode == GEMM_SKEW ? 0.5 : 1.0);
+}
+
 inline GemmBatch gemm_defaults() {
     GemmBatch g{};
     g.alpha = 1.0; g.beta = 0.0; g.diag = 0.0; g.sA2 = 0.0; g.sB2 = 0.0; g.Cin2 = nullptr; g.beta2 = 0.0;

@@ -95,6 +95,7 @@ template <int BN, int EPIW, int RING, bool BDBL> struct OzCfg {
 struct OzBuf {
     uint8_t* base = nullptr;
     size_t bytes = 0;
+    bool small_fma = false;        // products of small work run on the FP64 pipe (small_product)
 };
 
 // K-major operand rows as seen by the slicer: element (r, k) of op(X) is

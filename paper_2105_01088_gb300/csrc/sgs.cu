@@ -792,6 +792,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
             I.u_ok = true;
         }
     }
+    I.oz.small_fma = I.oz2.small_fma = true;
     if (I.fp64_path == SGS_FP64_EMULATED) {
         // emulated FP64 products: slice scratch for one batch chunk, and one for the side stream
         const size_t b = oz_scratch_bytes(n, M, I.oz_cap, Pc);
@@ -921,6 +922,20 @@ cudaError_t pf_panel(const PfPanelArgs& a, int batch, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// Whether an instance's product is small enough for the FP64 pipe, where one launch over all SMs does it
+// (a 64 x 64 x 64 product of 4 states in 3.5 us) before the emulated form's three launches, 25 to 40 us on
+// few tiles, are through.  Measured with the line at 0 (all emulated), 1, 3, 6 and 12 million FMAs: four steps
+// at 2N = 64, M = 4 take 4.71, 3.95, 2.50, 2.49 and 2.51 ms; serving at 2N up to 164 4.20, 4.19, 4.21, 4.24
+// and 4.33.
+constexpr double SMALL_FMAS = 3e6;
+bool small_product(const OzBuf* oz, const GemmBatch& g) { return oz && oz->small_fma && gemm_fmas(g) <= SMALL_FMAS; }
+// the same for a Gauss-Jordan update (one launch against two, 18 us on few tiles): (E, G, h) at 2N = 164, M = 6
+// with the line at 0, 1, 2 and 4 million: 1.70, 1.58, 1.50, 1.49 ms; at 2N = 388, M = 10 no difference
+constexpr double SMALL_GJ_FMAS = 4e6;
+bool small_gj_update(const OzBuf* oz, int n, int batch, int K, int w) {
+    return oz && oz->small_fma && K <= GJ_SMALL_K && (double)batch * n * w * K <= SMALL_GJ_FMAS;
+}
+
 // every FP64 product of the library goes through here; flops = algorithmic work of
 // the launch (antisymmetric outputs count half), < 0 = not profiled.  With slice
 // scratch (an instance or call on the emulated path) the product runs emulated on
@@ -929,13 +944,14 @@ cudaError_t pf_panel(const PfPanelArgs& a, int batch, cudaStream_t st) {
 // them, so the product's time below excludes the slicing)
 inline cudaError_t gemm(sgs_ctx* c, const GemmBatch& g, cudaStream_t st, double flops, const OzBuf* oz = nullptr,
                         int* oz_err = nullptr, bool presliced = false) {
-    const bool emulate = oz && oz->base && oz_err;
+    const bool small = small_product(oz, g);
+    const bool emulate = oz && oz->base && oz_err && !small;
     if (emulate) set_kernel_attributes();             // the kernels' shared-memory limits (once)
     if (emulate && !presliced) for (int i = oz_launches(g, *oz); i > 0; i--) counted();
     else counted();
     auto run = [&]() {
         if (emulate && presliced) return gemm_oz_presliced(g, *oz, oz_err, st);
-        return emulate ? gemm_oz(g, *oz, oz_err, st) : gemm_f64(g, st);
+        return emulate ? gemm_oz(g, *oz, oz_err, st) : small ? gemm_f64_small(g, st) : gemm_f64(g, st);
     };
     if (c && c->prof && flops >= 0.0) {
         cudaEvent_t a = c->next_event(), b = c->next_event();
@@ -951,6 +967,15 @@ inline cudaError_t gemm(sgs_ctx* c, const GemmBatch& g, cudaStream_t st, double 
 }
 inline cudaError_t gemm(sgs_ctx* c, Instance& I, const GemmBatch& g, cudaStream_t st, double flops) {
     return gemm(c, g, st, flops, I.oz_side ? &I.oz2 : &I.oz, I.err);
+}
+
+// The scratch as the products behind S^{-1} and Im Delta take it: in the mixed forms all of them stay
+// emulated, whatever their size.  There a last bit of S^{-1} can turn an fp32 or TF32 rounding, which moves
+// the state by up to 1e-7 of a step, so the line of small_product would show in the results.
+OzBuf factor_oz(const Instance& I, bool side) {
+    OzBuf o = side ? I.oz2 : I.oz;
+    o.small_fma = I.prec == SGS_FP64;
+    return o;
 }
 
 GemmBatch gb_basic(int m, int n, int k, double** A, int lda, double** B, int ldb, double** C, int ldc, int batch) {
@@ -1003,7 +1028,16 @@ bool gj_presliced(const OzBuf* oz, const int* err, int n, int batch, int K, int 
 cudaError_t gj_update(sgs_ctx* c, int n, int batch, double** W, double** Tup, int p0, int K, int t0, int w,
                       cudaStream_t st, const OzBuf* oz, int* err) {
     const GemmBatch g = gj_update_batch(n, batch, W, Tup, p0, K, t0, w);
-    const bool presliced = gj_presliced(oz, err, n, batch, K, w);
+    if (small_gj_update(oz, n, batch, K, w)) {
+        // two columns per CTA until there are CTAs for every SM
+        if (batch * ((w + 3) / 4) < 152)
+            gj_update_small_kernel<2><<<dim3((w + 1) / 2, batch), 256, 0, st>>>(W, n, p0, K, t0, w);
+        else
+            gj_update_small_kernel<4><<<dim3((w + 3) / 4, batch), 256, 0, st>>>(W, n, p0, K, t0, w);
+        counted();
+        return cudaGetLastError();
+    }
+    const bool presliced = !small_product(oz, g) && gj_presliced(oz, err, n, batch, K, w);
     if (presliced) {
         const OzLayout L = oz_layout(n, w, K, *oz, batch);
         gj_update_slice_kernel<<<dim3((L.mp + GJ_SLICE_ROWS - 1) / GJ_SLICE_ROWS + 1, batch), 256, 0, st>>>(
@@ -1060,7 +1094,9 @@ cudaError_t launch_pf(sgs_ctx* c, int n, int batch, int bsmax, double** Y, doubl
         GemmBatch g = gb_basic(n - e0, n - e0, 4 * bs, upA, 4 * bs, upB, 4 * bs, upC, n, 2 * batch);
         // emulated update: the panel writes the operands' slices itself when the whole batch
         // fits the slice scratch (no FP64 packs, no slicing launches)
-        const bool sliced = e0 < n && oz && oz->base && err && bs % 4 == 0 && oz_chunk_entries(g, *oz) >= g.batch;
+        g.mode = GEMM_SKEW;
+        const bool sliced = e0 < n && oz && oz->base && err && bs % 4 == 0 && !small_product(oz, g) &&
+                            oz_chunk_entries(g, *oz) >= g.batch;
         if (sliced) {
             const OzLayout L = oz_layout(g.m, g.n, g.k, *oz, g.batch);
             a.sa = L.as; a.sb = L.bs; a.ea = L.ea; a.eb = L.eb; a.mp = L.mp; a.np = L.np;
@@ -1077,7 +1113,6 @@ cudaError_t launch_pf(sgs_ctx* c, int n, int batch, int bsmax, double** Y, doubl
         // upper triangle current, so Cin(r, c) = -Y[c][r]: read transposed with beta = -1
         g.Cin = (const double* const*)upC; g.offCin = g.offC; g.ldcin = n; g.beta = -1.0;
         g.cin_trans = 1;
-        g.mode = GEMM_SKEW;
         const double m2 = (double)(n - e0) * (n - e0);
         const cudaError_t e = gemm(c, g, st, m2 * 4.0 * bs * 2 * batch, oz, err, sliced);
         if (e != cudaSuccess) return e;
@@ -1106,7 +1141,8 @@ cudaError_t pair_inverse(sgs_ctx* c, Instance& I, cudaStream_t st) {
     const size_t nn = (size_t)I.n * I.n;
     pair_sum_kernel<<<dim3(grid_chunks(nn, 256, 64), I.ccnt()), 256, 0, st>>>(I.dev(), I.work);
     counted();
-    return inverse_range(c, I, 0, I.ccnt(), st, &I.oz);
+    const OzBuf oz = factor_oz(I, false);
+    return inverse_range(c, I, 0, I.ccnt(), st, &oz);
 }
 
 // Im Delta^{a,b} = (G_a - G_b) S^{-1} of pairs p0 .. p0 + cnt - 1 of the current chunk (side: with
@@ -1117,10 +1153,8 @@ cudaError_t delta_range(sgs_ctx* c, Instance& I, int p0, int cnt, cudaStream_t s
     g.A2 = (const double* const*)(I.p_gb + I.coff() + p0); g.sA2 = -1.0;
     g.mode = GEMM_SKEW;
     g.b_antisym = 1;        // S^{-1} (antisymmetric up to the inversion's rounding)
-    I.oz_side = side;
-    const cudaError_t e = gemm(c, I, g, st, (double)n * n * n * cnt);   // antisymmetric product: half of 2 n^3
-    I.oz_side = 0;
-    return e;
+    const OzBuf oz = factor_oz(I, side != 0);
+    return gemm(c, g, st, (double)n * n * n * cnt, &oz, I.err);      // antisymmetric product: half of 2 n^3
 }
 
 // phase Pfaffians Pf(Gamma_0 + Delta^{a,b}) of the pairs without the reference state
@@ -1156,8 +1190,9 @@ cudaError_t pair_factors(sgs_ctx* c, Instance& I, cudaStream_t st, bool split = 
     counted();
     if ((e = cudaEventRecord(I.ev_fork, st)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(I.st2, I.ev_fork, 0)) != cudaSuccess) return e;
-    if ((e = inverse_range(c, I, 0, PA, st, &I.oz)) != cudaSuccess) return e;
-    if ((e = inverse_range(c, I, PA, PB, I.st2, &I.oz2)) != cudaSuccess) return e;
+    const OzBuf oz = factor_oz(I, false), oz2 = factor_oz(I, true);
+    if ((e = inverse_range(c, I, 0, PA, st, &oz)) != cudaSuccess) return e;
+    if ((e = inverse_range(c, I, PA, PB, I.st2, &oz2)) != cudaSuccess) return e;
     if ((e = delta_range(c, I, 0, PA, st, 0)) != cudaSuccess) return e;
     if ((e = delta_range(c, I, PA, PB, I.st2, 1)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(I.ev_join, I.st2)) != cudaSuccess) return e;
