@@ -10,7 +10,10 @@
 // inverse iteration, and back.  All of it sits in shared memory.  "None can be dropped" is
 // decided by bounds: lambda_min >= 1 / tr(G^{-1}) and lambda_max <= tr(G), both traces at
 // hand after the factorisation, so tr(G) tr(G^{-1}) < AMP_COND (1e8, four orders inside
-// the cut of 1e-12) suffices.
+// the cut of 1e-12) suffices.  The route is for states with order-one amplitudes: its errors are
+// normwise, u |lambda|, while c_mu divides by lambda_mu, and on a G that is diagonal to rounding
+// (random states: overlaps down to 1e-40) Jacobi leaves exact zeros, which freeze a state.  So
+// overlaps all below AMP_SMALL, or an amplitude below AMP_SMALL times the largest, go to Jacobi.
 //
 // Otherwise (nearly dependent states, NaN) the solve takes amp_jacobi: the M x M Hermitian
 // pair (G, h) is embedded as the real symmetric 2M x 2M pair [[Re, -Im], [Im, Re]] (every
@@ -129,6 +132,7 @@ __device__ __forceinline__ void amp_embed(const double* X, double* R, int M) {
 
 #define AMP_THREADS 256
 #define AMP_COND 1e8
+#define AMP_SMALL 1e-6
 
 // lr (2M: real and imaginary parts of a solution lambda) and E from two Jacobi eigenproblems on
 // the real embedding; false if nothing is kept of G.  scratch: 6 (2M)^2 + 8 (2M) doubles (global);
@@ -255,7 +259,8 @@ __device__ __forceinline__ bool amp_posdef(const double* d, const double* e2, in
 }
 
 // The direct route: lr and E as amp_jacobi gives them, up to lambda's scale and phase.  Returns false
-// (nothing decided) where a pivot is not positive or tr(G) tr(G^{-1}) >= AMP_COND.  M <= SGS_MAX_RANK;
+// (nothing decided) where a pivot is not positive, tr(G) tr(G^{-1}) >= AMP_COND, or overlaps or amplitudes
+// are small (AMP_SMALL).  M <= SGS_MAX_RANK;
 // sm: 3 M (M + 1) complex.  Threads: AMP_THREADS, warp w taking rows w, w + 8, ...; odd row strides keep
 // both row and column walks free of bank conflicts.
 __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, double& E) {
@@ -268,9 +273,14 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     cplx* W = A + M * ld;           // U^{-1} (unit lower triangular)
     cplx* B = W + M * ld;           // h, then H', then T and the reflectors
     double trg = 0.0;
+    // |G_ij| >= AMP_SMALL somewhere off the diagonal, on the high words (an FP64 compare costs a warp 64 clocks)
+    const int least = __double2hiint(AMP_SMALL);
+    int overlap = M == 1;
     for (int i = warp; i < M; i += NW)
         for (int j = lane; j < M; j += 32) {
             const int e = 2 * (i * M + j);
+            if (i != j && (int)(max(__double2hiint(a.Gm[e]) & 0x7fffffff, __double2hiint(a.Gm[e + 1]) & 0x7fffffff)) >= least)
+                overlap = 1;
             A[i * ld + j] = cmk(a.Gm[e], a.Gm[e + 1]);
             B[i * ld + j] = cmk(a.hm[e], a.hm[e + 1]);
             W[i * ld + j] = cmk(i == j ? 1.0 : 0.0, 0.0);
@@ -282,6 +292,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
         s_d[0] = d;
         s_rcp[0] = 1.0 / d;
     }
+    if (!__syncthreads_or(overlap)) return false;
     trg = block_sum(trg, red);
     // step k: rows i > k lose l times row k, l = A_ik / d_k: the trailing lower triangle of G and
     // the columns j <= k of U^{-1}.  Column and row k are not written in step k; the thread that
@@ -488,7 +499,16 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     E = s_E;
     if (tid == 0 && !isfinite(s_E)) atomicOr(a.err, SGS_DEV_EIG);
     __syncthreads();
-    return true;
+    // every |lambda_j| at least AMP_SMALL times the largest (the larger part of each, on the high words)
+    int mine = 0x7fffffff, most = 0;
+    for (int j = lane; j < M; j += 32) {
+        const int x = max(__double2hiint(lr[j]) & 0x7fffffff, __double2hiint(lr[M + j]) & 0x7fffffff);
+        mine = min(mine, x);
+        most = max(most, x);
+    }
+    mine = __reduce_min_sync(0xffffffffu, mine);
+    most = __reduce_max_sync(0xffffffffu, most);
+    return !(most - mine > __double2hiint(1.0) - least);
 }
 
 // dynamic shared memory of amp_solve_kernel

@@ -42,3 +42,17 @@ def test_amplitudes(M, spread):
     else:
         assert w[0] < 1e-12 * w[-1]
         assert abs(E - Eo) <= 1e-9 * abs(Eo)
+
+
+def test_random_states_keep_exact_zeros():
+    """States whose overlaps are below rounding: the solve leaves the other amplitudes exactly zero (frozen states),
+    and a step runs."""
+    model = pkg.build_anderson(63, 2.0, -1.0, 0.5)
+    g, lam = pkg.seeded_states(model.n_modes, 6, 3)
+    s = pkg.Solver(model, g, lam, dtau=0.05)
+    s.step(3)
+    _, lam = s.get_state()
+    G, _ = s.pair_matrices()
+    s.close()
+    assert np.abs(G - np.eye(6)).max() < 1e-9
+    assert np.isfinite(lam).all() and np.sort(np.abs(lam))[-1] > 0.99
