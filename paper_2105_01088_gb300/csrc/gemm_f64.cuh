@@ -34,7 +34,8 @@ struct GemmBatch {
     double alpha; double diag;
     const double* alpha_b;               // optional per-batch multiplier of alpha
     const int* active_flag;              // optional: batch b computes only if active_flag[b] > active_cmp
-    int active_cmp;                      //   otherwise C = Cin (pass-through)
+    int active_cmp;                      //   otherwise C = Cin (pass-through), or with skip_inactive
+    int skip_inactive;                   //   C is left as it is
     int mode; int gj_k0; int gj_b;
     int gj_cols;                         // GJ: 1 = output columns gj_k0 .. gj_k0 + gj_b - 1 not written
     int gj_acc;                          // GJ: 1 = rows gj_k0 .. gj_k0 + gj_b - 1 add Cin like the others
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(GemmBatch g) {
     const int tid = threadIdx.x;
 
     const bool active = (g.active_flag == nullptr) || (g.active_flag[b] > g.active_cmp);
+    if (!active && g.skip_inactive) return;
     double alpha = g.alpha * (g.alpha_b ? g.alpha_b[b] : 1.0);
 
     double acc[4][4][2];
@@ -245,6 +247,7 @@ __global__ void __launch_bounds__(128) gemm_f64_small_kernel(GemmBatch g) {
     const bool skew = g.mode == GEMM_SKEW;
     if (skew && m0 + GSM <= n0) return;                 // above the diagonal: written as a mirror
     const bool active = (g.active_flag == nullptr) || (g.active_flag[b] > g.active_cmp);
+    if (!active && g.skip_inactive) return;
     const int rr = tid >> 3, cc = tid & 7, r = m0 + rr, c = n0 + cc;
     double acc = 0.0;
     if (active && g.k > 0) {
@@ -348,7 +351,7 @@ inline double gemm_fmas(const GemmBatch& g) {
 inline GemmBatch gemm_defaults() {
     GemmBatch g{};
     g.alpha = 1.0; g.beta = 0.0; g.diag = 0.0; g.sA2 = 0.0; g.sB2 = 0.0; g.Cin2 = nullptr; g.beta2 = 0.0;
-    g.mode = GEMM_FULL; g.active_flag = nullptr; g.alpha_b = nullptr; g.active_cmp = 0; g.b_antisym = 0;
+    g.mode = GEMM_FULL; g.active_flag = nullptr; g.alpha_b = nullptr; g.active_cmp = 0; g.skip_inactive = 0; g.b_antisym = 0;
     g.gj_cols = 1;
     g.gj_acc = 0;
     g.cin_trans = 0;

@@ -372,6 +372,7 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
 
     const GemmBatch& g = p.g;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (g.skip_inactive && !oz_active(g.active_flag, g.active_cmp, p.b0 + blockIdx.y)) return;
     if (tid == 0) skip = (*(volatile int*)p.err & SGS_DEV_TC_TIMEOUT) != 0;
     __syncthreads();
     if (skip) return;

@@ -113,7 +113,8 @@ struct Instance {
     double *fimp = nullptr, *fimp_state = nullptr, *lr = nullptr;
     double* s[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int* sq = nullptr;
-    double* scale = nullptr;
+    double* exp_part = nullptr;         // exponential: partial sums of the norms
+    double** p_R = nullptr;             // and where each state's result is
     double *Gm = nullptr, *hm = nullptr, *lam = nullptr, *lt = nullptr, *coef = nullptr;
     double* Ehist = nullptr;
     int Ecap = 0;
@@ -626,7 +627,8 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
     I.fimp = c->alloc<double>(Pm * ni * ni * 2); I.fimp_state = c->alloc<double>((size_t)M * ni * ni);
     I.lr = c->alloc<double>(Pcm * 2 * n * ni);
     for (int j = 0; j < 5; j++) I.s[j] = c->alloc<double>(M * nn);
-    I.sq = c->alloc<int>(M); I.scale = c->alloc<double>(M);
+    I.sq = c->alloc<int>(M); I.exp_part = c->alloc<double>((size_t)M * EXP_PARTS);
+    I.p_R = c->alloc<double*>(M);
     I.Gm = c->alloc<double>(2 * M * M); I.hm = c->alloc<double>(2 * M * M);
     I.lam = c->alloc<double>(2 * M); I.lt = c->alloc<double>(2 * M); I.coef = c->alloc<double>(6 * M * M);
     I.Ecap = 1;
@@ -1501,13 +1503,13 @@ cudaError_t eom_pass(sgs_ctx* c, Instance& I, cudaStream_t st) {
     return eom_close(c, I, st);
 }
 
-// exp(X_s) for the first `batch` states (App. A), X_s = 2^-s X in s1 as exp_prepare_kernel
-// leaves it: the degree-10 Taylor polynomial by Paterson-Stockmeyer in blocks of three,
-//   X2 = X_s^2 (s0), Y = X_s^3 (s2, antisymmetric), P = B3 (s3),
+// exp(X) of the first `batch` states (App. A), X = (ds/4)(Y - Y^T) with Y in s0, by scaling and squaring
+// (update.cuh): X (s1), X2 = X^2 (s0), Y = X^3 (s2, antisymmetric), the squarings s from ||X^3||_F and the
+// powers scaled, P = B3 (s3),
 //   P <- P Y + B_j for j = 2, 1, 0, B_j = c_{3j} I + c_{3j+1} X_s + c_{3j+2} X2, c_k = 1/k!
-// (the addends fused into the products' epilogue), then the squarings each state needs
-// (states with fewer pass their matrix through).  *cur_out <- the s buffer (3 or 4) that holds R.
-cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, cudaStream_t st, int* cur_out) {
+// (the addends fused into the products' epilogue), then the squarings each state needs, between s4 and s3
+// (a state with fewer is left where it is).  The results are at the device pointers p_R.
+cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, double ds, cudaStream_t st) {
     const int n = I.n;
     const size_t nn = (size_t)n * n;
     const double n3 = (double)n * n * n;
@@ -1517,14 +1519,18 @@ cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, cudaStream_t st, in
     for (int k = 1; k < 12; k++) cf[k] = cf[k - 1] / k;
     cf[11] = 0.0;                                         // degree 10
     cudaError_t e;
+    exp_commutator_kernel<<<dim3(EXP_PARTX, batch), 256, 0, st>>>(I.s[0], I.s[1], n, ds, I.exp_part);
+    counted();
     GemmBatch g = gb_basic(n, n, n, I.p_s[1], n, I.p_s[1], n, I.p_s[0], n, batch);
     if ((e = gemm(c, I, g, st, 2.0 * n3 * batch)) != cudaSuccess) return e;         // X2
     g = gb_basic(n, n, n, I.p_s[0], n, I.p_s[1], n, I.p_s[2], n, batch);
-    g.mode = GEMM_SKEW;                                                            // Y = X2 X_s
+    g.mode = GEMM_SKEW;                                                            // X3 = X2 X
     if ((e = gemm(c, I, g, st, n3 * batch)) != cudaSuccess) return e;
-    scaled_plus_identity_kernel<<<grid_chunks(batch * nn, 256, 4096), 256, 0, st>>>(I.s[1], cf[10], cf[9], n, I.s[3],
-                                                                                   batch * nn);
-    counted();
+    exp_norm_kernel<<<dim3(EXP_PART3, batch), 256, 0, st>>>(I.s[2], n, I.exp_part);
+    exp_scale_kernel<<<dim3(grid_chunks(nn, 1024, 256), batch), 256, 0, st>>>(I.s[1], I.s[0], I.s[2], cf[10], cf[9], n,
+                                                                            I.s[3], I.exp_part, I.s[4], I.s[3], I.p_R,
+                                                                            I.sq, I.err);
+    counted(); counted();
     int cur = 3;
     for (int j = 2; j >= 0; j--) {
         const int nxt = (cur == 3) ? 4 : 3;
@@ -1535,15 +1541,13 @@ cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, cudaStream_t st, in
         if ((e = gemm(c, I, g, st, 2.0 * n3 * batch)) != cudaSuccess) return e;
         cur = nxt;
     }
-    for (int j = 0; j < EXP_MAX_SQUARINGS; j++) {
+    for (int j = 0; j < EXP_MAX_SQUARINGS; j++) {         // from s4 (even) to s3 (odd) and back
         const int nxt = (cur == 3) ? 4 : 3;
         g = gb_basic(n, n, n, I.p_s[cur], n, I.p_s[cur], n, I.p_s[nxt], n, batch);
-        g.active_flag = I.sq; g.active_cmp = j;
-        g.Cin = (const double* const*)I.p_s[cur]; g.ldcin = n; g.beta = 0.0;
+        g.active_flag = I.sq; g.active_cmp = j; g.skip_inactive = 1;
         if ((e = gemm(c, I, g, st, -1.0)) != cudaSuccess) return e;
         cur = nxt;
     }
-    *cur_out = cur;
     return cudaSuccess;
 }
 
@@ -1672,17 +1676,14 @@ cudaError_t update_pass(sgs_ctx* c, Instance& I, cudaStream_t st) {
     // R Gamma 2, (R Gamma) R^T 1 (antisymmetric), one Newton-Schulz iteration (X X and X (X X),
     // half each) 2; squarings are added when profiles are read
     c->stage_flops[SGS_STAGE_UPDATE] += (2.0 + 9.0 + 2.0 + 1.0 + 2.0) * n3 * M;
-    // Y = Gamma dGamma -> s0 ; X_s -> s1
+    // Y = Gamma dGamma -> s0 ; R -> p_R
     GemmBatch g = gb_basic(n, n, n, I.p_gamma, n, I.p_dgamma, n, I.p_s[0], n, M);
     if ((e = gemm(c, I, g, st, 2.0 * n3 * M)) != cudaSuccess) return e;
-    exp_prepare_kernel<<<M, 1024, 0, st>>>(I.s[0], I.s[1], n, I.dtau, I.sq, I.scale, I.err);
-    counted();
-    int cur = 3;
-    if ((e = exp_products(c, I, M, st, &cur)) != cudaSuccess) return e;
+    if ((e = exp_products(c, I, M, I.dtau, st)) != cudaSuccess) return e;
     // T = R Gamma -> s0 ; Gamma' = T R^T -> s2
-    g = gb_basic(n, n, n, I.p_s[cur], n, I.p_gamma, n, I.p_s[0], n, M);
+    g = gb_basic(n, n, n, I.p_R, n, I.p_gamma, n, I.p_s[0], n, M);
     if ((e = gemm(c, I, g, st, 2.0 * n3 * M)) != cudaSuccess) return e;
-    g = gb_basic(n, n, n, I.p_s[0], n, I.p_s[cur], n, I.p_s[2], n, M);
+    g = gb_basic(n, n, n, I.p_s[0], n, I.p_R, n, I.p_s[2], n, M);
     g.transB = 1; g.mode = GEMM_SKEW;
     if ((e = gemm(c, I, g, st, n3 * M)) != cudaSuccess) return e;
     // R is orthogonal to rounding, so R Gamma R^T leaves purity only at rounding level, which one
@@ -2098,22 +2099,16 @@ sgs_status sgs_add_state(sgs_ctx* c, int slot, const double* K, int src) {
     if (s == SGS_OK) {
         e = cudaMemcpyAsync(J.gamma, I.gamma, M * nn * sizeof(double), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(J.lam, I.lam, 2 * M * sizeof(double), cudaMemcpyDeviceToDevice, st);
-        // X = K: exp_prepare_kernel forms (ds/4)(Y - Y^T), which is K for Y = K and ds = 2
+        // X = K: exp_products takes (ds/4)(Y - Y^T), which is K for Y = K and ds = 2
         if (e == cudaSuccess) e = cudaMemcpyAsync(J.s[0], K, nn * sizeof(double), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) {
-            exp_prepare_kernel<<<1, 1024, 0, st>>>(J.s[0], J.s[1], n, 2.0, J.sq, J.scale, J.err);
-            counted();
-            e = cudaGetLastError();
-        }
-        int cur = 3;
-        if (e == cudaSuccess) e = exp_products(c, J, 1, st, &cur);
+        if (e == cudaSuccess) e = exp_products(c, J, 1, 2.0, st);
         // Q Gamma_src -> s0 ; (Q Gamma_src) Q^T -> Gamma_M
         if (e == cudaSuccess) {
-            GemmBatch g = gb_basic(n, n, n, J.p_s[cur], n, J.p_gamma + src, n, J.p_s[0], n, 1);
+            GemmBatch g = gb_basic(n, n, n, J.p_R, n, J.p_gamma + src, n, J.p_s[0], n, 1);
             e = gemm(c, J, g, st, -1.0);
         }
         if (e == cudaSuccess) {
-            GemmBatch g = gb_basic(n, n, n, J.p_s[0], n, J.p_s[cur], n, J.p_gamma + M, n, 1);
+            GemmBatch g = gb_basic(n, n, n, J.p_s[0], n, J.p_R, n, J.p_gamma + M, n, 1);
             g.transB = 1; g.mode = GEMM_SKEW;
             e = gemm(c, J, g, st, -1.0);
         }
