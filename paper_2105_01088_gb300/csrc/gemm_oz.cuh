@@ -258,6 +258,14 @@ __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
     }
 }
 
+// four doubles' bits at a 32-byte boundary, as one access
+__device__ __forceinline__ void oz_ld4(unsigned long long (&x)[4], const double* p) {
+    asm volatile("ld.global.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3]) : "l"(p));
+}
+__device__ __forceinline__ void oz_st4(unsigned long long* p, const unsigned long long (&x)[4]) {
+    asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};" :: "l"(p), "l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]) : "memory");
+}
+
 struct OzGemm {
     CUtensorMap ta, tb;       // slices: 3-D [chunk * 8][rows_pad][k] bf16, box 64 x rows x 1
     GemmBatch g;              // sizes, output and epilogue fields (batch index = b0 + local)
@@ -279,7 +287,7 @@ __device__ __forceinline__ void oz_tma_load(uint32_t dst, const CUtensorMap* map
 // 0 <= L < 2^28: hi = sum_{G<4} v_G 2^(7 (3 - G)) and lo = sum_{G>=4} v_G 2^(7 (7 - G))
 // (|hi|, |lo| < 2^46, each a chain of 32 x 32 -> 64-bit multiply-adds), V = hi 2^28 + lo,
 // H = hi + floor(lo / 2^28), L = lo mod 2^28.
-__device__ __forceinline__ void oz_combine(const uint32_t (&u)[OZ_G][8], int j, long long& H, unsigned& L) {
+__device__ __forceinline__ void oz_combine(const uint32_t (&u)[OZ_G][4], int j, long long& H, unsigned& L) {
     int v[OZ_G];
 #pragma unroll
     for (int G = 0; G < OZ_G; G++) v[G] = __float2int_rn(__uint_as_float(u[G][j]));
@@ -362,12 +370,12 @@ __device__ __forceinline__ unsigned long long oz_to_double_bits_normal(long long
 
 template <int BN, int EPIW, int RING, bool BDBL>
 __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(const __grid_constant__ OzGemm p) {
-    constexpr int SLAB_B = BN * 128, TS = BN + 1, NB = BDBL ? 2 : 1;
+    constexpr int SLAB_B = BN * 128, NB = BDBL ? 2 : 1;
     constexpr uint32_t TCOLS = 8u * BN;          // TMEM columns: eight groups of BN
     extern __shared__ uint8_t oz_smem_raw[];
     __shared__ uint64_t bfull[2], bempty[2], afull[RING], aempty[RING], tfull, done;
     __shared__ uint32_t tmem_base;
-    __shared__ int skip, abort_flag, s_ok, s_fcmin, s_fcmax;
+    __shared__ int skip, abort_flag;
     __shared__ int col_e[BN];
 
     const GemmBatch& g = p.g;
@@ -543,71 +551,61 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
             mbar_wait(smem_u32(&done), 0u, p.err);
         }
     } else {
-        // epilogue: warps 0 .. EPIW - 1.  Warp w drains TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 (output
-        // rows) for the columns of part w / 4; the store pass gives thread tid the elements tid + 32 EPIW q.
-        constexpr int NE = 32 * EPIW, PER = OZ_BM * BN / NE;
+        // epilogue: warps 0 .. EPIW - 1.  Warp w has TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, an output row per
+        // thread, and the columns of part w / 4, four at a time: a sector of the row.  Results go from the
+        // registers to memory: a row's four columns are one 32-byte access per lane, the mirrored block of an
+        // antisymmetric result and a transposed Cin run along the lanes.  Every element is read and written by
+        // the one thread that computes it (Cin may be C itself).
+        constexpr int PCOLS = BN / (EPIW / 4), PASSES = PCOLS / 4;
+        static_assert(PCOLS % 4 == 0, "four-column passes");
         const double* Cinb = g.Cin ? g.Cin[b] + g.offCin : nullptr;
         const double* Cin2b = g.Cin2 ? g.Cin2[b] + g.offCin : nullptr;
         double* Cb = g.C[b] + g.offC;
         const bool skew = g.mode == GEMM_SKEW, gj = g.mode == GEMM_GJ;
+        const int lq = warp & 3, part = warp >> 2;          // lane quarter, column part
+        const int row = m0 + lq * 32 + lane, cp0 = n0 + part * PCOLS;
+        const bool use_cin = Cinb && (!active || g.beta != 0.0);
+        const bool ct = g.cin_trans != 0;
+        // in-place update: C = Cin + A B, or the sign of a transposed Cin flipped by an integer XOR; a
+        // Gauss-Jordan update's pivot rows take the product alone
+        const bool cin_neg = active && ct && g.beta == -1.0;
+        const bool plain = active && p.alpha_pow2 && !Cin2b && (!use_cin || g.beta == 1.0 || cin_neg);
+        const bool drop_cin = active && gj && !g.gj_acc && row >= g.gj_k0 && row < g.gj_k0 + g.gj_b;
+        const unsigned long long cin_sign = cin_neg ? 0x8000000000000000ull : 0ull;
+        // 32-byte (or 16-byte) accesses along the rows where every row starts on one
+        auto align_of = [&](const double* x, int ld) {
+            const uintptr_t a = reinterpret_cast<uintptr_t>(x + cp0) | ((uintptr_t)ld * 8);
+            return (a & 31) == 0 ? 32 : (a & 15) == 0 ? 16 : 8;
+        };
+        const int al_in = use_cin && !ct ? align_of(Cinb, g.ldcin) : 8, al_out = align_of(Cb, g.ldc);
+        // Cin's four elements of columns c .. c + 3 of this row
+        auto load_cin = [&](unsigned long long (&x)[4], int c) {
+            if (!use_cin || drop_cin || row >= g.m || (skew && row < c)) {
+                x[0] = x[1] = x[2] = x[3] = 0ull;
+                return;
+            }
+            const double* s = Cinb + (ct ? (long long)c * g.ldcin + row : (long long)row * g.ldcin + c);
+            if (al_in == 32 && c + 3 < g.n) {
+                oz_ld4(x, s);
+            } else if (al_in == 16 && c + 3 < g.n) {
+                const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(s), d = *reinterpret_cast<const ulonglong2*>(s + 2);
+                x[0] = a.x; x[1] = a.y; x[2] = d.x; x[3] = d.y;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    x[j] = c + j < g.n ? reinterpret_cast<const unsigned long long*>(s)[ct ? (long long)j * g.ldcin : j] : 0ull;
+            }
+        };
+        unsigned long long ci[4], cn[4];
+        load_cin(ci, cp0);                                   // in flight while the MMAs run
         bool ok = true;
         if (nslab > 0) {
-            if (tid == 0) {
-                // the range of the tile's nonzero column exponent fields (for the normal-range test)
-                int lo = 4096, hi = 0;
-                for (int c = 0; c < BN; c++)
-                    if (col_e[c] > 0) { lo = min(lo, col_e[c]); hi = max(hi, col_e[c]); }
-                s_fcmin = lo;
-                s_fcmax = hi;
-                s_ok = mbar_wait_or_abort(smem_u32(&tfull), 0u, p.err) ? 1 : 0;
-            }
-            asm volatile("bar.sync 1, %0;" :: "n"(NE) : "memory");
-            ok = s_ok != 0;
+            if (lane == 0) ok = mbar_wait_or_abort(smem_u32(&tfull), 0u, p.err);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         }
         if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;");
-            // every MMA has completed, so every load has been consumed: the stage buffers
-            // become the (padded) FP64 output tile
-            double* tile = reinterpret_cast<double*>(oz_smem_raw + (sbase - raw));
-            // Cin's tile is copied into the free stage memory after the output tile with cp.async,
-            // overlapping the drain and combination (a barrier does not wait for these asynchronous
-            // copies, unlike ordinary loads); rows must start on 16 bytes, else the store pass reads
-            // Cin itself.  Cin may be C itself: every Cin element is read before this CTA stores any.
-            double* cin_s = tile + OZ_BM * TS;
-            const bool use_cin = Cinb && (!active || g.beta != 0.0);
-            const bool ct = g.cin_trans != 0;
-            const bool cin_async = use_cin && ((reinterpret_cast<uintptr_t>(Cinb) & 15) == 0) &&
-                                   ((g.ldcin & 1) == 0);
-            // transposed Cin: element (rr, cc) at cin_s[cc OZ_BM + (rr ^ 2 (cc & 7))], copied 16 bytes
-            // (two rows) at a time along the memory rows; the swizzle spreads the reads of consecutive
-            // cc over eight bank pairs
-            // one load at an integer-selected index (a select between two loaded doubles would issue
-            // on the FP64 pipe)
-            auto cin_smem = [&](int rr, int cc) {
-                return cin_s[ct ? cc * OZ_BM + (rr ^ ((cc & 7) << 1)) : rr * BN + cc];
-            };
-            if (cin_async && ct) {
-                for (int x = tid; x < BN * (OZ_BM / 2); x += NE) {
-                    const int cc = x / (OZ_BM / 2), rp = 2 * (x % (OZ_BM / 2)), r = m0 + rp, c = n0 + cc;
-                    const uint32_t bytes = c < g.n ? (r + 1 < g.m ? 16u : (r < g.m ? 8u : 0u)) : 0u;
-                    const double* src = bytes ? Cinb + (long long)c * g.ldcin + r : Cinb;
-                    cp_async16(smem_u32(cin_s + cc * OZ_BM + (rp ^ ((cc & 7) << 1))), src, bytes);
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-            } else if (cin_async) {
-                for (int x = tid; x < OZ_BM * (BN / 2); x += NE) {
-                    const int rr = x / (BN / 2), c = n0 + 2 * (x % (BN / 2)), r = m0 + rr;
-                    const uint32_t bytes = r < g.m ? (c + 1 < g.n ? 16u : (c < g.n ? 8u : 0u)) : 0u;
-                    const double* src = bytes ? Cinb + (long long)r * g.ldcin + c : Cinb;
-                    cp_async16(smem_u32(cin_s + rr * BN + (c - n0)), src, bytes);
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-            }
             const double alpha = g.alpha * (g.alpha_b ? g.alpha_b[b] : 1.0);
-            constexpr int PCOLS = BN / (EPIW / 4);                 // columns per warp
-            static_assert(PCOLS % 8 == 0, "eight-column TMEM loads");
-            const int lq = warp & 3, part = warp >> 2;          // lane quarter, column part
-            const int rr0 = lq * 32 + lane, row = m0 + rr0;
             const int er = (active && row < g.m) ? p.ea[(size_t)bl * p.m_pad + row] : 0;
             const int ae = p.alpha_pow2 ? p.alpha_e : 0;
             const bool an = p.alpha_pow2 && p.alpha_neg;
@@ -615,110 +613,107 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
             // the leading bit P of |V| in 0 .. 74, the biased exponent P + e + 1023 stays in 1 .. 2046
             // (rows or columns with a zero exponent field give zeros either way); then the
             // combination takes the form without the range-end selects (the same bits)
-            const bool row_normal = er == 0 || s_fcmax == 0 ||
-                                    (er + s_fcmin - 2107 + ae + 1023 >= 1 && er + s_fcmax - 2107 + ae + 1023 + 74 <= 2046);
+            const int fe = lane < PCOLS ? col_e[part * PCOLS + lane] : 0;
+            const int fcmin = __reduce_min_sync(0xffffffffu, fe > 0 ? fe : 4096);
+            const int fcmax = __reduce_max_sync(0xffffffffu, fe);
+            const bool row_normal = er == 0 || fcmax == 0 ||
+                                    (er + fcmin - 2107 + ae + 1023 >= 1 && er + fcmax - 2107 + ae + 1023 + 74 <= 2046);
             const bool fast = __all_sync(0xffffffffu, row_normal);
-            if (nslab > 0) {
-                // eight columns per pass: one 8-column TMEM load per group, then eight independent
-                // combinations
 #pragma unroll 1
-                for (int cb = part * (PCOLS / 8); cb < (part + 1) * (PCOLS / 8); cb++) {
-                    uint32_t u[OZ_G][8];
+            for (int pass = 0; pass < PASSES; pass++) {
+                const int cl = part * PCOLS + 4 * pass, c0 = n0 + cl;
+                if (c0 >= g.n || (skew && m0 + lq * 32 + 31 < c0)) break;     // warp-uniform
+                unsigned long long t[4] = {0ull, 0ull, 0ull, 0ull};
+                if (nslab > 0) {
+                    uint32_t u[OZ_G][4];
 #pragma unroll
                     for (int G = 0; G < OZ_G; G++) {
-                        const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(G * BN + cb * 8);
-                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                                     : "=r"(u[G][0]), "=r"(u[G][1]), "=r"(u[G][2]), "=r"(u[G][3]),
-                                       "=r"(u[G][4]), "=r"(u[G][5]), "=r"(u[G][6]), "=r"(u[G][7])
+                        const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(G * BN + cl);
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(u[G][0]), "=r"(u[G][1]), "=r"(u[G][2]), "=r"(u[G][3])
                                      : "r"(ta));
                     }
+                    if (pass + 1 < PASSES) load_cin(cn, c0 + 4);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int j = 0; j < 8; j++) {
+                    for (int j = 0; j < 4; j++) {
                         // computed for every column and selected (no branch between the columns)
-                        const int c = cb * 8 + j, fc = col_e[c];
+                        const int fc = col_e[cl + j];
                         long long H;
                         unsigned L;
                         oz_combine(u, j, H, L);
                         const unsigned long long v = fast ? oz_to_double_bits_normal(H, L, er + fc - 2107 + ae, an)
                                                           : oz_to_double_bits(H, L, er + fc - 2107 + ae, an);
-                        reinterpret_cast<unsigned long long*>(tile)[rr0 * TS + c] = (er > 0 && fc > 0) ? v : 0ull;
+                        t[j] = (er > 0 && fc > 0) ? v : 0ull;
+                    }
+                } else if (pass + 1 < PASSES) {
+                    load_cin(cn, c0 + 4);
+                }
+                // The common forms issue no FP64 instruction beyond the one addition an update needs (FP64
+                // issues at a small fraction of the integer rate on this part)
+                if (plain) {
+                    if (use_cin && !drop_cin) {
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            t[j] = (unsigned long long)__double_as_longlong(
+                                __longlong_as_double((long long)(ci[j] ^ cin_sign)) + __longlong_as_double((long long)t[j]));
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        double v = 0.0;
+                        if (use_cin && !drop_cin) {
+                            v = __longlong_as_double((long long)ci[j]);
+                            if (active && g.beta != 1.0) v *= g.beta;
+                        }
+                        if (active) {
+                            if (Cin2b && row < g.m && c0 + j < g.n)
+                                v = fma(g.beta2, Cin2b[(long long)row * g.ldcin + c0 + j], v);
+                            double x = __longlong_as_double((long long)t[j]);
+                            if (!p.alpha_pow2) x *= alpha;
+                            v += x;
+                        }
+                        t[j] = (unsigned long long)__double_as_longlong(v);
                     }
                 }
-            }
-            if (cin_async) asm volatile("cp.async.wait_all;" ::: "memory");
-            asm volatile("bar.sync 1, %0;" :: "n"(NE) : "memory");
-            const bool scale_cin = active && g.beta != 1.0;          // beta = 1 (the in-place updates): no product
-            // Cin(r, c) = -Cin^T: the sign bit flipped by an integer XOR, then the one addition
-            const unsigned long long cin_sign = (active && ct && g.beta == -1.0) ? 0x8000000000000000ull : 0ull;
-            const bool cin_neg = cin_sign != 0ull;
-            const bool keep_tile = skew || (active && g.diag != 0.0);
-            // an element's final value: kept in the tile for the mirrored block and the diagonal,
-            // stored unless its column is one of the Gauss-Jordan panel's
-            auto emit = [&](int rr, int cc, int r, int c, double v) {
-                if (skew && r == c) v = 0.0;
-                if (keep_tile) tile[rr * TS + cc] = v;
-                if (!gj || !g.gj_cols || c < g.gj_k0 || c >= g.gj_k0 + g.gj_b) Cb[(long long)r * g.ldc + c] = v;
-            };
-            // The common forms get loops of their own, so that no FP64 instruction is issued where
-            // none is needed (FP64 issues at a small fraction of the integer rate on this part):
-            // the plain product, and the in-place update C = Cin + A B.
-            if (active && p.alpha_pow2 && !Cin2b && !use_cin) {
-#pragma unroll 4
-                for (int q = 0; q < PER; q++) {
-                    const int e = tid + NE * q, rr = e / BN, cc = e % BN, r = m0 + rr, c = n0 + cc;
-                    if (r >= g.m || c >= g.n || (skew && r < c)) continue;
-                    emit(rr, cc, r, c, tile[rr * TS + cc]);
+                if (active && g.diag != 0.0 && !skew && __any_sync(0xffffffffu, row >= c0 && row < c0 + 4)) {
+#pragma unroll
+                    for (int j = 0; j < 4; j++)
+                        if (row == c0 + j)
+                            t[j] = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)t[j]) + g.diag);
                 }
-            } else if (active && p.alpha_pow2 && !Cin2b && use_cin && (!scale_cin || cin_neg) && cin_async) {
-#pragma unroll 4
-                for (int q = 0; q < PER; q++) {
-                    const int e = tid + NE * q, rr = e / BN, cc = e % BN, r = m0 + rr, c = n0 + cc;
-                    if (r >= g.m || c >= g.n || (skew && r < c)) continue;
-                    const double t = tile[rr * TS + cc];
-                    const bool gj_row = gj && !g.gj_acc && r >= g.gj_k0 && r < g.gj_k0 + g.gj_b;
-                    const double ci = __longlong_as_double(__double_as_longlong(cin_smem(rr, cc)) ^ (long long)cin_sign);
-                    emit(rr, cc, r, c, gj_row ? t : ci + t);
-                }
-            } else {
-#pragma unroll 4
-                for (int q = 0; q < PER; q++) {
-                    const int e = tid + NE * q, rr = e / BN, cc = e % BN, r = m0 + rr, c = n0 + cc;
-                    if (r >= g.m || c >= g.n || (skew && r < c)) continue;
-                    double v = 0.0;
-                    if (use_cin && !(active && gj && !g.gj_acc && r >= g.gj_k0 && r < g.gj_k0 + g.gj_b)) {
-                        v = cin_async ? cin_smem(rr, cc)
-                                      : Cinb[ct ? (long long)c * g.ldcin + r : (long long)r * g.ldcin + c];
-                        if (scale_cin) v *= g.beta;
+                if (row < g.m) {
+                    unsigned long long* d = reinterpret_cast<unsigned long long*>(Cb + (long long)row * g.ldc + c0);
+                    const bool panel = gj && g.gj_cols;       // columns gj_k0 .. gj_k0 + gj_b - 1 are not written
+                    if (!panel && c0 + 3 < g.n && (!skew || row > c0 + 3)) {
+                        if (al_out == 32) oz_st4(d, t);
+                        else if (al_out == 16) {
+                            reinterpret_cast<ulonglong2*>(d)[0] = make_ulonglong2(t[0], t[1]);
+                            reinterpret_cast<ulonglong2*>(d)[1] = make_ulonglong2(t[2], t[3]);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; j++) d[j] = t[j];
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            const int c = c0 + j;
+                            if (c >= g.n || (skew && row < c) || (panel && c >= g.gj_k0 && c < g.gj_k0 + g.gj_b)) continue;
+                            d[j] = (skew && row == c) ? 0ull : t[j];
+                        }
                     }
-                    if (active) {
-                        if (Cin2b) v = fma(g.beta2, Cin2b[(long long)r * g.ldcin + c], v);
-                        double t = tile[rr * TS + cc];
-                        if (!p.alpha_pow2) t *= alpha;
-                        v += t;
+                    if (skew) {                               // mirrored block: C[c][r] = -C[r][c] below the diagonal
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            if (c0 + j < g.n && row > c0 + j)
+                                reinterpret_cast<unsigned long long*>(Cb)[(long long)(c0 + j) * g.ldc + row] =
+                                    t[j] ^ 0x8000000000000000ull;
                     }
-                    emit(rr, cc, r, c, v);
                 }
+#pragma unroll
+                for (int j = 0; j < 4; j++) ci[j] = cn[j];
             }
-            if (active && g.diag != 0.0 && !skew) {
-                // the diagonal term, added to the stored values of the tile's diagonal elements
-                asm volatile("bar.sync 1, %0;" :: "n"(NE) : "memory");
-                const int c = n0 + tid, rr = c - m0;
-                if (tid < BN && rr >= 0 && rr < OZ_BM && c < g.m && c < g.n &&
-                    (!gj || !g.gj_cols || c < g.gj_k0 || c >= g.gj_k0 + g.gj_b))
-                    Cb[(long long)c * g.ldc + c] = tile[rr * TS + tid] + g.diag;
-            }
-            if (skew) {
-                // mirrored block: C[c][r] = -C[r][c] below the diagonal, rows of the mirror coalesced
-                asm volatile("bar.sync 1, %0;" :: "n"(NE) : "memory");
-                for (int e = tid; e < OZ_BM * BN; e += NE) {
-                    const int cc = e / OZ_BM, rr = e % OZ_BM;
-                    const int r = m0 + rr, c = n0 + cc;
-                    if (r >= g.m || c >= g.n || r <= c) continue;
-                    Cb[(long long)c * g.ldc + r] = -tile[rr * TS + cc];
-                }
-            }
-        } else if (tid == 0) {
+        } else if (lane == 0) {
             abort_flag = 1;
         }
     }
