@@ -40,21 +40,28 @@
 // Kernels per batch chunk: exponents and slices of op(A) and op(B), one pass
 // over each (a warp per row where the operand's K rows are contiguous and long,
 // else a block of whole rows at a time through shared memory), then the product
-// kernel.  It takes a 128 x 32 output tile per CTA of 10 warps (256 TMEM
-// columns, 97 KB of shared memory), so two CTAs share an SM and one's epilogue
-// overlaps the other's loads and MMAs.  In the kernel:
+// kernel.  It takes 128 x 32 output tiles with CTAs of 10 warps (256 TMEM
+// columns, 97 KB of shared memory), two to an SM, each running over every
+// (2 x SMs)-th tile, so that CTAs side by side work on tiles side by side and share
+// their slices in L2 (consecutive tiles per CTA read them from DRAM: 1.5 to 2.3 ms
+// where this order takes 0.86).  In the kernel:
 //   * one producer lane loads, per 64-element K slab, the eight B slices as one
-//     TMA box (TMA issue costs about the same per box whatever its size, so
-//     boxes are made large) and the A slices in pairs (one 32 KB box per pair of
+//     TMA box and the A slices in pairs (one 32 KB box per pair of
 //     adjacent planes) through a ring, 128-byte swizzle, zero fill beyond K;
-//     the B buffer is reloaded once the previous slab's MMAs have released it;
+//     the B buffer is reloaded once the previous slab's MMAs have released it, and
+//     the next tile's first slabs load during this tile's epilogue;
 //   * one MMA lane issues, per A slice and K16 step, one MMA of N up to 256
 //     covering all the products of that slice (the B slices and the groups they
 //     feed are adjacent) into the eight accumulators;
-//   * the epilogue warps wait for the MMAs, issue the loads of the tile's Cin
-//     terms (for in-place updates every Cin element is read before the CTA
-//     stores any), drain TMEM and combine, and write the output through a
-//     shared-memory tile (coalesced rows).
+//   * the epilogue warps read the tile's Cin terms while the MMAs run, drain TMEM,
+//     combine, and write the output from their registers; the next tile's MMAs start
+//     when TMEM is drained.
+// One tile per CTA (set-up, first loads and last stores all exposed: 2 + 0.8 us of a
+// K = 64 tile's 12.6) took 13.4 us for the SM's two tiles at K = 64, 11.7 at K = 16 and
+// 36.2 at K = 512; now 11.8, 9.0 and 34.0.  What bounds it: at K = 512 the MMAs, 26 of
+// the 34 us (below N = 180 an MMA takes about 90 clocks whatever its N: 790 clocks per
+// K16 step and tile against 576 at full rate; with the loads left out it takes 29); at
+// small K the integer work of the combination, about 150 instructions per output.
 // Every mbarrier wait is bounded; on a timeout the launch records
 // SGS_DEV_TC_TIMEOUT in the error word, waits (bounded) for its loads and MMAs
 // in flight, frees TMEM and returns.
@@ -63,6 +70,7 @@
 #include "gemm_tma.cuh"
 #include "oz_digits.cuh"
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 
@@ -75,20 +83,18 @@ namespace sgs {
 #define OZ_UNIT 2             // A slices per TMA box (one ring slot)
 #define OZ_SLAB_A (OZ_BM * 128)
 
-// Kernel shapes: BN output columns per tile (TMEM: 8 BN columns), EPIW epilogue warps,
-// RING A-ring depth (units), BDBL double-buffered B slabs.  The form launched (32, 8, 2,
-// single) fits two CTAs per SM.  A 128 x 64 tile (64, 16, 3, double) takes all of an SM's
-// TMEM and shared memory; with its epilogue serialised after the main loop it measured
-// about half the throughput at K = 512, so it is not launched.
-template <int BN, int EPIW, int RING, bool BDBL> struct OzCfg {
+// Kernel shapes: BN output columns per tile (TMEM: 8 BN columns), EPIW epilogue warps, RING A-ring depth
+// (units).  Both forms fit two CTAs per SM.  A 128 x 64 tile takes all of an SM's TMEM and shared memory;
+// with its epilogue serialised after the main loop it measured about half the throughput at K = 512.
+template <int BN, int EPIW, int RING> struct OzCfg {
     static constexpr int SLAB_B = BN * 128;
-    static constexpr int SMEM = (BDBL ? 2 : 1) * OZ_S * SLAB_B + RING * OZ_UNIT * OZ_SLAB_A + 1024;
+    static constexpr int SMEM = OZ_S * SLAB_B + RING * OZ_UNIT * OZ_SLAB_A + 1024;
     static constexpr int THREADS = 32 * (EPIW + 2);
 };
-#define OZ_NARROW 32, 8, 2, false
+#define OZ_NARROW 32, 8, 2
 // 128 x 16 tiles for products of at most 16 output columns (the Gauss-Jordan leaf updates):
 // half the epilogue of a 128 x 32 tile whose other half would be discarded
-#define OZ_NARROW16 16, 8, 2, false
+#define OZ_NARROW16 16, 8, 2
 
 // device scratch of one owner (an instance, or a temporary context): slices and
 // exponent fields of one batch chunk
@@ -270,6 +276,7 @@ struct OzGemm {
     CUtensorMap ta, tb;       // slices: 3-D [chunk * 8][rows_pad][k] bf16, box 64 x rows x 1
     GemmBatch g;              // sizes, output and epilogue fields (batch index = b0 + local)
     int b0;
+    int tiles, total;         // tiles per batch entry and of the launch
     int m_pad, n_pad;
     const int* ea; const int* eb;
     int* err;
@@ -368,49 +375,50 @@ __device__ __forceinline__ unsigned long long oz_to_double_bits_normal(long long
     return (Hm | Lm) ? bits : 0ull;
 }
 
-template <int BN, int EPIW, int RING, bool BDBL>
-__global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(const __grid_constant__ OzGemm p) {
-    constexpr int SLAB_B = BN * 128, NB = BDBL ? 2 : 1;
+// Output tile x of a batch entry: tile row tm (128 rows) and tile column tn (BN columns); an antisymmetric
+// result has the tiles that hold an element on or below the diagonal
+template <int BN>
+__device__ __forceinline__ void oz_tile(const GemmBatch& g, int x, int& m0, int& n0) {
+    const int tnn = (g.n + BN - 1) / BN;
+    int tm = 0, tn = x;
+    if (g.mode == GEMM_SKEW) {
+        for (int cnt; tn >= (cnt = min((tm + 1) * (OZ_BM / BN), tnn)); tm++) tn -= cnt;
+    } else {
+        tm = x / tnn;
+        tn = x - tm * tnn;
+    }
+    m0 = tm * OZ_BM;
+    n0 = tn * BN;
+}
+
+template <int BN, int EPIW, int RING>
+__global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __grid_constant__ OzGemm p) {
+    constexpr int SLAB_B = BN * 128, NU = OZ_S / OZ_UNIT;
     constexpr uint32_t TCOLS = 8u * BN;          // TMEM columns: eight groups of BN
     extern __shared__ uint8_t oz_smem_raw[];
-    __shared__ uint64_t bfull[2], bempty[2], afull[RING], aempty[RING], tfull, done;
+    __shared__ uint64_t bfull, bempty, afull[RING], aempty[RING], tfull, tempty, done;
     __shared__ uint32_t tmem_base;
     __shared__ int skip, abort_flag;
-    __shared__ int col_e[BN];
 
     const GemmBatch& g = p.g;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (g.skip_inactive && !oz_active(g.active_flag, g.active_cmp, p.b0 + blockIdx.y)) return;
+    const int t0 = blockIdx.x, t1 = p.total, dt = gridDim.x;
+    // tile t's batch entry, whether it computes, and (inactive entries left alone) whether it does anything
+    auto entry = [&](int t) { return p.b0 + t / p.tiles; };
+    auto is_active = [&](int t) { return oz_active(g.active_flag, g.active_cmp, entry(t)); };
+    if (g.skip_inactive) {
+        bool any = false;
+        for (int t = t0; t < t1; t += dt) any = any || is_active(t);
+        if (!any) return;
+    }
     if (tid == 0) skip = (*(volatile int*)p.err & SGS_DEV_TC_TIMEOUT) != 0;
     __syncthreads();
     if (skip) return;
-    const int bl = blockIdx.y, b = p.b0 + bl;
-    const int tnn = (g.n + BN - 1) / BN;
-    int tm, tn;
-    if (g.mode == GEMM_SKEW) {      // tiles holding an element on or below the diagonal
-        int t = blockIdx.x;
-        tm = 0;
-        while (true) {
-            const int cnt = min((tm + 1) * (OZ_BM / BN), tnn);
-            if (t < cnt) break;
-            t -= cnt;
-            tm++;
-        }
-        tn = t;
-    } else {
-        tm = blockIdx.x / tnn;
-        tn = blockIdx.x % tnn;
-    }
-    const int m0 = tm * OZ_BM, n0 = tn * BN;
-    const bool active = oz_active(g.active_flag, g.active_cmp, b);
-    const int nslab = active ? (g.k + OZ_KS - 1) / OZ_KS : 0;      // k <= OZ_KC (the host splits K)
+    const int nslab = (g.k + OZ_KS - 1) / OZ_KS;      // k <= OZ_KC (the host splits K)
 
     const uint32_t raw = smem_u32(oz_smem_raw);
     const uint32_t sbase = (raw + 1023u) & ~1023u;
-    auto sB = [&](int bb, int j) { return sbase + (uint32_t)(bb * OZ_S + j) * SLAB_B; };
-    auto sA = [&](int slot) { return sbase + (uint32_t)NB * OZ_S * SLAB_B + (uint32_t)slot * (OZ_UNIT * OZ_SLAB_A); };
-    auto bslot = [&](int sb) { return BDBL ? (sb & 1) : 0; };
-    auto bphase = [&](int sb) { return (uint32_t)((BDBL ? (sb >> 1) : sb) & 1); };
+    auto sA = [&](int slot) { return sbase + (uint32_t)OZ_S * SLAB_B + (uint32_t)slot * (OZ_UNIT * OZ_SLAB_A); };
 
     if (warp == EPIW + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -418,136 +426,131 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int s = 0; s < 2; s++) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&bfull[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&bempty[s])));
-        }
+        auto init = [](uint64_t& bar, int count) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&bar)), "r"(count));
+        };
+        init(bfull, 1);
+        init(bempty, 1);
         for (int s = 0; s < RING; s++) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&afull[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&aempty[s])));
+            init(afull[s], 1);
+            init(aempty[s], 1);
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&tfull)));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&done)));
+        init(tfull, 1);
+        init(tempty, EPIW);
+        init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
         abort_flag = 0;
     }
-    if (tid < BN) col_e[tid] = (active && n0 + tid < g.n) ? p.eb[(size_t)bl * p.n_pad + n0 + tid] : 0;
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
 
+    // A CTA takes its tiles one after the other: the producer runs ahead into the next tile's slabs as the
+    // MMAs release the buffers, and the MMAs of the next tile start when the epilogue warps have drained
+    // TMEM, so the loads (and most of the MMAs of the SM's other CTA) run during an epilogue.
     if (warp == EPIW) {
         if (lane == 0) {            // producer
-            // one TMA box per B slab (the eight slices, 8 BN rows) and per A unit (two slices, 32 KB).
-            // Double-buffered B: B(0); then per slab s: A units 0 and 1, B(s + 1) (once slab s - 1 has
-            // released its buffer), A units 2 and 3, so the next slab's B loads during slab s's MMAs.
-            // Single buffer: B(s) once slab s - 1 has released it.
-            constexpr int NU = OZ_S / OZ_UNIT;
+            // one TMA box per B slab (the eight slices, 8 BN rows; one buffer, reloaded once the previous
+            // slab's MMAs have released it) and per A unit (two slices, 32 KB)
             int nb = 0, q = 0;      // B slabs and A units issued
             bool ok = true;
-            auto issue_b = [&](int sb) {
-                const int bb = bslot(sb);
-                mbar_expect_tx(smem_u32(&bfull[bb]), (uint32_t)(OZ_S * SLAB_B));
-                oz_tma_load(sB(bb, 0), &p.tb, sb * OZ_KS, n0, bl * OZ_S, smem_u32(&bfull[bb]));
-                nb = sb + 1;
-            };
-            if (nslab > 0) issue_b(0);
-            for (int s = 0; s < nslab && ok; s++) {
-                if (!BDBL && s > 0) {
-                    if (!mbar_wait_or_abort(smem_u32(&bempty[0]), bphase(s - 1), p.err)) { ok = false; break; }
-                    issue_b(s);
-                }
-                for (int u = 0; u < NU; u++) {
-                    if (BDBL && u == NU / 2 && s + 1 < nslab) {
-                        if (s >= 1 && !mbar_wait_or_abort(smem_u32(&bempty[(s + 1) & 1]), bphase(s - 1), p.err)) {
+            for (int t = t0; t < t1 && ok; t += dt) {
+                if (!is_active(t)) continue;
+                const int bl = t / p.tiles;
+                int m0, n0;
+                oz_tile<BN>(g, t - bl * p.tiles, m0, n0);
+                for (int s = 0; s < nslab && ok; s++) {
+                    if (nb > 0 && !mbar_wait_or_abort(smem_u32(&bempty), (uint32_t)((nb - 1) & 1), p.err)) { ok = false; break; }
+                    mbar_expect_tx(smem_u32(&bfull), (uint32_t)(OZ_S * SLAB_B));
+                    oz_tma_load(sbase, &p.tb, s * OZ_KS, n0, bl * OZ_S, smem_u32(&bfull));
+                    nb++;
+                    for (int u = 0; u < NU; u++) {
+                        const int slot = q % RING;
+                        if (q >= RING &&
+                            !mbar_wait_or_abort(smem_u32(&aempty[slot]), (uint32_t)(((q / RING) - 1) & 1), p.err)) {
                             ok = false;
                             break;
                         }
-                        issue_b(s + 1);
+                        mbar_expect_tx(smem_u32(&afull[slot]), (uint32_t)(OZ_UNIT * OZ_SLAB_A));
+                        oz_tma_load(sA(slot), &p.ta, s * OZ_KS, m0, bl * OZ_S + OZ_UNIT * u, smem_u32(&afull[slot]));
+                        q++;
                     }
-                    const int slot = q % RING;
-                    if (q >= RING &&
-                        !mbar_wait_or_abort(smem_u32(&aempty[slot]), (uint32_t)(((q / RING) - 1) & 1), p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_expect_tx(smem_u32(&afull[slot]), (uint32_t)(OZ_UNIT * OZ_SLAB_A));
-                    oz_tma_load(sA(slot), &p.ta, s * OZ_KS, m0, bl * OZ_S + OZ_UNIT * u, smem_u32(&afull[slot]));
-                    q++;
+                    if (*(volatile int*)&abort_flag) ok = false;
                 }
-                if (*(volatile int*)&abort_flag) ok = false;
             }
             if (!ok) abort_flag = 1;
             // every load issued has landed before the CTA can leave
-            for (int x = (nb > NB ? nb - NB : 0); x < nb; x++)
-                mbar_wait(smem_u32(&bfull[bslot(x)]), bphase(x), p.err);
+            if (nb > 0) mbar_wait(smem_u32(&bfull), (uint32_t)((nb - 1) & 1), p.err);
             for (int x = (q > RING ? q - RING : 0); x < q; x++)
                 mbar_wait(smem_u32(&afull[x % RING]), (uint32_t)((x / RING) & 1), p.err);
         }
     } else if (warp == EPIW + 1) {
         if (lane == 0) {            // MMA issuer
             constexpr int MAXB = 256 / BN;             // B slices per MMA (N <= 256)
-            // descriptors of slot 0 / buffer 0 slice 0; other slabs offset the 16-byte address field
-            const uint64_t dA0 = tma_smem_desc(sA(0)), dB0 = tma_smem_desc(sB(0, 0));
-            int q = 0;
+            // descriptors of slot 0 / slice 0; other slots and slices offset the 16-byte address field
+            const uint64_t dA0 = tma_smem_desc(sA(0)), dB0 = tma_smem_desc(sbase);
+            auto commit = [](uint64_t& bar) {
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(smem_u32(&bar)) : "memory");
+            };
+            int nb = 0, q = 0, nt = 0;                 // slabs, units and tiles taken
             bool ok = true;
-            for (int s = 0; s < nslab && ok; s++) {
-                const int bb = bslot(s);
-                if (!mbar_wait_or_abort(smem_u32(&bfull[bb]), bphase(s), p.err)) {
-                    ok = false;
-                    break;
-                }
-                const int kv = min(OZ_KS, g.k - s * OZ_KS);
-                const int nk16 = (kv + 15) / 16;
-                const uint64_t dB = dB0 + (uint64_t)((bb * OZ_S * SLAB_B) >> 4);
-                for (int u = 0; u < OZ_S / OZ_UNIT; u++, q++) {
-                    const int slot = q % RING;
-                    if (!mbar_wait_or_abort(smem_u32(&afull[slot]), (uint32_t)((q / RING) & 1), p.err)) {
+            for (int t = t0; t < t1 && ok; t += dt) {
+                if (!is_active(t)) continue;
+                // the accumulators have been drained
+                if (nt > 0 && !mbar_wait_or_abort(smem_u32(&tempty), (uint32_t)((nt - 1) & 1), p.err)) { ok = false; break; }
+                nt++;
+                for (int s = 0; s < nslab && ok; s++, nb++) {
+                    if (!mbar_wait_or_abort(smem_u32(&bfull), (uint32_t)(nb & 1), p.err)) {
                         ok = false;
                         break;
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const int kv = min(OZ_KS, g.k - s * OZ_KS);
+                    const int nk16 = (kv + 15) / 16;
+                    for (int u = 0; u < NU; u++, q++) {
+                        const int slot = q % RING;
+                        if (!mbar_wait_or_abort(smem_u32(&afull[slot]), (uint32_t)((q / RING) & 1), p.err)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-                    for (int h = 0; h < OZ_UNIT; h++) {
-                        const int i = oz_order(OZ_UNIT * u + h);
-                        const uint64_t da = dA0 + (uint64_t)(((slot * OZ_UNIT + h) * OZ_SLAB_A) >> 4);
-                        // the first slice (i = 0, taken first) opens every group's accumulator
-                        const uint32_t first = (s == 0 && u == 0 && h == 0) ? 1u : 0u;
-                        // products (i, j), j = 0 .. 7 - i, land in groups i .. 7: adjacent 64-column
-                        // accumulators, and the B slices j are adjacent 64-row blocks in shared
-                        // memory, so one MMA of N = 64 (8 - i) (at most 256 per instruction) covers them
+                        for (int h = 0; h < OZ_UNIT; h++) {
+                            const int i = oz_order(OZ_UNIT * u + h);
+                            const uint64_t da = dA0 + (uint64_t)(((slot * OZ_UNIT + h) * OZ_SLAB_A) >> 4);
+                            // the first slice (i = 0, taken first) opens every group's accumulator
+                            const uint32_t first = (s == 0 && u == 0 && h == 0) ? 1u : 0u;
+                            // products (i, j), j = 0 .. 7 - i, land in groups i .. 7: adjacent BN-column
+                            // accumulators, and the B slices j are adjacent BN-row blocks in shared
+                            // memory, so one MMA of N = BN (8 - i) (at most 256 per instruction) covers them
 #pragma unroll
-                        for (int kk = 0; kk < OZ_KS / 16; kk++) {
-                            if (kk < nk16) {
+                            for (int kk = 0; kk < OZ_KS / 16; kk++) {
+                                if (kk < nk16) {
 #pragma unroll
-                                for (int c = 0; c < OZ_S; c += MAXB) {
-                                    const int nb = min(MAXB, OZ_S - i - c);
-                                    if (nb > 0) {
-                                        const uint32_t acc = tmem + (uint32_t)((i + c) * BN);
-                                        const uint64_t db = dB + (uint64_t)((c * SLAB_B) >> 4) + 2 * kk;
-                                        tc_mma(acc, da + 2 * kk, db, tc_idesc(TC_BF16, BN * nb),
-                                               (first && kk == 0) ? 0u : 1u, TC_BF16);
+                                    for (int c = 0; c < OZ_S; c += MAXB) {
+                                        const int nn = min(MAXB, OZ_S - i - c);
+                                        if (nn > 0) {
+                                            const uint32_t acc = tmem + (uint32_t)((i + c) * BN);
+                                            const uint64_t db = dB0 + (uint64_t)((c * SLAB_B) >> 4) + 2 * kk;
+                                            tc_mma(acc, da + 2 * kk, db, tc_idesc(TC_BF16, BN * nn),
+                                                   (first && kk == 0) ? 0u : 1u, TC_BF16);
+                                        }
                                     }
                                 }
                             }
                         }
+                        commit(aempty[slot]);
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                 :: "r"(smem_u32(&aempty[slot])) : "memory");
+                    if (!ok) break;
+                    commit(bempty);
+                    if (s == nslab - 1) commit(tfull);
+                    if (*(volatile int*)&abort_flag) ok = false;
                 }
-                if (!ok) break;
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(smem_u32(&bempty[bb])) : "memory");
-                if (s == nslab - 1)
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                 :: "r"(smem_u32(&tfull)) : "memory");
-                if (*(volatile int*)&abort_flag) ok = false;
             }
             if (!ok) abort_flag = 1;
             // every MMA issued has completed before TMEM is freed
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(&done)) : "memory");
+            commit(done);
             mbar_wait(smem_u32(&done), 0u, p.err);
         }
     } else {
@@ -558,11 +561,19 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
         // the one thread that computes it (Cin may be C itself).
         constexpr int PCOLS = BN / (EPIW / 4), PASSES = PCOLS / 4;
         static_assert(PCOLS % 4 == 0, "four-column passes");
+        const int lq = warp & 3, part = warp >> 2;          // lane quarter, column part
+        int nt = 0;                                         // tiles drained
+        bool ok = true;
+        for (int t = t0; t < t1 && ok; t += dt) {
+        const bool active = is_active(t);
+        if (!active && g.skip_inactive) continue;
+        const int bl = t / p.tiles, b = p.b0 + bl;
+        int m0, n0;
+        oz_tile<BN>(g, t - bl * p.tiles, m0, n0);
         const double* Cinb = g.Cin ? g.Cin[b] + g.offCin : nullptr;
         const double* Cin2b = g.Cin2 ? g.Cin2[b] + g.offCin : nullptr;
         double* Cb = g.C[b] + g.offC;
         const bool skew = g.mode == GEMM_SKEW, gj = g.mode == GEMM_GJ;
-        const int lq = warp & 3, part = warp >> 2;          // lane quarter, column part
         const int row = m0 + lq * 32 + lane, cp0 = n0 + part * PCOLS;
         const bool use_cin = Cinb && (!active || g.beta != 0.0);
         const bool ct = g.cin_trans != 0;
@@ -598,33 +609,43 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
         };
         unsigned long long ci[4], cn[4];
         load_cin(ci, cp0);                                   // in flight while the MMAs run
-        bool ok = true;
-        if (nslab > 0) {
-            if (lane == 0) ok = mbar_wait_or_abort(smem_u32(&tfull), 0u, p.err);
+        const int er = (active && row < g.m) ? p.ea[(size_t)bl * p.m_pad + row] : 0;
+        // the exponent fields of this part's columns, one per lane
+        const int fe = (active && lane < PCOLS && cp0 + lane < g.n) ? p.eb[(size_t)bl * p.n_pad + cp0 + lane] : 0;
+        if (active) {
+            if (lane == 0) ok = mbar_wait_or_abort(smem_u32(&tfull), (uint32_t)(nt & 1), p.err);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            nt++;
         }
         if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;");
             const double alpha = g.alpha * (g.alpha_b ? g.alpha_b[b] : 1.0);
-            const int er = (active && row < g.m) ? p.ea[(size_t)bl * p.m_pad + row] : 0;
             const int ae = p.alpha_pow2 ? p.alpha_e : 0;
             const bool an = p.alpha_pow2 && p.alpha_neg;
             // every result of this warp's rows is a normal number: with e = er + fc - 2107 + ae and
             // the leading bit P of |V| in 0 .. 74, the biased exponent P + e + 1023 stays in 1 .. 2046
             // (rows or columns with a zero exponent field give zeros either way); then the
             // combination takes the form without the range-end selects (the same bits)
-            const int fe = lane < PCOLS ? col_e[part * PCOLS + lane] : 0;
             const int fcmin = __reduce_min_sync(0xffffffffu, fe > 0 ? fe : 4096);
             const int fcmax = __reduce_max_sync(0xffffffffu, fe);
             const bool row_normal = er == 0 || fcmax == 0 ||
                                     (er + fcmin - 2107 + ae + 1023 >= 1 && er + fcmax - 2107 + ae + 1023 + 74 <= 2046);
             const bool fast = __all_sync(0xffffffffu, row_normal);
+            // this warp has read its accumulators: the next tile's MMAs may start
+            bool held = active;
+            auto release = [&] {
+                held = false;
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&tempty)) : "memory");
+            };
 #pragma unroll 1
             for (int pass = 0; pass < PASSES; pass++) {
                 const int cl = part * PCOLS + 4 * pass, c0 = n0 + cl;
                 if (c0 >= g.n || (skew && m0 + lq * 32 + 31 < c0)) break;     // warp-uniform
                 unsigned long long t[4] = {0ull, 0ull, 0ull, 0ull};
-                if (nslab > 0) {
+                if (active) {
                     uint32_t u[OZ_G][4];
 #pragma unroll
                     for (int G = 0; G < OZ_G; G++) {
@@ -635,10 +656,11 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
                     }
                     if (pass + 1 < PASSES) load_cin(cn, c0 + 4);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (pass == PASSES - 1) release();
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
                         // computed for every column and selected (no branch between the columns)
-                        const int fc = col_e[cl + j];
+                        const int fc = __shfl_sync(0xffffffffu, fe, 4 * pass + j);
                         long long H;
                         unsigned L;
                         oz_combine(u, j, H, L);
@@ -713,8 +735,10 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), BDBL ? 1 : 2) oz_gemm_kernel(
 #pragma unroll
                 for (int j = 0; j < 4; j++) ci[j] = cn[j];
             }
+            if (held) release();
         } else if (lane == 0) {
             abort_flag = 1;
+        }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -814,6 +838,17 @@ inline int oz_chunk_entries(const GemmBatch& g, const OzBuf& buf) {
     return (int)std::min<size_t>(g.batch, buf.bytes > 8192 ? (buf.bytes - 8192) / per : 0);
 }
 
+// SMs of the current device
+inline int oz_sms() {
+    static std::atomic<int> known[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    if ((n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+    known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 // the product kernel on slices in place (layout L) for batch entries b0 .. b0 + bc - 1;
 // b_rows: B's slices are its rows (an antisymmetric B), so alpha changes sign
 inline cudaError_t oz_product(const GemmBatch& g, const OzLayout& L, int b0, int bc, bool b_rows, int* err,
@@ -831,11 +866,14 @@ inline cudaError_t oz_product(const GemmBatch& g, const OzLayout& L, int b0, int
     if (!g.alpha_b && (fr == 0.5 || fr == -0.5)) {
         p.alpha_pow2 = 1; p.alpha_e = ex - 1; p.alpha_neg = p.g.alpha < 0.0;
     }
+    p.tiles = oz_tiles(g, bn);
+    p.total = p.tiles * bc;
+    // two CTAs per SM and no more: with a few CTAs over, those few run their tiles after all others
+    const unsigned grid = (unsigned)std::min(p.total, 2 * oz_sms());
     if (bn == 16)
-        oz_gemm_kernel<OZ_NARROW16>
-            <<<dim3(oz_tiles(g, bn), bc), OzCfg<OZ_NARROW16>::THREADS, OzCfg<OZ_NARROW16>::SMEM, st>>>(p);
+        oz_gemm_kernel<OZ_NARROW16><<<grid, OzCfg<OZ_NARROW16>::THREADS, OzCfg<OZ_NARROW16>::SMEM, st>>>(p);
     else
-        oz_gemm_kernel<OZ_NARROW><<<dim3(oz_tiles(g, bn), bc), OzCfg<OZ_NARROW>::THREADS, OzCfg<OZ_NARROW>::SMEM, st>>>(p);
+        oz_gemm_kernel<OZ_NARROW><<<grid, OzCfg<OZ_NARROW>::THREADS, OzCfg<OZ_NARROW>::SMEM, st>>>(p);
     return cudaGetLastError();
 }
 
