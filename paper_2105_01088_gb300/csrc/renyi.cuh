@@ -15,11 +15,12 @@
 // of ordered pairs (u <= v) are evaluated once.
 #pragma once
 #include "common.cuh"
+#include "factor.cuh"
 #include "pair.cuh"
 
 namespace sgs {
 
-#define RENYI_MAX_DIM 104     // 2 * 2 N_A <= 104 (impurity + up to 12 sites) in one CTA's shared memory
+#define RENYI_MAX_DIM 152     // 2 * 2 N_A <= 152 (impurity + up to 18 sites) in one CTA's shared memory
 
 // blocks[u] = Delta^{ab}_A (complex, na2 x na2), w[u] = lambda_a conj(lambda_b) G_ba, u = a M + b
 __global__ void renyi_blocks_kernel(InstDev d, const double* si, const double* imd, const double* Gm,
@@ -51,98 +52,159 @@ __global__ void renyi_blocks_kernel(InstDev d, const double* si, const double* i
     }
 }
 
-// one CTA per unordered pair (u <= v) of ordered pairs: complex Parlett-Reid in shared memory
+// dynamic shared memory of renyi_pf_kernel: the packed upper triangles (re, im), four vectors, and the packed
+// entries' row and column
+inline size_t renyi_smem(int m) {
+    return (size_t)m * (m - 1) / 2 * (2 * sizeof(double) + 2) + 4 * (size_t)m * sizeof(double) + 16;
+}
+
+// One CTA per unordered pair (u <= v) of ordered pairs: complex Parlett-Reid elimination of
+// Z = [[Delta_u, i 1], [-i 1, Delta_v]] in shared memory.  Z is antisymmetric: only its upper triangle is kept,
+// packed by rows, so that what is live after a step is the tail of the storage and every lane of the rank-2
+// update has an element (their rows and columns from a table).  The step's rows k and q = k + 1 are done after
+// it, so the interchange of q and the pivot p only writes row and column p.
+// Bound by the FP64 pipe: 8 FMAs per live element and step, m^3 / 12 elements in all.  2080 matrices' worth of
+// the earlier form (both triangles, the scaled row formed again for every element, a logarithm per step) took
+// 8.0 ms for m = 24, 64 and 104 at 666 matrices each.
 __global__ void __launch_bounds__(256) renyi_pf_kernel(const double* blocks, const double* w, long long npairs,
                                                        int na2, double log_norm, double* partial) {
     extern __shared__ double sm[];
-    const int m = 2 * na2;
-    const int ld = m + 1;
-    double* Zr = sm;
-    double* Zi = sm + (size_t)m * ld;
-    __shared__ double red_v[32];
-    __shared__ int red_i[32];
-    __shared__ double s_log, s_pr, s_pi;
-    const long long q = blockIdx.x + (long long)blockIdx.y * gridDim.x;
-    if (q >= npairs) return;
-    // decode q = v (v + 1) / 2 + u, u <= v
-    long long v = (long long)((sqrt(8.0 * (double)q + 1.0) - 1.0) * 0.5);
-    while ((v + 1) * (v + 2) / 2 <= q) ++v;
-    while (v * (v + 1) / 2 > q) --v;
-    const long long u = q - v * (v + 1) / 2;
-    const double* Bu = blocks + (size_t)u * na2 * na2 * 2;
-    const double* Bv = blocks + (size_t)v * na2 * na2 * 2;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int r = e / m, c = e % m;
-        double zr = 0.0, zi = 0.0;
-        if (r < na2 && c < na2) { zr = Bu[2 * (r * na2 + c)]; zi = Bu[2 * (r * na2 + c) + 1]; }
-        else if (r >= na2 && c >= na2) { zr = Bv[2 * ((r - na2) * na2 + c - na2)]; zi = Bv[2 * ((r - na2) * na2 + c - na2) + 1]; }
-        else if (c == r + na2) zi = 1.0;          // i 1
-        else if (r == c + na2) zi = -1.0;         // -i 1
-        Zr[r * ld + c] = zr;
-        Zi[r * ld + c] = zi;
+    const int m = 2 * na2, T = m * (m - 1) / 2, NT = blockDim.x, NW = NT >> 5;
+    double* Zr = sm;                            // row i, column j > i at off(i) + j
+    double* Zi = Zr + T;
+    double* tr = Zi + T;                        // tau and u of the step
+    double* ti = tr + m;
+    double* ur = ti + m;
+    double* ui = ur + m;
+    uchar2* ij = reinterpret_cast<uchar2*>(ui + m);
+    __shared__ long long red_v[8];
+    __shared__ int red_i[8];
+    __shared__ double s_inv[2], s_pr[RENYI_MAX_DIM / 2], s_pi[RENYI_MAX_DIM / 2];
+    __shared__ long long s_u, s_v;
+    __shared__ int s_flip;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto off = [m](int i) { return i * (2 * m - i - 1) / 2 - i - 1; };
+    const long long q0 = blockIdx.x + (long long)blockIdx.y * gridDim.x;
+    if (q0 >= npairs) return;
+    if (tid == 0) {             // decode q0 = v (v + 1) / 2 + u, u <= v
+        long long v = (long long)((sqrt(8.0 * (double)q0 + 1.0) - 1.0) * 0.5);
+        while ((v + 1) * (v + 2) / 2 <= q0) ++v;
+        while (v * (v + 1) / 2 > q0) --v;
+        s_v = v;
+        s_u = q0 - v * (v + 1) / 2;
+        s_flip = 0;
     }
-    if (threadIdx.x == 0) { s_log = 0.0; s_pr = 1.0; s_pi = 0.0; }
+    __syncthreads();
+    const long long u = s_u, v = s_v;
+    const double2* Bu = reinterpret_cast<const double2*>(blocks) + (size_t)u * na2 * na2;
+    const double2* Bv = reinterpret_cast<const double2*>(blocks) + (size_t)v * na2 * na2;
+    for (int i = warp; i < m - 1; i += NW)
+        for (int j = i + 1 + lane; j < m; j += 32) {
+            double2 z = make_double2(0.0, 0.0);
+            if (j < na2) z = Bu[i * na2 + j];
+            else if (i >= na2) z = Bv[(i - na2) * na2 + j - na2];
+            else if (j == i + na2) z.y = 1.0;               // i 1
+            const int e = off(i) + j;
+            Zr[e] = z.x;
+            Zi[e] = z.y;
+            ij[e] = make_uchar2((unsigned char)i, (unsigned char)j);
+        }
     __syncthreads();
     bool zero = false;
     for (int k = 0; k < m - 1; k += 2) {
-        double best = -1.0;
-        int bi = 0x7fffffff;
-        for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) {
-            const double x = Zr[i * ld + k] * Zr[i * ld + k] + Zi[i * ld + k] * Zi[i * ld + k];
-            if (x > best) { best = x; bi = i; }
+        const int q = k + 1, ok = off(k), oq = off(q);
+        // the pivot: the largest entry of row k, the smaller column on a tie
+        long long key = -1;
+        int p = 0x7fffffff;
+        for (int i = q + tid; i < m; i += NT) {
+            const double x = Zr[ok + i], y = Zi[ok + i];
+            const long long m2 = abs_key(fma(x, x, y * y));
+            if (m2 > key) { key = m2; p = i; }
         }
-        double mv;
-        int p;
-        block_argmax(best, bi, red_v, red_i, mv, p);
-        if (!(mv > 0.0)) { zero = true; break; }
-        if (p != k + 1) {
-            const int a = k + 1;
-            for (int j = threadIdx.x; j < m; j += blockDim.x) {
-                double t = Zr[a * ld + j]; Zr[a * ld + j] = Zr[p * ld + j]; Zr[p * ld + j] = t;
-                t = Zi[a * ld + j]; Zi[a * ld + j] = Zi[p * ld + j]; Zi[p * ld + j] = t;
+        warp_argmax(key, p);
+        if (lane == 0) { red_v[warp] = key; red_i[warp] = p; }
+        __syncthreads();
+        key = lane < NW ? red_v[lane] : -1ll;
+        p = lane < NW ? red_i[lane] : 0x7fffffff;
+        warp_argmax(key, p);
+        if (!(key > 0 && key <= 0x7FF0000000000000ll)) { zero = true; break; }     // zero (or NaN)
+        const int op = off(p);
+        if (tid == NT - 1) {
+            const double pr = Zr[ok + p], pi = Zi[ok + p];
+            const double rm = 1.0 / fma(pr, pr, pi * pi);
+            s_inv[0] = pr * rm;
+            s_inv[1] = -pi * rm;
+            s_pr[k >> 1] = pr;
+            s_pi[k >> 1] = pi;
+            if (p != q) s_flip ^= 1;
+        }
+        // u_i = -Z'[q][i] with the interchange of q and p: Z'[q][i] = Z[p][i] (i > p), -Z[i][p] (q < i < p),
+        // -Z[q][p] (i = p); Z'[p][i] = Z[q][i], Z'[i][p] = -Z[q][i]
+        for (int i = q + 1 + tid; i < m; i += NT) {
+            const double zr = Zr[oq + i], zi = Zi[oq + i];
+            if (i == p) {
+                ur[i] = zr;
+                ui[i] = zi;
+            } else {
+                const int e = i > p ? op + i : off(i) + p;
+                const double yr = p == q ? zr : Zr[e], yi = p == q ? zi : Zi[e];
+                ur[i] = i > p ? -yr : yr;
+                ui[i] = i > p ? -yi : yi;
+                if (p != q) {
+                    Zr[e] = i > p ? zr : -zr;
+                    Zi[e] = i > p ? zi : -zi;
+                }
             }
-            __syncthreads();
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                double t = Zr[i * ld + a]; Zr[i * ld + a] = Zr[i * ld + p]; Zr[i * ld + p] = t;
-                t = Zi[i * ld + a]; Zi[i * ld + a] = Zi[i * ld + p]; Zi[i * ld + p] = t;
-            }
-            if (threadIdx.x == 0) { s_pr = -s_pr; s_pi = -s_pi; }
-            __syncthreads();
         }
-        const double pr = Zr[k * ld + k + 1], pi = Zi[k * ld + k + 1];
-        const double pm2 = pr * pr + pi * pi;
-        if (threadIdx.x == 0) {
-            const double am = sqrt(pm2);
-            s_log += log(am);
-            const double ur = pr / am, ui = pi / am;
-            const double nr = s_pr * ur - s_pi * ui, ni = s_pr * ui + s_pi * ur;
-            s_pr = nr; s_pi = ni;
+        __syncthreads();
+        for (int i = q + 1 + tid; i < m; i += NT) {         // tau_i = Z'[k][i] / pivot
+            const int e = ok + (i == p ? q : i);
+            const double xr = Zr[e], xi = Zi[e], ir = s_inv[0], ii = s_inv[1];
+            tr[i] = xr * ir - xi * ii;
+            ti[i] = xr * ii + xi * ir;
         }
-        // A[k+2:, k+2:] += tau u^T - u tau^T with tau = A[k, k+2:] / pivot, u = A[k+2:, k+1]
-        const double ir = pr / pm2, ii = -pi / pm2;
-        const int t0 = k + 2, mt = m - t0;
-        for (int e = threadIdx.x; e < mt * mt; e += blockDim.x) {
-            const int i = t0 + e / mt, j = t0 + e % mt;
-            const double ti_r = Zr[k * ld + i] * ir - Zi[k * ld + i] * ii, ti_i = Zr[k * ld + i] * ii + Zi[k * ld + i] * ir;
-            const double tj_r = Zr[k * ld + j] * ir - Zi[k * ld + j] * ii, tj_i = Zr[k * ld + j] * ii + Zi[k * ld + j] * ir;
-            const double uj_r = Zr[j * ld + k + 1], uj_i = Zi[j * ld + k + 1];
-            const double ui_r = Zr[i * ld + k + 1], ui_i = Zi[i * ld + k + 1];
-            Zr[i * ld + j] += (ti_r * uj_r - ti_i * uj_i) - (ui_r * tj_r - ui_i * tj_i);
-            Zi[i * ld + j] += (ti_r * uj_i + ti_i * uj_r) - (ui_r * tj_i + ui_i * tj_r);
+        __syncthreads();
+        // Z[i][j] += tau_i u_j - u_i tau_j on the live triangle, rows k + 2 on
+        for (int e = off(k + 2) + k + 3 + tid; e < T; e += NT) {
+            const uchar2 x = ij[e];
+            const double ar = tr[x.x], ai = ti[x.x], br = ur[x.x], bi = ui[x.x];
+            const double cr = tr[x.y], ci = ti[x.y], dr = ur[x.y], di = ui[x.y];
+            double r = Zr[e], s = Zi[e];
+            r = fma(ar, dr, r);
+            s = fma(ar, di, s);
+            r = fma(-ai, di, r);
+            s = fma(ai, dr, s);
+            r = fma(-br, cr, r);
+            s = fma(-br, ci, s);
+            r = fma(bi, ci, r);
+            s = fma(-bi, cr, s);
+            Zr[e] = r;
+            Zi[e] = s;
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        double tr = 0.0, ti = 0.0;
-        if (!zero) {
-            const cplx wu = cmk(w[2 * u], w[2 * u + 1]), wv = cmk(w[2 * v], w[2 * v + 1]);
-            cplx x = cmul(cmul(wu, wv), cmk(s_pr, s_pi));
-            const double mag = exp(s_log + log_norm) * (u < v ? 2.0 : 1.0);
-            tr = x.x * mag;
-            ti = x.y * mag;
+    // the pivots' product as mantissa and exponent of two, by one warp
+    if (warp == 0) {
+        int e = 0;
+        cplx x = cmk(1.0, 0.0);
+        for (int t = lane; t < m / 2 && !zero; t += 32) {
+            x = cmul(x, cmk(s_pr[t], s_pi[t]));
+            const int f = min(max(2046 - max(expo_field(x.x), expo_field(x.y)), 1), 2046);
+            x = cscale(x, __hiloint2double(f << 20, 0));    // 2^(f - 1023)
+            e += 1023 - f;
         }
-        partial[2 * q] = tr;
-        partial[2 * q + 1] = ti;
+        for (int o = 16; o > 0; o >>= 1) {
+            x = cmul(x, cmk(__shfl_xor_sync(0xffffffffu, x.x, o), __shfl_xor_sync(0xffffffffu, x.y, o)));
+            e += __shfl_xor_sync(0xffffffffu, e, o);
+        }
+        if (lane == 0) {
+            if (zero) x = cmk(0.0, 0.0);
+            const cplx wu = cmk(w[2 * u], w[2 * u + 1]), wv = cmk(w[2 * v], w[2 * v + 1]);
+            const double mag = exp(e * 0.693147180559945309417 + log_norm) * (u < v ? 2.0 : 1.0);
+            x = cscale(cmul(cmul(wu, wv), x), s_flip ? -mag : mag);
+            partial[2 * q0] = zero ? 0.0 : x.x;
+            partial[2 * q0 + 1] = zero ? 0.0 : x.y;
+        }
     }
 }
 

@@ -2404,11 +2404,11 @@ sgs_status sgs_correlator(sgs_ctx* c, int instance, sgs_corr_kind kind, const in
             counted();
             const double log_norm = -(na2 / 2) * 0.6931471805599453;
             if (m <= RENYI_MAX_DIM) {
-                const size_t smem = 2 * (size_t)m * (m + 1) * sizeof(double);
                 set_kernel_attributes();
                 const unsigned gx = (unsigned)std::min<long long>(npairs, 65535);
                 const unsigned gy = (unsigned)((npairs + gx - 1) / gx);
-                renyi_pf_kernel<<<dim3(gx, gy), 256, smem, c->stream>>>(blocks, wts, npairs, na2, log_norm, partial);
+                renyi_pf_kernel<<<dim3(gx, gy), m <= 48 ? 128 : 256, renyi_smem(m), c->stream>>>(blocks, wts, npairs, na2,
+                                                                                        log_norm, partial);
                 counted();
             } else {
                 sgs_status rs = renyi_large(c, I, blocks, wts, npairs, na2, log_norm, partial);
