@@ -104,18 +104,83 @@ __global__ void __launch_bounds__(256) eom_pairs_kernel(InstDev d, const double*
     store_antisym_tile(out, n, k0, l0, st[1]);
 }
 
-// parts of eom_finish_kernel: the pairs' impurity terms (per chunk of pairs), the rest (the
-// sparse A terms on the summed T and sum w2 of every pair, and the beta = mu term), or both
+// parts of the assembly's end: the pairs' impurity terms (per chunk of pairs, eom_imp_kernel), the rest
+// (the sparse A terms on the summed T and sum w2 of every pair, and the beta = mu term,
+// eom_finish_kernel), or both in that order: the rest first
 enum { EOM_FINISH_PAIRS = 1, EOM_FINISH_REST = 2, EOM_FINISH_ALL = 3 };
+
+// The pairs' F_imp terms of [Delta, F] and Q + F on the rows and columns of the impurity modes: a warp per
+// entry (a, imp[j]) of a state, its lanes over the pairs, whose loads are then in flight together (one thread
+// that walked the pairs of its entry took 0.48 of the assembly's 0.58 ms at n = 244, M = 16).  Float terms
+// are added to the entry in the order of the pairs.  Grid (ceil(n nimp / 8), M), 256 threads.
+template <typename R>
+__global__ void __launch_bounds__(256) eom_imp_kernel(InstDev d, const double* si, const double* imd, const double* fimp,
+                                                      const double* coef, const int* pair_index, double* dgamma) {
+    const int mu = blockIdx.y, n = d.n, ni = d.nimp, M = d.M, lane = threadIdx.x & 31;
+    const int t = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (t >= n * ni) return;
+    const int a = t / ni, b = d.imp[t % ni], sa = d.slot[a];
+    if (a == b || (sa >= 0 && a < b)) return;          // an entry of two impurity modes: once
+    const int k = max(a, b), l = min(a, b), sk = d.slot[k], sl = d.slot[l];
+    const size_t N = nn(d);
+    double* out = dgamma + (size_t)mu * N;
+    R acc = (R)out[(size_t)k * n + l];
+    R sum = 0;
+    for (int b0 = 0; b0 < M; b0 += 32) {
+        const int be = b0 + lane;
+        const int p = be < M && be != mu ? pair_index[mu * M + be] - d.p_off : -1;
+        const bool held = p >= 0 && p < d.p_cnt;       // not another chunk's or another rank's
+        R term = 0;
+        if (held) {
+            const R sgn = (d.pa[p] == mu) ? (R)-1 : (R)1;
+            const double* s = si + (size_t)p * N;
+            const double* im = imd + (size_t)p * N;
+            const double* fp = fimp + (size_t)p * ni * ni * 2;
+            R dfx = 0, dfy = 0, fdx = 0, fdy = 0, Fx = 0, Fy = 0;
+            if (sl >= 0)
+                for (int m = 0; m < ni; m++) {
+                    const R ax = (R)-2 * (R)s[(size_t)k * n + d.imp[m]], ay = sgn * (R)im[(size_t)k * n + d.imp[m]];
+                    const R bx = (R)fp[2 * (m * ni + sl)], by = sgn * (R)fp[2 * (m * ni + sl) + 1];
+                    dfx += ax * bx - ay * by;
+                    dfy += ax * by + ay * bx;
+                }
+            if (sk >= 0)
+                for (int m = 0; m < ni; m++) {
+                    const R ax = (R)fp[2 * (sk * ni + m)], ay = sgn * (R)fp[2 * (sk * ni + m) + 1];
+                    const R bx = (R)-2 * (R)s[(size_t)d.imp[m] * n + l], by = sgn * (R)im[(size_t)d.imp[m] * n + l];
+                    fdx += ax * bx - ay * by;
+                    fdy += ax * by + ay * bx;
+                }
+            if (sk >= 0 && sl >= 0) {
+                Fx = (R)fp[2 * (sk * ni + sl)];
+                Fy = sgn * (R)fp[2 * (sk * ni + sl) + 1];
+            }
+            const double* co = coef + (size_t)(mu * M + be) * 6;
+            term = (R)2 * ((R)co[0] * (dfx - fdx) - (R)co[1] * (dfy - fdy) + (R)co[2] * Fx - (R)co[3] * Fy);
+        }
+        if (sizeof(R) == sizeof(float)) {
+            unsigned m = __ballot_sync(0xffffffffu, held);
+            for (; m; m &= m - 1) acc += __shfl_sync(0xffffffffu, term, __ffs(m) - 1);
+        } else {
+            sum += term;
+        }
+    }
+    if (sizeof(R) != sizeof(float)) {
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        acc += sum;
+    }
+    if (lane == 0) {
+        out[(size_t)k * n + l] = (double)acc;
+        out[(size_t)l * n + k] = -(double)acc;
+    }
+}
 
 // self_mask (may be nullptr): state mu's beta = mu term is added only where self_mask[mu] != 0
 // (a pair-sharded step adds it on one rank, so that the ranks' partial sums add up to dGamma)
 template <typename R>
-__global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double* si, const double* imd,
-                                                         const double* fimp, const double* fimp_state,
-                                                         const double* gfg, const double* coef, const int* pair_index,
-                                                         const double* tsum, double* dgamma, const int* self_mask,
-                                                         int part) {
+__global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double* fimp_state, const double* gfg,
+                                                         const double* coef, const int* pair_index, const double* tsum,
+                                                         double* dgamma, const int* self_mask) {
     extern __shared__ double eom_sraw[];
     __shared__ R s_w2;
     __shared__ double sf[32][33];
@@ -134,8 +199,7 @@ __global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double
     }
     __syncthreads();
     const size_t N = nn(d);
-    const bool rest = (part & EOM_FINISH_REST) != 0, pair_imp = (part & EOM_FINISH_PAIRS) != 0;
-    const bool self_term = rest && (self_mask == nullptr || self_mask[mu] != 0);
+    const bool self_term = self_mask == nullptr || self_mask[mu] != 0;
     const double* gm = d.gamma + (size_t)mu * N;
     const double* fs = fimp_state + (size_t)mu * ni * ni;
     const double* gfgm = gfg + (size_t)mu * N;
@@ -155,7 +219,6 @@ __global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double
         }
         const size_t e = (size_t)k * n + l;
         const int sk = d.slot[k], sl = d.slot[l];
-        if (!rest && sk < 0 && sl < 0) continue;            // the pairs' impurity terms only
         // one pass over each of the CSR rows l and k of A (read-only loads) for A_kl, the pairs'
         // commutator terms against A, -(T A^T)_kl - (A T)_kl, and the beta = mu term's
         // (Gamma F)_kl, (F Gamma)_kl: the T and Gamma loads of a row entry issue together
@@ -165,7 +228,7 @@ __global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double
             for (int q = q0; q < q1; q++) {
                 const int cq = __ldg(d.a_col + q);
                 const R v = (R)__ldg(d.a_val + q);
-                if (rest) ta = fma((R)T[(size_t)k * n + cq], v, ta);
+                ta = fma((R)T[(size_t)k * n + cq], v, ta);
                 if (self_term) gf = fma(-(R)gm[(size_t)k * n + cq], v, gf);
             }
         }
@@ -175,15 +238,13 @@ __global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double
                 const int cq = __ldg(d.a_col + q);
                 const R v = (R)__ldg(d.a_val + q);
                 if (cq == l) akl = v;
-                if (rest) at = fma(v, (R)T[(size_t)cq * n + l], at);
+                at = fma(v, (R)T[(size_t)cq * n + l], at);
                 if (self_term) fg = fma(v, (R)gm[(size_t)cq * n + l], fg);
             }
         }
         R acc = (R)out[e];
-        if (rest) {
-            acc = fma(akl, s_w2, acc);
-            acc = acc - ta - at;
-        }
+        acc = fma(akl, s_w2, acc);
+        acc = acc - ta - at;
         if (self_term) {   // beta = mu: Delta = Gamma_mu, Delta F Delta = Gamma F Gamma
             const double* co = coef + (size_t)(mu * M + mu) * 6;
             const R g = (R)gm[e];
@@ -191,38 +252,6 @@ __global__ void __launch_bounds__(256) eom_finish_kernel(InstDev d, const double
             if (sl >= 0) for (int m = 0; m < ni; m++) gf += (R)gm[(size_t)k * n + d.imp[m]] * (R)fs[m * ni + sl];
             if (sk >= 0) for (int m = 0; m < ni; m++) fg += (R)fs[sk * ni + m] * (R)gm[(size_t)d.imp[m] * n + l];
             acc += (R)2 * ((R)co[0] * (gf - fg) + (R)co[2] * ((R)gfgm[e] + f) + (R)co[4] * g);
-        }
-        if (pair_imp && (sk >= 0 || sl >= 0)) {
-            // rows and columns of the impurity modes: the pairs' F_imp terms of [Delta, F] and Q + F
-            for (int be = 0; be < M; be++) {
-                const int p = sp[be];
-                if (p < 0) continue;
-                const R sgn = (d.pa[p] == mu) ? (R)-1 : (R)1;
-                const double* s = si + (size_t)p * N;
-                const double* im = imd + (size_t)p * N;
-                const double* fp = fimp + (size_t)p * ni * ni * 2;
-                R dfx = 0, dfy = 0, fdx = 0, fdy = 0, Fx = 0, Fy = 0;
-                if (sl >= 0)
-                    for (int m = 0; m < ni; m++) {
-                        const R ax = (R)-2 * (R)s[(size_t)k * n + d.imp[m]], ay = sgn * (R)im[(size_t)k * n + d.imp[m]];
-                        const R bx = (R)fp[2 * (m * ni + sl)], by = sgn * (R)fp[2 * (m * ni + sl) + 1];
-                        dfx += ax * bx - ay * by;
-                        dfy += ax * by + ay * bx;
-                    }
-                if (sk >= 0)
-                    for (int m = 0; m < ni; m++) {
-                        const R ax = (R)fp[2 * (sk * ni + m)], ay = sgn * (R)fp[2 * (sk * ni + m) + 1];
-                        const R bx = (R)-2 * (R)s[(size_t)d.imp[m] * n + l], by = sgn * (R)im[(size_t)d.imp[m] * n + l];
-                        fdx += ax * bx - ay * by;
-                        fdy += ax * by + ay * bx;
-                    }
-                if (sk >= 0 && sl >= 0) {
-                    Fx = (R)fp[2 * (sk * ni + sl)];
-                    Fy = sgn * (R)fp[2 * (sk * ni + sl) + 1];
-                }
-                const double* co = coef + (size_t)(mu * M + be) * 6;
-                acc += (R)2 * ((R)co[0] * (dfx - fdx) - (R)co[1] * (dfy - fdy) + (R)co[2] * Fx - (R)co[3] * Fy);
-            }
         }
         sf[j][tx] = (double)acc;
         sh[j][tx] = 1;

@@ -174,19 +174,31 @@ __global__ void __launch_bounds__(256) pair_gh_kernel(InstDev d, const double* s
     }
     tr_r = block_sum(tr_r, red);
     tr_i = block_sum(tr_i, red);
-    if (threadIdx.x == 0) {
-        cplx q = cmk(0.0, 0.0);
-        const int ni = d.nimp;
-        cplx F[SGS_MAX_IMP * SGS_MAX_IMP];
-        for (int e = 0; e < ni * ni; e++) F[e] = cmk(0.0, 0.0);
-        for (int e = 0; e < d.nq; e++) {
-            const int* ix = d.q_idx + 4 * e;
+    // The quartic entries are sorted by their indices, so those of one Fock entry (the first two indices)
+    // are consecutive: a thread takes the run that starts at its entry.  One thread over all of them took
+    // 320 us for the two-channel Kondo coupling's 576.
+    __shared__ cplx F[SGS_MAX_IMP * SGS_MAX_IMP];
+    const int ni = d.nimp;
+    for (int e = threadIdx.x; e < ni * ni; e += blockDim.x) F[e] = cmk(0.0, 0.0);
+    __syncthreads();
+    cplx q = cmk(0.0, 0.0);
+    for (int e0 = threadIdx.x; e0 < d.nq; e0 += blockDim.x) {
+        const int* ix = d.q_idx + 4 * e0;
+        const int i0 = ix[0], i1 = ix[1];
+        if (e0 > 0 && ix[-4] == i0 && ix[-3] == i1) continue;
+        cplx f = cmk(0.0, 0.0), qs = cmk(0.0, 0.0);
+        for (int e = e0; e < d.nq && ix[0] == i0 && ix[1] == i1; e++, ix += 4) {
             const double v = d.q_val[e];
-            cplx x = delta(ix[2], ix[3]);
-            q = cadd(q, cscale(cmul(delta(ix[0], ix[1]), x), v));
-            int s0 = d.slot[ix[0]], s1 = d.slot[ix[1]];
-            F[s0 * ni + s1] = cadd(F[s0 * ni + s1], cscale(x, 6.0 * v));
+            const cplx x = delta(ix[2], ix[3]);
+            qs = cadd(qs, cscale(x, v));
+            f = cadd(f, cscale(x, 6.0 * v));
         }
+        q = cadd(q, cmul(delta(i0, i1), qs));
+        F[d.slot[i0] * ni + d.slot[i1]] = f;
+    }
+    q.x = block_sum(q.x, red);
+    q.y = block_sum(q.y, red);
+    if (threadIdx.x == 0) {
         // terms of six or eight Majoranas: energy h_val Pf(Delta_S); Fock entries
         // F_{s_a s_b} = -(1/2) h_val (-1)^(a + b + 1) Pf(Delta_S without a, b) (a < b), antisymmetric
         cplx qh = cmk(0.0, 0.0);

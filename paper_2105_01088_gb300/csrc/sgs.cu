@@ -1460,15 +1460,23 @@ void eom_sums(sgs_ctx* c, Instance& I, cudaStream_t st, int accumulate, int part
                                                                            I.pair_index, tsum, I.dgamma, accumulate);
         counted();
     }
-    if (I.tc_kind >= 0)
-        eom_finish_kernel<float><<<eg, 256, eom_smem<float>(M), st>>>(d, I.si, I.imd, fimp, I.fimp_state, I.s[4],
-                                                                      I.coef, I.pair_index, tsum, I.dgamma,
-                                                                      I.self_mask, part);
-    else
-        eom_finish_kernel<double><<<eg, 256, eom_smem<double>(M), st>>>(d, I.si, I.imd, fimp, I.fimp_state, I.s[4],
-                                                                        I.coef, I.pair_index, tsum, I.dgamma,
-                                                                        I.self_mask, part);
-    counted();
+    if (part & EOM_FINISH_REST) {
+        if (I.tc_kind >= 0)
+            eom_finish_kernel<float><<<eg, 256, eom_smem<float>(M), st>>>(d, I.fimp_state, I.s[4], I.coef, I.pair_index,
+                                                                          tsum, I.dgamma, I.self_mask);
+        else
+            eom_finish_kernel<double><<<eg, 256, eom_smem<double>(M), st>>>(d, I.fimp_state, I.s[4], I.coef,
+                                                                            I.pair_index, tsum, I.dgamma, I.self_mask);
+        counted();
+    }
+    if ((part & EOM_FINISH_PAIRS) && I.nimp > 0 && d.P > 0) {
+        const dim3 ig((n * I.nimp + 7) / 8, M);
+        if (I.tc_kind >= 0)
+            eom_imp_kernel<float><<<ig, 256, 0, st>>>(d, I.si, I.imd, fimp, I.coef, I.pair_index, I.dgamma);
+        else
+            eom_imp_kernel<double><<<ig, 256, 0, st>>>(d, I.si, I.imd, fimp, I.coef, I.pair_index, I.dgamma);
+        counted();
+    }
 }
 
 // the end of the assembly: byte accounting (the assembly kernels store dGamma exactly
@@ -2442,7 +2450,7 @@ sgs_status sgs_variance(sgs_ctx* c, int instance, double* energy, double* varian
     CUDA_TRY(c, pair_pass(c, I, I.Ecur, c->stream));
     c->stage(-1);
     const size_t rows = (size_t)I.P + I.M;
-    const size_t need = rows + 8;
+    const size_t need = rows * (1 + 2 * VAR_SPLIT) + 8;
     if (I.corr_cap < need) {
         c->owner = &I;
         I.corr_scratch = c->alloc<double>(need);
@@ -2452,7 +2460,9 @@ sgs_status sgs_variance(sgs_ctx* c, int instance, double* energy, double* varian
     }
     double* partial = I.corr_scratch;
     double* dout = partial + rows;
-    VarArgs va{I.dev(), I.si, I.imd, I.Gm, I.lam, I.c_idx, I.c_val, I.nc, I.trA2, partial};
+    VarArgs va{I.dev(), I.si, I.imd, I.Gm, I.lam, I.c_idx, I.c_val, I.nc, I.trA2, dout + 8, partial};
+    variance_t2_kernel<<<dim3(VAR_SPLIT, (unsigned)rows), 256, 0, c->stream>>>(va);
+    counted();
     variance_kernel<<<(unsigned)rows, 256, 0, c->stream>>>(va);
     column_sum_kernel<<<1, 32, 0, c->stream>>>(partial, (int)rows, 1, dout);
     counted(); counted();

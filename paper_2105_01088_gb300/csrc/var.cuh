@@ -83,8 +83,47 @@ struct VarArgs {
     const double* c_val;
     int nc;
     double trA2;             // tr(A^2)
+    double* t2;              // [P + M][VAR_SPLIT] complex: shares of tr(A Delta A Delta)
     double* partial;         // [P + M]: Re of the weighted <H^2> of each pair / state
 };
+
+// Shares of t2 = tr(A Delta A Delta) of each pair and state: with X = A Delta, t2 = sum_kl X_kl X_lk, the
+// diagonal once and every k < l twice.  A share takes the rows k of one residue, a warp per row.  Bound by the
+// FP64 pipe (about 18 instructions per entry); one CTA per pair left most SMs idle (1.3 ms at n = 388, M = 10).
+// Grid (VAR_SPLIT, P + M), 256 threads.
+#define VAR_SPLIT 8
+__global__ void __launch_bounds__(256) variance_t2_kernel(VarArgs v) {
+    __shared__ double red[32];
+    const InstDev& d = v.d;
+    const int blk = blockIdx.y, n = d.n, lane = threadIdx.x & 31;
+    const bool diag = blk >= d.P;
+    const double* re = diag ? d.gamma + (size_t)(blk - d.P) * nn(d) : v.si + (size_t)blk * nn(d);
+    const double* im = diag ? nullptr : v.imd + (size_t)blk * nn(d);
+    // row r of A times column c of (re, im)
+    auto ax = [&](int r, int c) -> cplx {
+        cplx x = cmk(0.0, 0.0);
+        for (int p = d.a_rowptr[r]; p < d.a_rowptr[r + 1]; p++) {
+            const double a = d.a_val[p];
+            const size_t o = (size_t)d.a_col[p] * n + c;
+            x.x = fma(a, re[o], x.x);
+            if (!diag) x.y = fma(a, im[o], x.y);
+        }
+        return diag ? x : cmk(-2.0 * x.x, -x.y);
+    };
+    cplx t2 = cmk(0.0, 0.0);
+    for (int k = blockIdx.x + VAR_SPLIT * (threadIdx.x >> 5); k < n; k += 8 * VAR_SPLIT)
+        for (int l = k + lane; l < n; l += 32) {
+            const cplx x = ax(k, l);
+            if (__double_as_longlong(x.x) << 1 == 0 && __double_as_longlong(x.y) << 1 == 0) continue;
+            const cplx y = l == k ? x : ax(l, k), z = cmul(x, y);
+            t2 = cadd(t2, l == k ? z : cscale(z, 2.0));
+        }
+    t2 = block_csum(t2, red);
+    if (threadIdx.x == 0) {
+        v.t2[2 * (blk * VAR_SPLIT + blockIdx.x)] = t2.x;
+        v.t2[2 * (blk * VAR_SPLIT + blockIdx.x) + 1] = t2.y;
+    }
+}
 
 // one CTA per unordered pair (blocks 0..P-1) and per state (P..P+M-1)
 __global__ void __launch_bounds__(256) variance_kernel(VarArgs v) {
@@ -115,18 +154,9 @@ __global__ void __launch_bounds__(256) variance_kernel(VarArgs v) {
     for (int j = tid; j < d.a_nnz; j += nt) T = cadd(T, cscale(D(d.a_col[j], d.a_row[j]), d.a_val[j]));
     T = block_csum(T, red);
 
-    // t2 = tr(A Delta A Delta) = sum_kl (A Delta)_kl (Delta A)_kl,
-    // (Delta A)_kl = -sum_{j in row l} Delta_kj A_lj  (A antisymmetric)
     cplx t2 = cmk(0.0, 0.0);
-    for (size_t e = tid; e < (size_t)n * n; e += nt) {
-        const int k = (int)(e / n), l = (int)(e % n);
-        cplx x = cmk(0.0, 0.0), y = cmk(0.0, 0.0);
-        for (int p = d.a_rowptr[k]; p < d.a_rowptr[k + 1]; p++) x = cadd(x, cscale(D(d.a_col[p], l), d.a_val[p]));
-        if (x.x == 0.0 && x.y == 0.0) continue;
-        for (int p = d.a_rowptr[l]; p < d.a_rowptr[l + 1]; p++) y = csub(y, cscale(D(k, d.a_col[p]), d.a_val[p]));
-        t2 = cadd(t2, cmul(x, y));
-    }
-    t2 = block_csum(t2, red);
+    for (int j = 0; j < VAR_SPLIT; j++)
+        t2 = cadd(t2, cmk(v.t2[2 * (blk * VAR_SPLIT + j)], v.t2[2 * (blk * VAR_SPLIT + j) + 1]));
 
     // B = g^T A g and B' = g A g^T on the Majoranas of the quartic terms
     const int tasks = 2 * ni * ni;
