@@ -120,6 +120,7 @@ struct OzOperand {
     int* expo;                // [chunk][rows_pad] exponent fields
     uint16_t* slices;         // [chunk][OZ_S][rows_pad][kp] bf16 digits (planes)
     int interleave;           // 1: slice i in plane oz_plane(i) (A operands), 0: plane i (B operands)
+    int rb;                   // rows of a block (oz_block_slice_kernel)
 };
 
 
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(256) oz_block_slice_kernel(OzOperand o) {
     if (!oz_active(o.active, o.active_cmp, b)) return;
     const double* x = o.X[b] + o.off;
     const double* x2 = o.X2 ? o.X2[b] + o.off : nullptr;
-    const int kp = o.kp, ts = kp + 1, rb = oz_block_rows(kp), r0 = blockIdx.x * rb;
+    const int kp = o.kp, ts = kp + 1, rb = o.rb, r0 = blockIdx.x * rb;
     const int total = rb * kp;
     if (o.strided) {
         // element idx: k = idx / rb, row idx % rb (rb consecutive doubles of one k)
@@ -235,8 +236,9 @@ __global__ void __launch_bounds__(256) oz_block_slice_kernel(OzOperand o) {
     }
 }
 
-// contiguous rows (K <= 512): one warp per row takes the row into registers, reduces the
+// contiguous rows (K <= 128 S): one warp per row takes the row into registers, reduces the
 // exponent field and writes the digits, four k per lane per step (one pass over the operand)
+template <int S>
 __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
     const int bl = blockIdx.y, b = o.b0 + bl;
     if (!oz_active(o.active, o.active_cmp, b)) return;
@@ -244,21 +246,20 @@ __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
     if (r >= o.rows_pad) return;
     const double* x = o.X[b] + o.off;
     const double* x2 = o.X2 ? o.X2[b] + o.off : nullptr;
-    unsigned long long v[4][4];          // k = 4 lane + 128 s + u, s < 4 (K <= 512)
+    unsigned long long v[S][4];          // k = 4 lane + 128 s + u
     int e = 0;
 #pragma unroll
-    for (int s = 0; s < 4; s++)
+    for (int s = 0; s < S; s++)
 #pragma unroll
         for (int u = 0; u < 4; u++) {
             const int k = 128 * s + 4 * lane + u;
             v[s][u] = (r < o.rows && k < o.k) ? oz_load(o, x, x2, r, k) : 0ull;
             e = max(e, oz_expo_field(v[s][u]));
         }
-#pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, sh));
+    e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0 && r < o.rows) o.expo[(size_t)bl * o.rows_pad + r] = e;
 #pragma unroll
-    for (int s = 0; s < 4; s++) {
+    for (int s = 0; s < S; s++) {
         const int k = 128 * s + 4 * lane;
         if (k < o.kp) oz_store4(o, bl, r, k, v[s], r < o.rows ? e : 0);
     }
@@ -773,16 +774,23 @@ inline bool make_slice_map(CUtensorMap* map, const void* base, int k, int kp, in
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// exponents and slices of one operand, one pass: long contiguous rows a warp per row in
-// registers, the others (strided, or short) a block of rows at a time through shared memory
-inline bool oz_row_pass(const OzOperand& o) { return !o.strided && o.k >= 256 && o.k <= OZ_KC; }
-inline size_t oz_block_smem(int kp) { return (size_t)oz_block_rows(kp) * (kp + 1) * 8; }
-inline void oz_prepare(const OzOperand& o, int bc, cudaStream_t st) {
+// exponents and slices of one operand, one pass: contiguous rows a warp per row in registers, the others
+// (strided, or of a few dozen entries) a block of rows at a time through shared memory, with smaller blocks
+// (down to the 16 rows of a 128-byte line) where there would be fewer than two per SM.  A 244 x 244 operand of
+// 16 states took 13.7 us by blocks of 32 rows.
+inline int oz_sms();
+inline bool oz_row_pass(const OzOperand& o) { return !o.strided && o.k >= 64 && o.k <= OZ_KC; }
+inline size_t oz_block_smem(int rb, int kp) { return (size_t)rb * (kp + 1) * 8; }
+inline void oz_prepare(OzOperand o, int bc, cudaStream_t st) {
     if (oz_row_pass(o)) {
-        oz_row_slice_kernel<<<dim3((o.rows_pad + 7) / 8, bc), 256, 0, st>>>(o);
+        const dim3 grid((o.rows_pad + 7) / 8, bc);
+        if (o.k <= 128) oz_row_slice_kernel<1><<<grid, 256, 0, st>>>(o);
+        else if (o.k <= 256) oz_row_slice_kernel<2><<<grid, 256, 0, st>>>(o);
+        else oz_row_slice_kernel<4><<<grid, 256, 0, st>>>(o);
     } else {
-        const int rb = oz_block_rows(o.kp);
-        oz_block_slice_kernel<<<dim3((o.rows_pad + rb - 1) / rb, bc), 256, oz_block_smem(o.kp), st>>>(o);
+        o.rb = oz_block_rows(o.kp);
+        while (o.rb > 16 && (long long)((o.rows_pad + o.rb - 1) / o.rb) * bc < 2 * oz_sms()) o.rb >>= 1;
+        oz_block_slice_kernel<<<dim3((o.rows_pad + o.rb - 1) / o.rb, bc), 256, oz_block_smem(o.rb, o.kp), st>>>(o);
     }
 }
 
@@ -885,12 +893,12 @@ inline cudaError_t gemm_oz_chunk(const GemmBatch& g, const OzBuf& buf, int* err,
         const int bc = std::min(chunk, g.batch - b0);
         const OzLayout L = oz_layout(g.m, g.n, g.k, buf, bc);
         OzOperand oa{g.A, g.A2, g.sA2, g.offA, g.lda, g.transA ? 1 : 0, g.m, g.k, L.mp, L.kp, b0,
-                     g.active_flag, g.active_cmp, L.ea, L.as, 1};
+                     g.active_flag, g.active_cmp, L.ea, L.as, 1, 0};
         // an antisymmetric B (not transposed): its K-major columns are its rows negated, so the
         // rows are sliced (contiguous, one pass) and alpha changes sign
         const bool b_rows = g.b_antisym && !g.transB;
         OzOperand ob{g.B, g.B2, g.sB2, b_rows ? g.offBr : g.offB, g.ldb, (g.transB || b_rows) ? 0 : 1, g.n, g.k, L.np,
-                     L.kp, b0, g.active_flag, g.active_cmp, L.eb, L.bs, 0};
+                     L.kp, b0, g.active_flag, g.active_cmp, L.eb, L.bs, 0, 0};
         oz_prepare(oa, bc, st);
         oz_prepare(ob, bc, st);
         const cudaError_t e = oz_product(g, L, b0, bc, b_rows, err, st);

@@ -1530,9 +1530,11 @@ cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, double ds, cudaStre
     exp_commutator_kernel<<<dim3(EXP_PARTX, batch), 256, 0, st>>>(I.s[0], I.s[1], n, ds, I.exp_part);
     counted();
     GemmBatch g = gb_basic(n, n, n, I.p_s[1], n, I.p_s[1], n, I.p_s[0], n, batch);
+    g.b_antisym = 1;    // X, as exp_commutator_kernel stores it
     if ((e = gemm(c, I, g, st, 2.0 * n3 * batch)) != cudaSuccess) return e;         // X2
     g = gb_basic(n, n, n, I.p_s[0], n, I.p_s[1], n, I.p_s[2], n, batch);
     g.mode = GEMM_SKEW;                                                            // X3 = X2 X
+    g.b_antisym = 1;
     if ((e = gemm(c, I, g, st, n3 * batch)) != cudaSuccess) return e;
     exp_norm_kernel<<<dim3(EXP_PART3, batch), 256, 0, st>>>(I.s[2], n, I.exp_part);
     exp_scale_kernel<<<dim3(grid_chunks(nn, 1024, 256), batch), 256, 0, st>>>(I.s[1], I.s[0], I.s[2], cf[10], cf[9], n,
@@ -1546,6 +1548,7 @@ cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, double ds, cudaStre
         g.Cin = (const double* const*)I.p_s[0]; g.ldcin = n; g.beta = cf[3 * j + 2];
         g.Cin2 = (const double* const*)I.p_s[1]; g.beta2 = cf[3 * j + 1];
         g.diag = cf[3 * j];
+        g.b_antisym = 1;    // X3 (an antisymmetric product)
         if ((e = gemm(c, I, g, st, 2.0 * n3 * batch)) != cudaSuccess) return e;
         cur = nxt;
     }
@@ -1561,8 +1564,8 @@ cudaError_t exp_products(sgs_ctx* c, Instance& I, int batch, double ds, cudaStre
 
 // Canonical-form renormalisation (App. A, Eq. CM-normal-form with every lambda_j = 1): the polar
 // factor of the matrices in s4 by `iters` Newton-Schulz steps X <- 1.5 X + 0.5 X (X X); the result
-// goes to gamma.
-cudaError_t polar_pass(sgs_ctx* c, Instance& I, int iters, cudaStream_t st, int from = 4) {
+// goes to gamma.  antisym: they are exactly antisymmetric (an antisymmetric product's result).
+cudaError_t polar_pass(sgs_ctx* c, Instance& I, int iters, cudaStream_t st, int from = 4, int antisym = 0) {
     const int n = I.n, M = I.M;
     const size_t nn = (size_t)n * n;
     const double n3 = (double)n * n * n;
@@ -1571,10 +1574,12 @@ cudaError_t polar_pass(sgs_ctx* c, Instance& I, int iters, cudaStream_t st, int 
     double** dst = I.p_gamma;
     for (int it = 0; it < iters; it++) {
         GemmBatch g = gb_basic(n, n, n, src, n, src, n, I.p_s[0], n, M);
+        g.b_antisym = antisym;
         if ((e = gemm(c, I, g, st, n3 * M)) != cudaSuccess) return e;     // X X: symmetric, half counted
         g = gb_basic(n, n, n, src, n, I.p_s[0], n, dst, n, M);
         g.alpha = 0.5; g.Cin = (const double* const*)src; g.ldcin = n; g.beta = 1.5; g.mode = GEMM_SKEW;
         if ((e = gemm(c, I, g, st, n3 * M)) != cudaSuccess) return e;
+        antisym = 1;
         std::swap(src, dst);
     }
     if (src == I.p_s[from]) {  // an even number of iterations ends in the source buffer
@@ -1686,6 +1691,7 @@ cudaError_t update_pass(sgs_ctx* c, Instance& I, cudaStream_t st) {
     c->stage_flops[SGS_STAGE_UPDATE] += (2.0 + 9.0 + 2.0 + 1.0 + 2.0) * n3 * M;
     // Y = Gamma dGamma -> s0 ; R -> p_R
     GemmBatch g = gb_basic(n, n, n, I.p_gamma, n, I.p_dgamma, n, I.p_s[0], n, M);
+    g.b_antisym = 1;    // dGamma, as the assembly stores it
     if ((e = gemm(c, I, g, st, 2.0 * n3 * M)) != cudaSuccess) return e;
     if ((e = exp_products(c, I, M, I.dtau, st)) != cudaSuccess) return e;
     // T = R Gamma -> s0 ; Gamma' = T R^T -> s2
@@ -1696,7 +1702,7 @@ cudaError_t update_pass(sgs_ctx* c, Instance& I, cudaStream_t st) {
     if ((e = gemm(c, I, g, st, n3 * M)) != cudaSuccess) return e;
     // R is orthogonal to rounding, so R Gamma R^T leaves purity only at rounding level, which one
     // Newton-Schulz iteration (error -> 1.5 error^2) removes
-    if ((e = polar_pass(c, I, 1, st, 2)) != cudaSuccess) return e;
+    if ((e = polar_pass(c, I, 1, st, 2, 1)) != cudaSuccess) return e;
     I.steps_since_profile++;
     return cudaGetLastError();
 }
