@@ -46,8 +46,8 @@ struct TmaBatch {
     const float* Cin; long long cin_stride; int ldcin; float beta; float diag;
     float* CT; long long ct_stride; int ldct;
     // optional pass-through: batch b with pass_flag[b] <= pass_cmp skips the product and
-    // copies Cin (C = Cin, CT = Cin^T)
-    const int* pass_flag; int pass_cmp;
+    // copies Cin (C = Cin, CT = Cin^T), or with skip_pass leaves C and CT as they are
+    const int* pass_flag; int pass_cmp; int skip_pass;
 };
 
 template <int KIND> struct TmaCfg {
@@ -85,8 +85,13 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
 }
 
+// Eight warps: thread 0 the producer, thread 32 the MMA issuer, all of them the epilogue (a TMEM lane quarter
+// is shared by two warps, half the columns each).  The epilogue's loops run over the tile's valid rows with
+// four elements per thread in flight; with four warps and one element at a time it was most of a small
+// product's 26 to 37 us.
+#define TMA_THREADS 256
 template <int KIND>
-__global__ void __launch_bounds__(128) gemm_tma_kernel(const __grid_constant__ TmaBatch g) {
+__global__ void __launch_bounds__(TMA_THREADS) gemm_tma_kernel(const __grid_constant__ TmaBatch g) {
     using Cfg = TmaCfg<KIND>;
     using T = typename std::conditional<KIND == TC_BF16, __nv_bfloat16, float>::type;
     constexpr int NST = Cfg::NST, SLAB = Cfg::SLAB, STAGE = Cfg::STAGE, NS = Cfg::NS;
@@ -106,6 +111,8 @@ __global__ void __launch_bounds__(128) gemm_tma_kernel(const __grid_constant__ T
     __syncthreads();
     if (skip) return;
     const int b = blockIdx.y;
+    const bool pass = g.pass_flag && g.pass_flag[b] <= g.pass_cmp;     // uniform in the CTA
+    if (pass && g.skip_pass) return;
     int tm, tn;
     if (g.skew) {
         const int t = blockIdx.x;
@@ -143,7 +150,6 @@ __global__ void __launch_bounds__(128) gemm_tma_kernel(const __grid_constant__ T
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
-    const bool pass = g.pass_flag && g.pass_flag[b] <= g.pass_cmp;     // uniform in the CTA
     const int nk = pass ? 0 : (g.k + KSLAB - 1) / KSLAB;
 
     if (tid == 0) {
@@ -204,19 +210,19 @@ __global__ void __launch_bounds__(128) gemm_tma_kernel(const __grid_constant__ T
         // TMEM (or, passing through, Cin) -> padded shared tile (row stride 129 floats:
         // conflict-free both ways)
         float* tile = reinterpret_cast<float*>(gbase);
-        constexpr int TS = TMA_BN + 1;
-        const int r = warp * 32 + lane;
+        constexpr int TS = TMA_BN + 1, NT = TMA_THREADS;
+        const int r = (warp & 3) * 32 + lane;
+        const int rows = min(TMA_BM, g.m - m0), cols = min(TMA_BN, g.n - n0);
+        const float* Cin = g.Cin ? g.Cin + (size_t)b * g.cin_stride + (size_t)m0 * g.ldcin + n0 : nullptr;
         if (pass) {
-            for (int e = tid; e < TMA_BM * TMA_BN; e += 128) {
+            for (int e = tid; e < rows * TMA_BN; e += NT) {
                 const int rr = e / TMA_BN, cc = e % TMA_BN;
-                const int row = m0 + rr, col = n0 + cc;
-                tile[rr * TS + cc] = (row < g.m && col < g.n)
-                                         ? g.Cin[(size_t)b * g.cin_stride + (size_t)row * g.ldcin + col] : 0.0f;
+                tile[rr * TS + cc] = cc < cols ? Cin[(size_t)rr * g.ldcin + cc] : 0.0f;
             }
         }
-        for (int c0 = 0; c0 < TMA_BN && !pass; c0 += 32) {
+        for (int c0 = (warp >> 2) * (TMA_BN / 2); c0 < (warp >> 2) * (TMA_BN / 2) + TMA_BN / 2 && c0 < cols && !pass; c0 += 32) {
             uint32_t v[32];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + c0;
+            const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                          "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
                          "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -234,45 +240,52 @@ __global__ void __launch_bounds__(128) gemm_tma_kernel(const __grid_constant__ T
         __syncthreads();
         // fp32 epilogue (FP64 arithmetic is slow on this part)
         const float alpha = pass ? 1.0f : (float)g.alpha;
-        const bool extra = !pass && (g.Cin || g.diag != 0.0f);
+        const bool extra = !pass && (Cin || g.diag != 0.0f);
         auto put = [&](int row, int col, float x) {
             if (g.out_f64) static_cast<double*>(g.C)[(size_t)b * g.c_stride + (size_t)row * g.ldc + col] = (double)x;
             else static_cast<float*>(g.C)[(size_t)b * g.c_stride + (size_t)row * g.ldc + col] = x;
         };
-        for (int e = tid; e < TMA_BM * TMA_BN; e += 128) {
-            const int rr = e / TMA_BN, cc = e % TMA_BN;
-            const int row = m0 + rr, col = n0 + cc;
-            if (row >= g.m || col >= g.n) continue;
-            if (!g.skew || tm != tn) {
-                float x = alpha * tile[rr * TS + cc];
-                if (extra) {
-                    if (g.Cin) x += g.beta * g.Cin[(size_t)b * g.cin_stride + (size_t)row * g.ldcin + col];
-                    if (row == col) x += g.diag;
-                    tile[rr * TS + cc] = x;            // kept for the transposed copy
+        for (int e0 = tid; e0 < rows * TMA_BN; e0 += 4 * NT) {
+            float ci[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int e = e0 + u * NT, rr = e / TMA_BN, cc = e % TMA_BN;
+                ci[u] = (extra && Cin && rr < rows && cc < cols) ? Cin[(size_t)rr * g.ldcin + cc] : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int e = e0 + u * NT, rr = e / TMA_BN, cc = e % TMA_BN;
+                const int row = m0 + rr, col = n0 + cc;
+                if (rr >= rows || cc >= cols) continue;
+                if (!g.skew || tm != tn) {
+                    float x = alpha * tile[rr * TS + cc];
+                    if (extra) {
+                        if (Cin) x += g.beta * ci[u];
+                        if (row == col) x += g.diag;
+                        tile[rr * TS + cc] = x;            // kept for the transposed copy
+                    }
+                    put(row, col, x);
+                } else {       // diagonal tile: lower part from the tile, upper part mirrored, zero diagonal
+                    put(row, col, rr > cc ? alpha * tile[rr * TS + cc] : (rr < cc ? -alpha * tile[cc * TS + rr] : 0.0f));
                 }
-                put(row, col, x);
-            } else {       // diagonal tile: lower part from the tile, upper part mirrored, zero diagonal
-                put(row, col, rr > cc ? alpha * tile[rr * TS + cc] : (rr < cc ? -alpha * tile[cc * TS + rr] : 0.0f));
             }
         }
         if (g.CT) {
             // CT[n0 + cc][m0 + rr] = C[m0 + rr][n0 + cc], rows of CT coalesced
             __syncthreads();
             const float a2 = extra ? 1.0f : alpha;
-            for (int e = tid; e < TMA_BM * TMA_BN; e += 128) {
+#pragma unroll 4
+            for (int e = tid; e < cols * TMA_BM; e += NT) {
                 const int cc = e / TMA_BM, rr = e % TMA_BM;
-                const int row = n0 + cc, col = m0 + rr;
-                if (row >= g.n || col >= g.m) continue;
-                g.CT[(size_t)b * g.ct_stride + (size_t)row * g.ldct + col] = a2 * tile[rr * TS + cc];
+                if (rr < rows) g.CT[(size_t)b * g.ct_stride + (size_t)(n0 + cc) * g.ldct + m0 + rr] = a2 * tile[rr * TS + cc];
             }
         }
         if (g.skew && tm != tn) {
             // mirrored block: C[n0 + cc][m0 + rr] = -C[m0 + rr][n0 + cc], rows of the mirror coalesced
-            for (int e = tid; e < TMA_BM * TMA_BN; e += 128) {
+#pragma unroll 4
+            for (int e = tid; e < cols * TMA_BM; e += NT) {
                 const int cc = e / TMA_BM, rr = e % TMA_BM;
-                const int row = n0 + cc, col = m0 + rr;
-                if (row >= g.n || col >= g.m) continue;
-                put(row, col, -alpha * tile[rr * TS + cc]);
+                if (rr < rows) put(n0 + cc, m0 + rr, -alpha * tile[rr * TS + cc]);
             }
         }
     }
@@ -321,7 +334,7 @@ template <int KIND>
 inline cudaError_t gemm_tma_launch(const TmaBatch& g, cudaStream_t st) {
     const int tmn = (g.m + TMA_BM - 1) / TMA_BM, tnn = (g.n + TMA_BN - 1) / TMA_BN;
     const unsigned gx = g.skew ? (unsigned)(tmn * (tmn + 1) / 2) : (unsigned)(tmn * tnn);
-    gemm_tma_kernel<KIND><<<dim3(gx, g.batch), 128, TmaCfg<KIND>::SMEM, st>>>(g);
+    gemm_tma_kernel<KIND><<<dim3(gx, g.batch), TMA_THREADS, TmaCfg<KIND>::SMEM, st>>>(g);
     return cudaGetLastError();
 }
 

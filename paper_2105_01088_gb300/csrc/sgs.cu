@@ -1622,8 +1622,10 @@ cudaError_t update_pass_lp(sgs_ctx* c, Instance& I, cudaStream_t st) {
     counted(); counted();
     // Y = Gamma dGamma (dGamma antisymmetric: its K-major form is -dGamma)
     if ((e = run(lp_product(I, 0, 1, -1.0, I.u_y, n, (long long)nn))) != cudaSuccess) return e;
-    exp_prepare_lp_kernel<<<M, 1024, 0, st>>>(I.u_y, n, ldp, I.dtau, I.u_f32[0], I.u_f32[1], I.sq, I.err);
-    counted();
+    exp_norm_lp_kernel<<<dim3(EXP_PARTX, M), 256, 0, st>>>(I.u_y, n, I.dtau, I.exp_part);
+    exp_prepare_lp_kernel<<<dim3(std::min(lower_tile_count(n), 128), M), 256, 0, st>>>(
+        I.u_y, n, ldp, I.dtau, I.exp_part, I.u_f32[0], I.u_f32[1], I.sq, I.err);
+    counted(); counted();
     split(0, 2);
     split(1, 3);
     // Horner on transposes: Q_j = I + (1/j) Q_{j+1} X_s^T (X_s^T's K-major form is X_s)
@@ -1643,20 +1645,26 @@ cudaError_t update_pass_lp(sgs_ctx* c, Instance& I, cudaStream_t st) {
         split(3, 5);
         split(4, 6);
     }
-    // squarings E^T <- E^T E^T + 2 E^T (K-major form of E^T is E); states that need
-    // fewer pass theirs through
+    // squarings E^T <- E^T E^T + 2 E^T (K-major form of E^T is E), between (3, 4) and (5, 6); a state that
+    // needs fewer is left where its last one wrote it, and lp_select_kernel brings E back to 4
     int et = 3, ee = 4, et2 = 5, ee2 = 6;
     for (int j = 0; j < EXP_MAX_SQUARINGS; j++) {
         TmaBatch t = lp_product(I, 2 + et, 2 + ee, 1.0, I.u_f32[et2], ldp, (long long)np);
         t.Cin = I.u_f32[et]; t.ldcin = ldp; t.cin_stride = (long long)np; t.beta = 2.0f;
         t.CT = I.u_f32[ee2]; t.ldct = ldp; t.ct_stride = (long long)np;
-        t.pass_flag = I.sq; t.pass_cmp = j;
+        t.pass_flag = I.sq; t.pass_cmp = j; t.skip_pass = 1;
         if ((e = run(t)) != cudaSuccess) return e;
-        split(et2, 2 + et2);
-        split(ee2, 2 + ee2);
+        lp_split2_kernel<<<dim3(grid_chunks(2 * np, 1024, 256), M), 256, 0, st>>>(
+            I.u_f32[et2], I.u_hi[2 + et2], I.u_f32[ee2], I.u_hi[2 + ee2], np, kind, I.sq, j);
+        counted();
         std::swap(et, et2);
         std::swap(ee, ee2);
     }
+    static_assert(EXP_MAX_SQUARINGS % 2 == 0, "the last pass ends in (3, 4)");
+    const size_t words = np * (kind == TC_BF16 ? 2 : 4) / 16;          // ldp is a multiple of 8
+    lp_select_kernel<<<dim3(grid_chunks(words, 256, 256), M), 256, 0, st>>>(
+        static_cast<const uint4*>(I.u_hi[8]), static_cast<uint4*>(I.u_hi[6]), words, I.sq);
+    counted();
     // F = E Gamma (Gamma's K-major form is -Gamma), G = F E^T (K-major form E)
     if ((e = run(lp_product(I, 2 + ee, 0, -1.0, I.u_f32[7], ldp, (long long)np))) != cudaSuccess) return e;
     split(7, 9);

@@ -17,43 +17,77 @@
 #pragma once
 #include <cuda_bf16.h>
 #include "common.cuh"
+#include "update.cuh"
 
 namespace sgs {
 
 #define EXP_LP_DEGREE 6        // Taylor degree: ||X_s|| <= 1/8 truncates below 1e-10 relative
 #define LP_NS_ITERS 3          // purity drift ~1e-3 ||E|| reaches rounding in three Newton-Schulz steps
 
-// X_s = 2^-s (ds/4)(Y - Y^T) with ||X_s||_F <= 1/8 and Q_d = I - X_s / d, one CTA per
-// state; Y: [M][n][n] fp32; X_s, Q: [M][n][ldp] fp32 with zero padding columns.
-__global__ void __launch_bounds__(1024) exp_prepare_lp_kernel(const float* Y, int n, int ldp, double ds, float* Xs,
-                                                               float* Q, int* sq, int* err) {
+// Partial sums of ||X||_F^2 of X = (ds/4)(Y - Y^T) (Y: [M][n][n] fp32), both entries of a pair from tiles
+// K >= L staged through shared memory.  Grid (EXP_PARTX, states), 256 threads.
+__global__ void __launch_bounds__(256) exp_norm_lp_kernel(const float* Y, int n, double ds, double* part) {
+    __shared__ float t[32][33];
     __shared__ double red[32];
-    const int mu = blockIdx.x;
+    const int mu = blockIdx.y, tiles = lower_tile_count(n), tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const float* y = Y + (size_t)mu * n * n;
     double ss = 0.0;
-    for (size_t e = threadIdx.x; e < (size_t)n * n; e += blockDim.x) {
-        const int k = (int)(e / n), l = (int)(e % n);
-        const double v = 0.25 * ds * ((double)y[e] - (double)y[(size_t)l * n + k]);
-        ss += v * v;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        int K, L;
+        lower_tile(tile, K, L);
+        const int k0 = K * 32, l0 = L * 32;
+        for (int j = ty; j < 32; j += 8)
+            t[j][tx] = (l0 + j < n && k0 + tx < n) ? y[(size_t)(l0 + j) * n + k0 + tx] : 0.0f;
+        __syncthreads();
+        for (int j = ty; j < 32; j += 8) {
+            const int k = k0 + j, l = l0 + tx;
+            if (k >= n || l >= n || k <= l) continue;
+            const double v = 0.25 * ds * ((double)y[(size_t)k * n + l] - (double)t[tx][j]);
+            ss = fma(2.0 * v, v, ss);
+        }
+        __syncthreads();
     }
     ss = block_sum(ss, red);
-    const double nrm = sqrt(ss);
+    if (threadIdx.x == 0) part[(size_t)mu * EXP_PARTS + blockIdx.x] = ss;
+}
+
+// X_s = 2^-s (ds/4)(Y - Y^T) with ||X_s||_F <= 1/8 and Q_d = I - X_s / d; X_s, Q: [M][n][ldp] fp32, whose
+// padding columns are zero already.  Grid (CTAs, states), 256 threads.
+__global__ void __launch_bounds__(256) exp_prepare_lp_kernel(const float* Y, int n, int ldp, double ds,
+                                                             const double* part, float* Xs, float* Q, int* sq, int* err) {
+    __shared__ float a[32][33], t[32][33];
+    __shared__ double red[32];
+    const int mu = blockIdx.y, tiles = lower_tile_count(n), tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const double nrm = sqrt(block_sum(threadIdx.x < EXP_PARTX ? part[(size_t)mu * EXP_PARTS + threadIdx.x] : 0.0, red));
     int s = 0;
     while (nrm * ldexp(1.0, -s) > EXP_THETA && s < 64) s++;
     if (s > EXP_MAX_SQUARINGS) {
-        if (threadIdx.x == 0) atomicOr(err, SGS_DEV_EXPNORM);
+        if (threadIdx.x == 0 && blockIdx.x == 0) atomicOr(err, SGS_DEV_EXPNORM);
         s = EXP_MAX_SQUARINGS;
     }
-    if (threadIdx.x == 0) sq[mu] = s;
+    if (threadIdx.x == 0 && blockIdx.x == 0) sq[mu] = s;
     const float sc = (float)(0.25 * ds * ldexp(1.0, -s));
+    const float* y = Y + (size_t)mu * n * n;
     float* xs = Xs + (size_t)mu * n * ldp;
     float* q = Q + (size_t)mu * n * ldp;
-    for (size_t e = threadIdx.x; e < (size_t)n * ldp; e += blockDim.x) {
-        const int k = (int)(e / ldp), l = (int)(e % ldp);
-        float v = 0.0f;
-        if (l < n) v = sc * (y[(size_t)k * n + l] - y[(size_t)l * n + k]);
-        xs[e] = v;
-        q[e] = (k == l ? 1.0f : 0.0f) - v * (1.0f / EXP_LP_DEGREE);
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        int K, L;
+        lower_tile(tile, K, L);
+        const int k0 = K * 32, l0 = L * 32;
+        for (int j = ty; j < 32; j += 8) {
+            a[j][tx] = (k0 + j < n && l0 + tx < n) ? y[(size_t)(k0 + j) * n + l0 + tx] : 0.0f;
+            t[j][tx] = (l0 + j < n && k0 + tx < n) ? y[(size_t)(l0 + j) * n + k0 + tx] : 0.0f;
+        }
+        __syncthreads();
+        for (int j = ty; j < 32; j += 8)
+            for (int side = 0; side < (K == L ? 1 : 2); side++) {         // tile (K, L), and (L, K)
+                const int k = (side ? l0 : k0) + j, l = (side ? k0 : l0) + tx;
+                if (k >= n || l >= n) continue;
+                const float v = sc * (side ? t[j][tx] - a[tx][j] : a[j][tx] - t[tx][j]);
+                xs[(size_t)k * ldp + l] = v;
+                q[(size_t)k * ldp + l] = (k == l ? 1.0f : 0.0f) - v * (1.0f / EXP_LP_DEGREE);
+            }
+        __syncthreads();
     }
 }
 
@@ -72,6 +106,31 @@ __global__ void lp_split_kernel(const float* src, void* hi, void* lo, size_t cou
             static_cast<float*>(lo)[e] = x - h;
         }
     }
+}
+
+// the same for two arrays of [M][count] whose state's flag is above cmp (the states a squaring has changed);
+// grid (CTAs, M)
+__global__ void lp_split2_kernel(const float* src0, void* hi0, const float* src1, void* hi1, size_t count, int kind,
+                                 const int* flag, int cmp) {
+    if (flag[blockIdx.y] <= cmp) return;
+    const size_t off = blockIdx.y * count;
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < 2 * count; e += (size_t)gridDim.x * blockDim.x) {
+        const bool second = e >= count;
+        const size_t o = off + (second ? e - count : e);
+        const float x = (second ? src1 : src0)[o];
+        void* hi = second ? hi1 : hi0;
+        if (kind == 1) static_cast<__nv_bfloat16*>(hi)[o] = __float2bfloat16_rn(x);
+        else static_cast<float*>(hi)[o] = round_tf32(x);
+    }
+}
+
+// the operand copies [M][bytes] of states with an odd flag from odd to even (the buffer a state's last
+// squaring wrote); grid (CTAs, M)
+__global__ void lp_select_kernel(const uint4* odd, uint4* even, size_t words, const int* flag) {
+    if ((flag[blockIdx.y] & 1) == 0) return;
+    const size_t off = blockIdx.y * words;
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (size_t)gridDim.x * blockDim.x)
+        even[off + e] = odd[off + e];
 }
 
 // FP64 [M][n][n] -> operand [M][n][ldp]: kind 0 tf32 (rounded), 1 bf16, 2 tf32 split (hi, lo)
