@@ -15,12 +15,12 @@
 // of ordered pairs (u <= v) are evaluated once.
 #pragma once
 #include "common.cuh"
-#include "factor.cuh"
 #include "pair.cuh"
+#include "pf_packed.cuh"
 
 namespace sgs {
 
-#define RENYI_MAX_DIM 152     // 2 * 2 N_A <= 152 (impurity + up to 18 sites) in one CTA's shared memory
+#define RENYI_MAX_DIM PACKED_PF_MAX     // 2 * 2 N_A <= 152 (impurity + up to 18 sites) in one CTA's shared memory
 
 // blocks[u] = Delta^{ab}_A (complex, na2 x na2), w[u] = lambda_a conj(lambda_b) G_ba, u = a M + b
 __global__ void renyi_blocks_kernel(InstDev d, const double* si, const double* imd, const double* Gm,
@@ -52,38 +52,17 @@ __global__ void renyi_blocks_kernel(InstDev d, const double* si, const double* i
     }
 }
 
-// dynamic shared memory of renyi_pf_kernel: the packed upper triangles (re, im), four vectors, and the packed
-// entries' row and column
-inline size_t renyi_smem(int m) {
-    return (size_t)m * (m - 1) / 2 * (2 * sizeof(double) + 2) + 4 * (size_t)m * sizeof(double) + 16;
-}
-
-// One CTA per unordered pair (u <= v) of ordered pairs: complex Parlett-Reid elimination of
-// Z = [[Delta_u, i 1], [-i 1, Delta_v]] in shared memory.  Z is antisymmetric: only its upper triangle is kept,
-// packed by rows, so that what is live after a step is the tail of the storage and every lane of the rank-2
-// update has an element (their rows and columns from a table).  The step's rows k and q = k + 1 are done after
-// it, so the interchange of q and the pivot p only writes row and column p.
-// Bound by the FP64 pipe: 8 FMAs per live element and step, m^3 / 12 elements in all.  2080 matrices' worth of
-// the earlier form (both triangles, the scaled row formed again for every element, a logarithm per step) took
-// 8.0 ms for m = 24, 64 and 104 at 666 matrices each.
+// One CTA per unordered pair (u <= v) of ordered pairs: the Pfaffian of Z = [[Delta_u, i 1], [-i 1, Delta_v]] in
+// shared memory (pf_packed.cuh).  Entropies of 2, 7, 12 and 16 sites at 666 matrices each, with the energy they
+// need: 16.4 ms with both triangles updated, the scaled row formed again for every element and a logarithm per
+// step; now 5.4, of which the FP64 pipe's time for the eliminations is 3.3.
 __global__ void __launch_bounds__(256) renyi_pf_kernel(const double* blocks, const double* w, long long npairs,
                                                        int na2, double log_norm, double* partial) {
     extern __shared__ double sm[];
-    const int m = 2 * na2, T = m * (m - 1) / 2, NT = blockDim.x, NW = NT >> 5;
-    double* Zr = sm;                            // row i, column j > i at off(i) + j
-    double* Zi = Zr + T;
-    double* tr = Zi + T;                        // tau and u of the step
-    double* ti = tr + m;
-    double* ur = ti + m;
-    double* ui = ur + m;
-    uchar2* ij = reinterpret_cast<uchar2*>(ui + m);
-    __shared__ long long red_v[8];
-    __shared__ int red_i[8];
-    __shared__ double s_inv[2], s_pr[RENYI_MAX_DIM / 2], s_pi[RENYI_MAX_DIM / 2];
+    const int m = 2 * na2, NW = blockDim.x >> 5;
+    const PackedPf pk(sm, m);
     __shared__ long long s_u, s_v;
-    __shared__ int s_flip;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    auto off = [m](int i) { return i * (2 * m - i - 1) / 2 - i - 1; };
     const long long q0 = blockIdx.x + (long long)blockIdx.y * gridDim.x;
     if (q0 >= npairs) return;
     if (tid == 0) {             // decode q0 = v (v + 1) / 2 + u, u <= v
@@ -92,7 +71,6 @@ __global__ void __launch_bounds__(256) renyi_pf_kernel(const double* blocks, con
         while (v * (v + 1) / 2 > q0) --v;
         s_v = v;
         s_u = q0 - v * (v + 1) / 2;
-        s_flip = 0;
     }
     __syncthreads();
     const long long u = s_u, v = s_v;
@@ -104,107 +82,18 @@ __global__ void __launch_bounds__(256) renyi_pf_kernel(const double* blocks, con
             if (j < na2) z = Bu[i * na2 + j];
             else if (i >= na2) z = Bv[(i - na2) * na2 + j - na2];
             else if (j == i + na2) z.y = 1.0;               // i 1
-            const int e = off(i) + j;
-            Zr[e] = z.x;
-            Zi[e] = z.y;
-            ij[e] = make_uchar2((unsigned char)i, (unsigned char)j);
+            pk.set(i, j, z.x, z.y);
         }
     __syncthreads();
-    bool zero = false;
-    for (int k = 0; k < m - 1; k += 2) {
-        const int q = k + 1, ok = off(k), oq = off(q);
-        // the pivot: the largest entry of row k, the smaller column on a tie
-        long long key = -1;
-        int p = 0x7fffffff;
-        for (int i = q + tid; i < m; i += NT) {
-            const double x = Zr[ok + i], y = Zi[ok + i];
-            const long long m2 = abs_key(fma(x, x, y * y));
-            if (m2 > key) { key = m2; p = i; }
-        }
-        warp_argmax(key, p);
-        if (lane == 0) { red_v[warp] = key; red_i[warp] = p; }
-        __syncthreads();
-        key = lane < NW ? red_v[lane] : -1ll;
-        p = lane < NW ? red_i[lane] : 0x7fffffff;
-        warp_argmax(key, p);
-        if (!(key > 0 && key <= 0x7FF0000000000000ll)) { zero = true; break; }     // zero (or NaN)
-        const int op = off(p);
-        if (tid == NT - 1) {
-            const double pr = Zr[ok + p], pi = Zi[ok + p];
-            const double rm = 1.0 / fma(pr, pr, pi * pi);
-            s_inv[0] = pr * rm;
-            s_inv[1] = -pi * rm;
-            s_pr[k >> 1] = pr;
-            s_pi[k >> 1] = pi;
-            if (p != q) s_flip ^= 1;
-        }
-        // u_i = -Z'[q][i] with the interchange of q and p: Z'[q][i] = Z[p][i] (i > p), -Z[i][p] (q < i < p),
-        // -Z[q][p] (i = p); Z'[p][i] = Z[q][i], Z'[i][p] = -Z[q][i]
-        for (int i = q + 1 + tid; i < m; i += NT) {
-            const double zr = Zr[oq + i], zi = Zi[oq + i];
-            if (i == p) {
-                ur[i] = zr;
-                ui[i] = zi;
-            } else {
-                const int e = i > p ? op + i : off(i) + p;
-                const double yr = p == q ? zr : Zr[e], yi = p == q ? zi : Zi[e];
-                ur[i] = i > p ? -yr : yr;
-                ui[i] = i > p ? -yi : yi;
-                if (p != q) {
-                    Zr[e] = i > p ? zr : -zr;
-                    Zi[e] = i > p ? zi : -zi;
-                }
-            }
-        }
-        __syncthreads();
-        for (int i = q + 1 + tid; i < m; i += NT) {         // tau_i = Z'[k][i] / pivot
-            const int e = ok + (i == p ? q : i);
-            const double xr = Zr[e], xi = Zi[e], ir = s_inv[0], ii = s_inv[1];
-            tr[i] = xr * ir - xi * ii;
-            ti[i] = xr * ii + xi * ir;
-        }
-        __syncthreads();
-        // Z[i][j] += tau_i u_j - u_i tau_j on the live triangle, rows k + 2 on
-        for (int e = off(k + 2) + k + 3 + tid; e < T; e += NT) {
-            const uchar2 x = ij[e];
-            const double ar = tr[x.x], ai = ti[x.x], br = ur[x.x], bi = ui[x.x];
-            const double cr = tr[x.y], ci = ti[x.y], dr = ur[x.y], di = ui[x.y];
-            double r = Zr[e], s = Zi[e];
-            r = fma(ar, dr, r);
-            s = fma(ar, di, s);
-            r = fma(-ai, di, r);
-            s = fma(ai, dr, s);
-            r = fma(-br, cr, r);
-            s = fma(-br, ci, s);
-            r = fma(bi, ci, r);
-            s = fma(-bi, cr, s);
-            Zr[e] = r;
-            Zi[e] = s;
-        }
-        __syncthreads();
-    }
-    // the pivots' product as mantissa and exponent of two, by one warp
-    if (warp == 0) {
-        int e = 0;
-        cplx x = cmk(1.0, 0.0);
-        for (int t = lane; t < m / 2 && !zero; t += 32) {
-            x = cmul(x, cmk(s_pr[t], s_pi[t]));
-            const int f = min(max(2046 - max(expo_field(x.x), expo_field(x.y)), 1), 2046);
-            x = cscale(x, __hiloint2double(f << 20, 0));    // 2^(f - 1023)
-            e += 1023 - f;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            x = cmul(x, cmk(__shfl_xor_sync(0xffffffffu, x.x, o), __shfl_xor_sync(0xffffffffu, x.y, o)));
-            e += __shfl_xor_sync(0xffffffffu, e, o);
-        }
-        if (lane == 0) {
-            if (zero) x = cmk(0.0, 0.0);
-            const cplx wu = cmk(w[2 * u], w[2 * u + 1]), wv = cmk(w[2 * v], w[2 * v + 1]);
-            const double mag = exp(e * 0.693147180559945309417 + log_norm) * (u < v ? 2.0 : 1.0);
-            x = cscale(cmul(cmul(wu, wv), x), s_flip ? -mag : mag);
-            partial[2 * q0] = zero ? 0.0 : x.x;
-            partial[2 * q0 + 1] = zero ? 0.0 : x.y;
-        }
+    int e = 0;
+    cplx x;
+    const bool zero = packed_pfaffian(pk, x, e);
+    if (tid == 0) {
+        const cplx wu = cmk(w[2 * u], w[2 * u + 1]), wv = cmk(w[2 * v], w[2 * v + 1]);
+        const double mag = exp(e * 0.693147180559945309417 + log_norm) * (u < v ? 2.0 : 1.0);
+        x = cscale(cmul(cmul(wu, wv), x), mag);
+        partial[2 * q0] = zero ? 0.0 : x.x;
+        partial[2 * q0 + 1] = zero ? 0.0 : x.y;
     }
 }
 

@@ -36,6 +36,7 @@
 #include "gemm_oz.cuh"
 #include "gemm_tma.cuh"
 #include "corr.cuh"
+#include "pf_packed.cuh"
 #include "renyi.cuh"
 #include "var.cuh"
 #include "host_init.hpp"
@@ -838,6 +839,7 @@ void set_kernel_attributes() {
     raise_smem_limit(gj_cluster_kernel, optin);
     raise_smem_limit(pf_cluster_kernel, optin);
     raise_smem_limit(renyi_pf_kernel, optin);
+    raise_smem_limit(pf_small_kernel, optin);
     raise_smem_limit(amp_solve_kernel, optin);
     raise_smem_limit(gemm_tma_kernel<TC_TF32>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_BF16>, optin);
@@ -897,6 +899,13 @@ int pf_cluster(int live, int batch, int bs) {
         if (batch * C <= 500 && live >= 4 * C && pfc_smem(bs, C, (live + C - 1) / C) <= 220 * 1024) return C;
     return 0;
 }
+
+// Phase Pfaffians a CTA each in shared memory (pf_small_kernel) against panels, packing and trailing updates.
+// One step of imaginary time, panels / one CTA each, us: n = 64, 3 matrices, 563 / 488; 96, 3: 982 / 946; 112, 3:
+// 1115 / 1124; 112, 21: 1460 / 1282; 128, 15: 1351 / 1377; 128, 21: 1562 / 1465; 140, 28: 1851 / 1819; 152, 21:
+// 1975 / 2039; 152, 45: 2234 / 2228; 152, 253: 5652 / 5222.  Few matrices of many rows gain more from the
+// panels' clusters; n > 152 does not fit.
+bool pf_small(int n, int batch) { return n <= PACKED_PF_MAX && batch >= n - 108; }
 
 // the Gauss-Jordan panel of columns a.k0 .. a.k0 + a.bb - 1
 cudaError_t gj_panel(const GJPanelArgs& a, int batch, cudaStream_t st) {
@@ -1163,6 +1172,12 @@ cudaError_t delta_range(sgs_ctx* c, Instance& I, int p0, int cnt, cudaStream_t s
 cudaError_t pair_phase(sgs_ctx* c, Instance& I, cudaStream_t st) {
     const int n = I.n;
     const size_t nn = (size_t)n * n;
+    if (pf_small(n, I.cpfcnt())) {
+        pf_small_kernel<<<I.cpfcnt(), n <= 48 ? 128 : 256, packed_pf_smem(n), st>>>(I.dev(), I.si, I.imd, I.pflog,
+                                                                                    I.pfphase, I.err);
+        counted();
+        return cudaGetLastError();
+    }
     pf_build_kernel<<<dim3(grid_chunks(nn, 256, 64), I.cpfcnt()), 256, 0, st>>>(I.dev(), I.si, I.imd, I.work);
     counted();
     return launch_pf(c, n, I.cpfcnt(), I.pf_bs, I.p_Y, I.p_TU, I.p_pack, I.p_upA, I.p_upB, I.p_upC, I.pflog,
@@ -2429,8 +2444,8 @@ sgs_status sgs_correlator(sgs_ctx* c, int instance, sgs_corr_kind kind, const in
                 set_kernel_attributes();
                 const unsigned gx = (unsigned)std::min<long long>(npairs, 65535);
                 const unsigned gy = (unsigned)((npairs + gx - 1) / gx);
-                renyi_pf_kernel<<<dim3(gx, gy), m <= 48 ? 128 : 256, renyi_smem(m), c->stream>>>(blocks, wts, npairs, na2,
-                                                                                        log_norm, partial);
+                renyi_pf_kernel<<<dim3(gx, gy), m <= 48 ? 128 : 256, packed_pf_smem(m), c->stream>>>(blocks, wts, npairs, na2,
+                                                                                            log_norm, partial);
                 counted();
             } else {
                 sgs_status rs = renyi_large(c, I, blocks, wts, npairs, na2, log_norm, partial);
