@@ -41,26 +41,28 @@
 // over each (a warp per row where the operand's K rows are contiguous and long,
 // else a block of whole rows at a time through shared memory), then the product
 // kernel.  It takes 128 x 32 output tiles with CTAs of 10 warps (256 TMEM
-// columns, 97 KB of shared memory), two to an SM, each running over every
-// (2 x SMs)-th tile, so that CTAs side by side work on tiles side by side and share
-// their slices in L2 (consecutive tiles per CTA read them from DRAM: 1.5 to 2.3 ms
-// where this order takes 0.86).  In the kernel:
+// columns, 97 KB of shared memory), two to an SM, or, for K >= 256, 128 x 64 tiles with
+// one CTA of 18 warps an SM (all of its TMEM, 225 KB), which load 3/5 of the bytes per
+// output.  Each CTA runs over every (grid)-th tile, so that CTAs side by side work on
+// tiles side by side and share their slices in L2 (consecutive tiles per CTA read them
+// from DRAM: 1.5 to 2.3 ms where this order took 0.86).  In the kernel:
 //   * one producer lane loads, per 64-element K slab, the eight B slices as one
 //     TMA box and the A slices in pairs (one 32 KB box per pair of
 //     adjacent planes) through a ring, 128-byte swizzle, zero fill beyond K;
-//     the B buffer is reloaded once the previous slab's MMAs have released it, and
+//     a B buffer is reloaded once its slab's MMAs have released it, and
 //     the next tile's first slabs load during this tile's epilogue;
-//   * one MMA lane issues, per A slice and K16 step, one MMA of N up to 256
-//     covering all the products of that slice (the B slices and the groups they
-//     feed are adjacent) into the eight accumulators;
+//   * one warp issues, per A slice and K16 step, one MMA of N up to 256 (wide tiles:
+//     two above that) covering all the products of that slice (the B slices and the
+//     groups they feed are adjacent) into the eight accumulators;
 //   * the epilogue warps read the tile's Cin terms while the MMAs run, drain TMEM,
 //     combine, and write the output from their registers; the next tile's MMAs start
-//     when TMEM is drained.
-// One tile per CTA (set-up, first loads and last stores all exposed: 2 + 0.8 us of a
-// K = 64 tile's 12.6) took 13.4 us for the SM's two tiles at K = 64, 11.7 at K = 16 and
-// 36.2 at K = 512; now 11.8, 9.0 and 34.0.  What bounds it: at K = 512 the MMAs, 26 of
-// the 34 us (below N = 180 an MMA takes about 90 clocks whatever its N: 790 clocks per
-// K16 step and tile against 576 at full rate; with the loads left out it takes 29); at
+//     when TMEM is drained (wide tiles: when the exact sums are in registers, before
+//     they are rounded and stored).
+// Per 128 x 64 outputs of an SM, K = 16 / 64 / 256 / 512: one tile per CTA (set-up, first
+// loads and last stores exposed) 11.7, 13.4, - and 36.2 us; CTAs over many tiles 9.0,
+// 11.8, 20.3 and 34.1; MMAs issued by a converged warp 17.6 and 30.8; wide tiles 15.7
+// and 25.8.  What bounds it: wide tiles at K = 512 the MMAs, 40000 clocks of 46000 (36900 at
+// full rate; the drain takes 5500); narrow tiles at K = 512 the loads (25.2 without them); at
 // small K the integer work of the combination, about 150 instructions per output.
 // Every mbarrier wait is bounded; on a timeout the launch records
 // SGS_DEV_TC_TIMEOUT in the error word, waits (bounded) for its loads and MMAs
@@ -84,17 +86,18 @@ namespace sgs {
 #define OZ_SLAB_A (OZ_BM * 128)
 
 // Kernel shapes: BN output columns per tile (TMEM: 8 BN columns), EPIW epilogue warps, RING A-ring depth
-// (units).  Both forms fit two CTAs per SM.  A 128 x 64 tile takes all of an SM's TMEM and shared memory;
+// (units), BBUF B buffers, CTAS CTAs per SM.  A 128 x 64 tile takes all of an SM's TMEM and shared memory;
 // with its epilogue serialised after the main loop it measured about half the throughput at K = 512.
-template <int BN, int EPIW, int RING> struct OzCfg {
+template <int BN, int EPIW, int RING, int BBUF, int CTAS> struct OzCfg {
     static constexpr int SLAB_B = BN * 128;
-    static constexpr int SMEM = OZ_S * SLAB_B + RING * OZ_UNIT * OZ_SLAB_A + 1024;
+    static constexpr int SMEM = BBUF * OZ_S * SLAB_B + RING * OZ_UNIT * OZ_SLAB_A + 1024;
     static constexpr int THREADS = 32 * (EPIW + 2);
 };
-#define OZ_NARROW 32, 8, 2
+#define OZ_WIDE 64, 16, 3, 2, 1
+#define OZ_NARROW 32, 8, 2, 1, 2
 // 128 x 16 tiles for products of at most 16 output columns (the Gauss-Jordan leaf updates):
 // half the epilogue of a 128 x 32 tile whose other half would be discarded
-#define OZ_NARROW16 16, 8, 2
+#define OZ_NARROW16 16, 8, 2, 1, 2
 
 // device scratch of one owner (an instance, or a temporary context): slices and
 // exponent fields of one batch chunk
@@ -304,7 +307,6 @@ __device__ __forceinline__ void oz_combine(const uint32_t (&u)[OZ_G][4], int j, 
     H = hi + (lo >> 28);
     L = (unsigned)lo & 0xFFFFFFFu;
 }
-
 // The bit pattern of (-1)^neg V 2^e as a double, V = H 2^28 + L (|H| < 2^47, 0 <= L < 2^28), rounded once to
 // 53 bits (to nearest, ties to even) in integer arithmetic: |V| = Hm 2^28 + Lm is
 // left-justified into one 64-bit word N (bits shifted out are kept as a sticky flag), N is
@@ -392,17 +394,18 @@ __device__ __forceinline__ void oz_tile(const GemmBatch& g, int x, int& m0, int&
     n0 = tn * BN;
 }
 
-template <int BN, int EPIW, int RING>
-__global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __grid_constant__ OzGemm p) {
+template <int BN, int EPIW, int RING, int BBUF, int CTAS>
+__global__ void __launch_bounds__(32 * (EPIW + 2), CTAS) oz_gemm_kernel(const __grid_constant__ OzGemm p) {
     constexpr int SLAB_B = BN * 128, NU = OZ_S / OZ_UNIT;
+    constexpr bool HOLD = CTAS == 1;             // a tile's sums are taken to registers before they are rounded
     constexpr uint32_t TCOLS = 8u * BN;          // TMEM columns: eight groups of BN
     extern __shared__ uint8_t oz_smem_raw[];
-    __shared__ uint64_t bfull, bempty, afull[RING], aempty[RING], tfull, tempty, done;
+    __shared__ uint64_t bfull[BBUF], bempty[BBUF], afull[RING], aempty[RING], tfull, tempty, done;
     __shared__ uint32_t tmem_base;
     __shared__ int skip, abort_flag;
 
     const GemmBatch& g = p.g;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int t0 = blockIdx.x, t1 = p.total, dt = gridDim.x;
     // tile t's batch entry, whether it computes, and (inactive entries left alone) whether it does anything
     auto entry = [&](int t) { return p.b0 + t / p.tiles; };
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __gri
 
     const uint32_t raw = smem_u32(oz_smem_raw);
     const uint32_t sbase = (raw + 1023u) & ~1023u;
-    auto sA = [&](int slot) { return sbase + (uint32_t)OZ_S * SLAB_B + (uint32_t)slot * (OZ_UNIT * OZ_SLAB_A); };
+    auto sA = [&](int slot) { return sbase + (uint32_t)BBUF * OZ_S * SLAB_B + (uint32_t)slot * (OZ_UNIT * OZ_SLAB_A); };
 
     if (warp == EPIW + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -430,8 +433,10 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __gri
         auto init = [](uint64_t& bar, int count) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&bar)), "r"(count));
         };
-        init(bfull, 1);
-        init(bempty, 1);
+        for (int s = 0; s < BBUF; s++) {
+            init(bfull[s], 1);
+            init(bempty[s], 1);
+        }
         for (int s = 0; s < RING; s++) {
             init(afull[s], 1);
             init(aempty[s], 1);
@@ -462,9 +467,13 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __gri
                 int m0, n0;
                 oz_tile<BN>(g, t - bl * p.tiles, m0, n0);
                 for (int s = 0; s < nslab && ok; s++) {
-                    if (nb > 0 && !mbar_wait_or_abort(smem_u32(&bempty), (uint32_t)((nb - 1) & 1), p.err)) { ok = false; break; }
-                    mbar_expect_tx(smem_u32(&bfull), (uint32_t)(OZ_S * SLAB_B));
-                    oz_tma_load(sbase, &p.tb, s * OZ_KS, n0, bl * OZ_S, smem_u32(&bfull));
+                    const int bb = nb % BBUF;
+                    if (nb >= BBUF && !mbar_wait_or_abort(smem_u32(&bempty[bb]), (uint32_t)((nb / BBUF - 1) & 1), p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_expect_tx(smem_u32(&bfull[bb]), (uint32_t)(OZ_S * SLAB_B));
+                    oz_tma_load(sbase + (uint32_t)(bb * OZ_S * SLAB_B), &p.tb, s * OZ_KS, n0, bl * OZ_S, smem_u32(&bfull[bb]));
                     nb++;
                     for (int u = 0; u < NU; u++) {
                         const int slot = q % RING;
@@ -482,78 +491,74 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __gri
             }
             if (!ok) abort_flag = 1;
             // every load issued has landed before the CTA can leave
-            if (nb > 0) mbar_wait(smem_u32(&bfull), (uint32_t)((nb - 1) & 1), p.err);
+            for (int x = (nb > BBUF ? nb - BBUF : 0); x < nb; x++)
+                mbar_wait(smem_u32(&bfull[x % BBUF]), (uint32_t)((x / BBUF) & 1), p.err);
             for (int x = (q > RING ? q - RING : 0); x < q; x++)
                 mbar_wait(smem_u32(&afull[x % RING]), (uint32_t)((x / RING) & 1), p.err);
         }
     } else if (warp == EPIW + 1) {
-        if (lane == 0) {            // MMA issuer
-            constexpr int MAXB = 256 / BN;             // B slices per MMA (N <= 256)
-            // descriptors of slot 0 / slice 0; other slots and slices offset the 16-byte address field
-            const uint64_t dA0 = tma_smem_desc(sA(0)), dB0 = tma_smem_desc(sbase);
-            auto commit = [](uint64_t& bar) {
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(smem_u32(&bar)) : "memory");
-            };
-            int nb = 0, q = 0, nt = 0;                 // slabs, units and tiles taken
-            bool ok = true;
-            for (int t = t0; t < t1 && ok; t += dt) {
-                if (!is_active(t)) continue;
-                // the accumulators have been drained
-                if (nt > 0 && !mbar_wait_or_abort(smem_u32(&tempty), (uint32_t)((nt - 1) & 1), p.err)) { ok = false; break; }
-                nt++;
-                for (int s = 0; s < nslab && ok; s++, nb++) {
-                    if (!mbar_wait_or_abort(smem_u32(&bfull), (uint32_t)(nb & 1), p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    const int kv = min(OZ_KS, g.k - s * OZ_KS);
-                    const int nk16 = (kv + 15) / 16;
-                    for (int u = 0; u < NU; u++, q++) {
-                        const int slot = q % RING;
-                        if (!mbar_wait_or_abort(smem_u32(&afull[slot]), (uint32_t)((q / RING) & 1), p.err)) {
-                            ok = false;
-                            break;
+        // MMA issuer: the whole warp runs the loop converged and one lane issues.  Issued behind a branch on the
+        // lane an MMA took 177 clocks (its operands moved to uniform registers one by one), more than the 144 its
+        // tensor work averages for the two CTAs of an SM.
+        constexpr int MAXB = 256 / BN;             // B slices per MMA (N <= 256)
+        const uint32_t el = tc_elect(), tm = __shfl_sync(0xffffffffu, tmem, 0);
+        // descriptors of slot 0 / slice 0; other slots and slices offset the 16-byte address field
+        const uint64_t dA0 = tma_smem_desc(sA(0)), dB0 = tma_smem_desc(sbase);
+        auto wait = [&](uint64_t& bar, int phase) {
+            return __all_sync(0xffffffffu, mbar_wait_or_abort(smem_u32(&bar), (uint32_t)(phase & 1), p.err)) != 0;
+        };
+        int nb = 0, q = 0, nt = 0;                 // slabs, units and tiles taken
+        bool ok = true;
+        for (int t = t0; t < t1 && ok; t += dt) {
+            if (!__any_sync(0xffffffffu, is_active(t))) continue;
+            if (nt > 0 && !wait(tempty, nt - 1)) { ok = false; break; }       // the accumulators have been drained
+            nt++;
+            for (int s = 0; s < nslab && ok; s++, nb++) {
+                const int bb = nb % BBUF;
+                if (!wait(bfull[bb], nb / BBUF)) { ok = false; break; }
+                const int nk16 = (min(OZ_KS, g.k - s * OZ_KS) + 15) / 16;
+                const uint64_t db = dB0 + (uint64_t)((bb * OZ_S * SLAB_B) >> 4);
+#pragma unroll
+                for (int u = 0; u < NU; u++, q++) {
+                    const int slot = q % RING;
+                    if (!wait(afull[slot], q / RING)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+                    for (int h = 0; h < OZ_UNIT; h++) {
+                        const int i = oz_order(OZ_UNIT * u + h);
+                        const uint64_t da = dA0 + (uint64_t)(((slot * OZ_UNIT + h) * OZ_SLAB_A) >> 4);
+                        // the first slice (i = 0, taken first) opens every group's accumulator
+                        const bool open = s == 0 && u == 0 && h == 0;
+                        // products (i, j), j = 0 .. 7 - i, land in groups i .. 7: adjacent BN-column
+                        // accumulators, and the B slices j are adjacent BN-row blocks in shared
+                        // memory, so one MMA of N = BN (8 - i) covers them; more than 256 columns
+                        // are two MMAs of about half the slices each
+                        const int n1 = OZ_S - i <= MAXB ? OZ_S - i : (OZ_S - i + 1) / 2, n2 = OZ_S - i - n1;
+                        const uint32_t acc = tm + (uint32_t)(i * BN);
+#pragma unroll
+                        for (int kk = 0; kk < OZ_KS / 16; kk++) {
+                            if (kk >= nk16) break;
+                            const uint32_t on = open && kk == 0 ? 0u : 1u;
+                            tc_mma_bf16_elect(acc, da + 2 * kk, db + 2 * kk, tc_idesc(TC_BF16, BN * n1), on, el);
+                            if (n2 > 0)
+                                tc_mma_bf16_elect(acc + (uint32_t)(n1 * BN), da + 2 * kk,
+                                                  db + (uint64_t)((n1 * SLAB_B) >> 4) + 2 * kk,
+                                                  tc_idesc(TC_BF16, BN * n2), on, el);
                         }
-                        asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-                        for (int h = 0; h < OZ_UNIT; h++) {
-                            const int i = oz_order(OZ_UNIT * u + h);
-                            const uint64_t da = dA0 + (uint64_t)(((slot * OZ_UNIT + h) * OZ_SLAB_A) >> 4);
-                            // the first slice (i = 0, taken first) opens every group's accumulator
-                            const uint32_t first = (s == 0 && u == 0 && h == 0) ? 1u : 0u;
-                            // products (i, j), j = 0 .. 7 - i, land in groups i .. 7: adjacent BN-column
-                            // accumulators, and the B slices j are adjacent BN-row blocks in shared
-                            // memory, so one MMA of N = BN (8 - i) (at most 256 per instruction) covers them
-#pragma unroll
-                            for (int kk = 0; kk < OZ_KS / 16; kk++) {
-                                if (kk < nk16) {
-#pragma unroll
-                                    for (int c = 0; c < OZ_S; c += MAXB) {
-                                        const int nn = min(MAXB, OZ_S - i - c);
-                                        if (nn > 0) {
-                                            const uint32_t acc = tmem + (uint32_t)((i + c) * BN);
-                                            const uint64_t db = dB0 + (uint64_t)((c * SLAB_B) >> 4) + 2 * kk;
-                                            tc_mma(acc, da + 2 * kk, db, tc_idesc(TC_BF16, BN * nn),
-                                                   (first && kk == 0) ? 0u : 1u, TC_BF16);
-                                        }
-                                    }
-                                }
-                            }
-                        }
-                        commit(aempty[slot]);
                     }
-                    if (!ok) break;
-                    commit(bempty);
-                    if (s == nslab - 1) commit(tfull);
-                    if (*(volatile int*)&abort_flag) ok = false;
+                    tc_commit_elect(smem_u32(&aempty[slot]), el);
                 }
+                if (!ok) break;
+                tc_commit_elect(smem_u32(&bempty[bb]), el);
+                if (s == nslab - 1) tc_commit_elect(smem_u32(&tfull), el);
+                if (__any_sync(0xffffffffu, *(volatile int*)&abort_flag)) ok = false;
             }
-            if (!ok) abort_flag = 1;
-            // every MMA issued has completed before TMEM is freed
-            commit(done);
-            mbar_wait(smem_u32(&done), 0u, p.err);
         }
+        if (!ok && lane == 0) abort_flag = 1;
+        // every MMA issued has completed before TMEM is freed
+        tc_commit_elect(smem_u32(&done), el);
+        mbar_wait(smem_u32(&done), 0u, p.err);
+        __syncwarp();
     } else {
         // epilogue: warps 0 .. EPIW - 1.  Warp w has TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, an output row per
         // thread, and the columns of part w / 4, four at a time: a sector of the row.  Results go from the
@@ -641,33 +646,67 @@ __global__ void __launch_bounds__(32 * (EPIW + 2), 2) oz_gemm_kernel(const __gri
                 if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&tempty)) : "memory");
             };
+            // the group sums of columns cl .. cl + 3 of this thread's row
+            auto load_sums = [&](uint32_t (&u)[OZ_G][4], int cl) {
+#pragma unroll
+                for (int G = 0; G < OZ_G; G++) {
+                    const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(G * BN + cl);
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                 : "=r"(u[G][0]), "=r"(u[G][1]), "=r"(u[G][2]), "=r"(u[G][3])
+                                 : "r"(ta));
+                }
+            };
+            // columns c0 .. c0 + 3 and on have no element of this warp's rows (warp-uniform)
+            auto beyond = [&](int c0) { return c0 >= g.n || (skew && m0 + lq * 32 + 31 < c0); };
+            // one CTA per SM: the sums of all columns first, so that the next tile's MMAs run during the rounding
+            // and the stores (the pass loop below takes entries 0 .. 3 and moves the others down)
+            long long hh[HOLD ? PCOLS : 4];
+            unsigned hl[HOLD ? PCOLS : 4];
+            if constexpr (HOLD) {
+                if (active) {
+#pragma unroll
+                    for (int pass = 0; pass < PASSES; pass++) {
+                        const int cl = part * PCOLS + 4 * pass;
+                        if (!beyond(n0 + cl)) {
+                            uint32_t u[OZ_G][4];
+                            load_sums(u, cl);
+                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                            for (int j = 0; j < 4; j++) oz_combine(u, j, hh[4 * pass + j], hl[4 * pass + j]);
+                        }
+                    }
+                    release();
+                }
+            }
 #pragma unroll 1
             for (int pass = 0; pass < PASSES; pass++) {
                 const int cl = part * PCOLS + 4 * pass, c0 = n0 + cl;
-                if (c0 >= g.n || (skew && m0 + lq * 32 + 31 < c0)) break;     // warp-uniform
+                if (beyond(c0)) break;
                 unsigned long long t[4] = {0ull, 0ull, 0ull, 0ull};
                 if (active) {
                     uint32_t u[OZ_G][4];
-#pragma unroll
-                    for (int G = 0; G < OZ_G; G++) {
-                        const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(G * BN + cl);
-                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(u[G][0]), "=r"(u[G][1]), "=r"(u[G][2]), "=r"(u[G][3])
-                                     : "r"(ta));
-                    }
+                    if constexpr (!HOLD) load_sums(u, cl);
                     if (pass + 1 < PASSES) load_cin(cn, c0 + 4);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (pass == PASSES - 1) release();
+                    if constexpr (!HOLD) {
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        if (pass == PASSES - 1) release();
+#pragma unroll
+                        for (int j = 0; j < 4; j++) oz_combine(u, j, hh[j], hl[j]);
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
                         // computed for every column and selected (no branch between the columns)
                         const int fc = __shfl_sync(0xffffffffu, fe, 4 * pass + j);
-                        long long H;
-                        unsigned L;
-                        oz_combine(u, j, H, L);
-                        const unsigned long long v = fast ? oz_to_double_bits_normal(H, L, er + fc - 2107 + ae, an)
-                                                          : oz_to_double_bits(H, L, er + fc - 2107 + ae, an);
+                        const unsigned long long v = fast ? oz_to_double_bits_normal(hh[j], hl[j], er + fc - 2107 + ae, an)
+                                                          : oz_to_double_bits(hh[j], hl[j], er + fc - 2107 + ae, an);
                         t[j] = (er > 0 && fc > 0) ? v : 0ull;
+                    }
+                    if constexpr (HOLD) {
+#pragma unroll
+                        for (int j = 0; j + 4 < PCOLS; j++) {
+                            hh[j] = hh[j + 4];
+                            hl[j] = hl[j + 4];
+                        }
                     }
                 } else if (pass + 1 < PASSES) {
                     load_cin(cn, c0 + 4);
@@ -857,11 +896,21 @@ inline int oz_sms() {
     return n;
 }
 
+// Tile width of a product: OZ_NARROW16's, OZ_NARROW's, or OZ_WIDE's for long sums with enough tiles that a last
+// partial round of whole SMs costs less than the wide tile gains.  Narrow / wide, us: 105 antisymmetric products of
+// 804^2 at K = 512 1162 / 945, at 292 1057 / 810; 45 of 388^2 at 388 201 / 164; 248 of 512 x 512 at K = 128 190 / 230;
+// general 512^2 at K = 512: 160 wide tiles 58 / 64, 192 61 / 64, 256 72 / 65, 320 99 / 90; at K = 256: 160 tiles
+// 37 / 44, 256 45 / 45.
+inline int oz_width(const GemmBatch& g, int bc) {
+    if (g.n <= 16) return 16;
+    return g.k >= 256 && (long long)oz_tiles(g, 64) * bc * 2 >= 3 * oz_sms() ? 64 : 32;
+}
+
 // the product kernel on slices in place (layout L) for batch entries b0 .. b0 + bc - 1;
 // b_rows: B's slices are its rows (an antisymmetric B), so alpha changes sign
 inline cudaError_t oz_product(const GemmBatch& g, const OzLayout& L, int b0, int bc, bool b_rows, int* err,
                               cudaStream_t st) {
-    const int bn = g.n <= 16 ? 16 : 32;                  // OZ_NARROW16's or OZ_NARROW's tile width
+    const int bn = oz_width(g, bc);
     OzGemm p;
     std::memset(&p, 0, sizeof(p));
     if (!make_slice_map(&p.ta, L.as, g.k, L.kp, L.mp, bc * OZ_S, OZ_BM, OZ_UNIT) ||
@@ -877,8 +926,10 @@ inline cudaError_t oz_product(const GemmBatch& g, const OzLayout& L, int b0, int
     p.tiles = oz_tiles(g, bn);
     p.total = p.tiles * bc;
     // two CTAs per SM and no more: with a few CTAs over, those few run their tiles after all others
-    const unsigned grid = (unsigned)std::min(p.total, 2 * oz_sms());
-    if (bn == 16)
+    const unsigned grid = (unsigned)std::min(p.total, (bn == 64 ? 1 : 2) * oz_sms());
+    if (bn == 64)
+        oz_gemm_kernel<OZ_WIDE><<<grid, OzCfg<OZ_WIDE>::THREADS, OzCfg<OZ_WIDE>::SMEM, st>>>(p);
+    else if (bn == 16)
         oz_gemm_kernel<OZ_NARROW16><<<grid, OzCfg<OZ_NARROW16>::THREADS, OzCfg<OZ_NARROW16>::SMEM, st>>>(p);
     else
         oz_gemm_kernel<OZ_NARROW><<<grid, OzCfg<OZ_NARROW>::THREADS, OzCfg<OZ_NARROW>::SMEM, st>>>(p);

@@ -844,6 +844,7 @@ void set_kernel_attributes() {
     raise_smem_limit(gemm_tma_kernel<TC_TF32>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_BF16>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_3XTF32>, optin);
+    raise_smem_limit(oz_gemm_kernel<OZ_WIDE>, optin);
     raise_smem_limit(oz_gemm_kernel<OZ_NARROW>, optin);
     raise_smem_limit(oz_gemm_kernel<OZ_NARROW16>, optin);
     raise_smem_limit(oz_block_slice_kernel, optin);

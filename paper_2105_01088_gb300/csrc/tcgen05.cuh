@@ -46,6 +46,25 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t da, uint64_t db
     }
 }
 
+// The same from a converged warp, issued by the lane with elect != 0.  In a warp-uniform flow the operands stay in
+// uniform registers; behind a branch on the lane each of them is moved there before every instruction.
+__device__ __forceinline__ uint32_t tc_elect() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+    return e;
+}
+__device__ __forceinline__ void tc_mma_bf16_elect(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accum,
+                                                  uint32_t elect) {
+    asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+                 :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accum), "r"(elect));
+}
+__device__ __forceinline__ void tc_commit_elect(uint32_t bar, uint32_t elect) {
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
+                 :: "r"(bar), "r"(elect) : "memory");
+}
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(bytes));
 }
@@ -68,6 +87,7 @@ constexpr uint64_t SGS_WAIT_LIMIT_NS = 2000000000ull;     // pipeline waits: 2 s
 
 template <class Done>
 __device__ __forceinline__ bool bounded_wait(Done done, uint64_t limit_ns, int* err, bool abort_on_flag) {
+    if (done()) return true;        // the clock is read only where there is something to wait for
     const uint64_t t0 = global_ns();
     for (uint32_t it = 0;; it++) {
         if (done()) return true;
