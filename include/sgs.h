@@ -214,7 +214,7 @@ sgs_status sgs_get_tuning(const sgs_ctx* ctx, int instance, int* gj_width, int* 
 /* Fix the panel widths of a live instance (for reproducible timings and
  * profiles): each must be one of the autotuner's candidates and fit the
  * instance's scratch (an instance admitted with autotuning on has room for
- * the widest).  Waits for the context's stream; drops a captured step graph.
+ * the widest), or the width the instance was admitted with.  Waits for the context's stream; drops a captured step graph.
  * SGS_EINVAL otherwise. */
 sgs_status sgs_set_panel_widths(sgs_ctx* ctx, int instance, int gj_width, int pf_width);
 

@@ -41,7 +41,7 @@
 // over each (a warp per row where the operand's K rows are contiguous and long,
 // else a block of whole rows at a time through shared memory), then the product
 // kernel.  It takes 128 x 32 output tiles with CTAs of 10 warps (256 TMEM
-// columns, 97 KB of shared memory), two to an SM, or, for K >= 256, 128 x 64 tiles with
+// columns, 97 KB of shared memory), two to an SM, or, for K > 240, 128 x 64 tiles with
 // one CTA of 18 warps an SM (all of its TMEM, 225 KB), which load 3/5 of the bytes per
 // output.  Each CTA runs over every (grid)-th tile, so that CTAs side by side work on
 // tiles side by side and share their slices in L2 (consecutive tiles per CTA read them
@@ -898,12 +898,13 @@ inline int oz_sms() {
 
 // Tile width of a product: OZ_NARROW16's, OZ_NARROW's, or OZ_WIDE's for long sums with enough tiles that a last
 // partial round of whole SMs costs less than the wide tile gains.  Narrow / wide, us: 105 antisymmetric products of
-// 804^2 at K = 512 1162 / 945, at 292 1057 / 810; 45 of 388^2 at 388 201 / 164; 248 of 512 x 512 at K = 128 190 / 230;
+// 804^2 at K = 512 1162 / 945, at 292 1057 / 810; 45 of 388^2 at 388 201 / 164; 120 general of 244^2 at 244 152 / 141;
+// 120 Gauss-Jordan updates of 512 x 128 at K = 128 96 / 131;
 // general 512^2 at K = 512: 160 wide tiles 58 / 64, 192 61 / 64, 256 72 / 65, 320 99 / 90; at K = 256: 160 tiles
 // 37 / 44, 256 45 / 45.
 inline int oz_width(const GemmBatch& g, int bc) {
     if (g.n <= 16) return 16;
-    return g.k >= 256 && (long long)oz_tiles(g, 64) * bc * 2 >= 3 * oz_sms() ? 64 : 32;
+    return g.k > 240 && (long long)oz_tiles(g, 64) * bc * 2 >= 3 * oz_sms() ? 64 : 32;
 }
 
 // the product kernel on slices in place (layout L) for batch entries b0 .. b0 + bc - 1;

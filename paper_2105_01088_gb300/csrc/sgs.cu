@@ -83,7 +83,8 @@ struct Instance {
     int* self_mask = nullptr;           // sharded: [M], 1 where this rank adds state mu's own term
     size_t oz_cap = 0;                  // emulated products: slice scratch cap (bytes)
     int gj_b = 32, pf_bs = 16;          // panel widths of the Gauss-Jordan inverse and the Pfaffian
-    int gj_cap = 32, pf_cap = 16;       // widest widths the scratch holds
+    int gj_cap = 32, pf_cap = 16;       // widest widths that may be set
+    int gj_def = 16;                    // the Gauss-Jordan width of an instance that was neither tuned nor fixed
     int tuned_from_cache = -1;          // -1 not tuned, 0 timed, 1 cached
     std::vector<int> h_pa, h_pb;
     std::vector<double> hA, hq_val;     // host copy of the model: rank growth rebuilds the instance
@@ -391,13 +392,24 @@ std::vector<int> gj_candidates(int n) {
         if (b <= n && (size_t)n * (b + 1) * sizeof(double) + b * sizeof(double) <= (size_t)limit) v.push_back(b);
     return v;
 }
-// leaf of the recursive form: 16 columns, or the widest candidate below it whose panel
-// fits shared memory (large n)
-int default_gj_width(int n) {
+int gj_cluster(int n, int batch, int bb);
+// leaf of the recursive form: 16 columns, or the widest candidate below it whose panel fits one CTA's shared memory
+// (n above about 1700).  In FP64, by the panels' cluster form for `batch` matrices:
+//   * 16 at those n too.  One step, leaf 12 / 16, ms: n = 2000, 28 pairs 151.1 / 142.7; 2000, 6: 61.9 / 59.0;
+//   * 32 where a CTA has at most 128 rows: half the panels and a level of updates less.  Leaf 16 / 32, us: n = 164,
+//     15 pairs 1438 / 1393 (energy); 164, 120: 3774 / 3667; 244, 120: 5740 / 5583; 388, 45: 6350 / 6225; 400, 66:
+//     10508 / 10213; 512, 28: 8711 / 8479; but 512, 120 (256 rows a CTA): 20361 / 20657; 800, 6: 12391 / 12463; 512,
+//     496 (no clusters): 68825 / 73030.
+// The mixed forms keep the first: their rounding to tf32 makes a change of S^{-1}'s last bits visible.
+int default_gj_width(int n, int batch, int prec) {
     int w = std::min(8, n);
     for (int b : gj_candidates(n))
         if (b <= 16) w = std::max(w, b);
-    return std::min(w, n);
+    w = std::min(w, n);
+    if (prec != SGS_FP64 || batch < 1) return w;
+    if (n >= 16 && w < 16 && gj_cluster(n, batch, 16) > 0) return 16;
+    const int C = gj_cluster(n, batch, 32);
+    return n >= 64 && n <= 512 && C > 0 && (n + C - 1) / C <= 128 ? 32 : w;
 }
 std::vector<int> pf_candidates(int n) {
     std::vector<int> v;
@@ -461,9 +473,8 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
     I.hA.assign(m.A, m.A + (size_t)n * n);
     I.hq_idx.assign(m.quartic_idx, m.quartic_idx + (m.n_quartic > 0 ? 4 * m.n_quartic : 0));
     I.hq_val.assign(m.quartic_val, m.quartic_val + (m.n_quartic > 0 ? m.n_quartic : 0));
-    I.gj_b = default_gj_width(n);
     I.pf_bs = default_pf_width(n);
-    I.gj_cap = I.gj_b;
+    I.gj_cap = default_gj_width(n, 0, I.prec);
     I.pf_cap = I.pf_bs;
     if (c->autotune) {          // scratch for the widest candidate
         for (int b : gj_candidates(n)) I.gj_cap = std::max(I.gj_cap, b);
@@ -593,6 +604,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
         I.Ppfc = std::max(I.Ppfc, k);
     }
     I.cur = 0;
+    I.gj_b = I.gj_def = default_gj_width(n, I.Pc, I.prec);
     if (pair_pf.empty()) pair_pf.push_back(-1);
     const int Pc = I.Pc;
 
@@ -619,7 +631,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
     I.work = c->alloc<double>(Pcm * 2 * nn);
     I.si = c->alloc<double>(Pcm * nn); I.imd = c->alloc<double>(Pcm * nn);
     I.wr = c->alloc<double>(Pcm * nn); I.va = c->alloc<double>(Pcm * nn); I.xa = c->alloc<double>(Pcm * nn);
-    I.tbuf = c->alloc<double>(Pcm * I.gj_cap * n);
+    I.tbuf = c->alloc<double>(Pcm * std::max(I.gj_cap, I.gj_def) * n);
     I.piv = c->alloc<int>(Pcm * n); I.perm = c->alloc<int>(Pcm * n);
     I.logdet = c->alloc<double>(Pcm); I.dsign = c->alloc<double>(Pcm);
     I.pfTU = c->alloc<double>(Pfc * 4 * n * I.pf_cap);
@@ -1323,8 +1335,12 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     };
     int gj = I.gj_b, pf = I.pf_bs;
     float best = 1e30f;
-    for (int b : gj_candidates(I.n)) {
-        if (b > I.gj_cap) continue;
+    const std::vector<int> gjc = gj_candidates(I.n);
+    const bool extra = std::find(gjc.begin(), gjc.end(), I.gj_def) == gjc.end();    // a width of the cluster form only
+    std::vector<int> tried = gjc;
+    if (extra) tried.push_back(I.gj_def);
+    for (int b : tried) {
+        if (b > I.gj_cap && b != I.gj_def) continue;
         if ((status = set_panel_pointers(c, I, b, pf)) != SGS_OK) break;
         const float t = timed([&] { return cudaSuccess; }, [&] { return pair_inverse(c, I, st); });
         if (t < best) { best = t; gj = b; }
@@ -1351,7 +1367,7 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     CUDA_TRY(c, cudaMemsetAsync(I.err, 0, sizeof(int), st));      // trial runs leave no error state
     CUDA_TRY(c, cudaStreamSynchronize(st));
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = {gj, pf};
+    if (!(extra && gj == I.gj_def)) g_tune_cache[key] = {gj, pf};      // that width depends on the number of pairs
     I.tuned_from_cache = 0;
     return SGS_OK;
 }
@@ -2075,7 +2091,7 @@ sgs_status sgs_set_panel_widths(sgs_ctx* c, int instance, int gj_width, int pf_w
     if (!c || instance < 0 || instance >= (int)c->inst.size() || !c->inst[instance].live) return SGS_EINVAL;
     Instance& I = c->inst[instance];
     const std::vector<int> gj = gj_candidates(I.n), pf = pf_candidates(I.n);
-    if (std::find(gj.begin(), gj.end(), gj_width) == gj.end() || gj_width > I.gj_cap ||
+    if ((gj_width != I.gj_def && (std::find(gj.begin(), gj.end(), gj_width) == gj.end() || gj_width > I.gj_cap)) ||
         std::find(pf.begin(), pf.end(), pf_width) == pf.end() || pf_width > I.pf_cap) {
         c->err = "panel width not a candidate, or wider than the instance's scratch";
         return SGS_EINVAL;

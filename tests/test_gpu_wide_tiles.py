@@ -15,6 +15,7 @@ def pkg():
 
 
 @pytest.mark.parametrize("batch,m,n,k,kw", [
+    (76, 129, 65, 241, dict()),
     (76, 129, 65, 256, dict()),
     (76, 200, 131, 257, dict(beta=1.0)),
     (120, 128, 66, 300, dict(alpha=0.7, beta=-0.3, diag=2.0)),
