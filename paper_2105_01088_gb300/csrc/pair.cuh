@@ -397,34 +397,95 @@ __global__ void __launch_bounds__(256) pair_q_kernel(InstDev d, const double* si
     store_antisym_tile(Qi, n, k0, l0, sq[1]);
 }
 
-// Tensor-core operands from FP64 (or fp32) data: x = src - src2 (src2 optional)
+// (float)x and, for the 3xTF32 split, h = (float)x with 13 bits cut off and lo = (float)(x - h), in integer
+// arithmetic on x's bits: an FP64 addition or a conversion from or to FP64 takes 19 clocks of an SM per warp.
+// x = m 2^(e - 1075), m of 53 bits; (float)x = q 2^(e - 1046), q = m 2^-29 rounded to nearest even (a carry
+// moves into the exponent); x - h is the integer d times m's unit, |d| <= 2^42, rounded once by the fma of its
+// two parts.  Exponents where the results are no normal numbers (zeros apart) take the FP64 instructions.
+__device__ __forceinline__ void lp_split(double x, bool split, float& f, float& h, float& lo) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)((u >> 52) & 0x7ff);
+    const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
+    if (e >= 949 && e <= 1149) {
+        const unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+        const unsigned q = (unsigned)((m + 0xFFFFFFFull + ((m >> 29) & 1ull)) >> 29);
+        const unsigned fb = sg | (((unsigned)(e - 897) << 23) + q);
+        f = __uint_as_float(fb);
+        h = __uint_as_float(fb & 0xffffe000u);
+        if (split) {
+            long long d = (long long)m - (long long)((unsigned long long)(q & 0xffffe000u) << 29);
+            if (sg) d = -d;
+            const float dh = (float)(int)(d >> 18), dl = (float)(int)(d & 0x3FFFFll);
+            lo = fmaf(dh, 262144.0f, dl) * __uint_as_float((unsigned)(e - 948) << 23);
+        }
+    } else if ((u << 1) == 0ull) {
+        f = h = __uint_as_float(sg);
+        lo = 0.0f;
+    } else {
+        f = (float)x;
+        h = __uint_as_float(__float_as_uint(f) & 0xffffe000u);
+        lo = (float)(x - (double)h);
+    }
+}
+__device__ __forceinline__ void lp_split(float x, bool, float& f, float& h, float& lo) {
+    f = x;
+    h = __uint_as_float(__float_as_uint(f) & 0xffffe000u);
+    lo = f - h;                                     // exact
+}
+
+// Tensor-core operands from FP64 (or fp32) data: x = src - src2 (src2 optional, FP64)
 // to fp32 (TF32 kind), bf16, or an exact fp32 split hi + lo with hi on the
 // tf32 grid (3xTF32).  Sources are n x n with leading dimension n; operands
 // have leading dimension ldp >= n (a multiple of 8: a 16-byte chunk holds 8
-// bf16 values), columns n..ldp-1 zero.
+// bf16 values), columns n..ldp-1 zero.  Four columns per thread.
+// Bound by memory: 120 operands of 804^2 from FP64 to a split 720 us with an FP64 subtraction and three conversions
+// per element (855 us from fp32, by way of FP64); now 221 and 136.
 template <typename S>
-__global__ void lp_convert_kernel(const S* const* src, const double* const* src2, void* const* hi, void* const* lo,
-                                  int n, int ldp, int kind) {
+__global__ void __launch_bounds__(256) lp_convert_kernel(const S* const* src, const double* const* src2, void* const* hi,
+                                                         void* const* lo, int n, int ldp, int kind) {
     const int b = blockIdx.y;
     const S* x0 = src[b];
     const double* x1 = src2 ? src2[b] : nullptr;
-    const size_t count = (size_t)n * ldp;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / ldp), q = (int)(e % ldp);
-        double x = 0.0;
-        if (q < n) {
-            const size_t o = (size_t)r * n + q;
-            x = (double)x0[o] - (x1 ? x1[o] : 0.0);
-        }
-        if (kind == 1) {
-            static_cast<__nv_bfloat16*>(hi[b])[e] = __float2bfloat16_rn((float)x);
-        } else if (kind == 2) {
-            const float f = (float)x;
-            const float h = __uint_as_float(__float_as_uint(f) & 0xffffe000u);
-            static_cast<float*>(hi[b])[e] = h;
-            static_cast<float*>(lo[b])[e] = (float)(x - (double)h);
+    const unsigned cols = (unsigned)ldp >> 2, count = (unsigned)n * cols;
+    // pairs of elements at their natural alignment (n even and the base aligned)
+    const bool pairs = (n & 1) == 0 && ((uintptr_t)x0 & (2 * sizeof(S) - 1)) == 0 && ((uintptr_t)x1 & 15) == 0;
+    struct alignas(2 * sizeof(S)) S2 { S a, b; };
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < count; t += gridDim.x * blockDim.x) {
+        const unsigned r = t / cols;
+        const int q = 4 * (int)(t - r * cols);
+        S x[4];
+        const S* row = x0 + (size_t)r * n;
+        if (pairs) {
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                const S2 v = q + j < n ? *reinterpret_cast<const S2*>(row + q + j) : S2{S(0), S(0)};
+                x[j] = v.a;
+                x[j + 1] = v.b;
+            }
         } else {
-            static_cast<float*>(hi[b])[e] = round_tf32((float)x);
+#pragma unroll
+            for (int j = 0; j < 4; j++) x[j] = q + j < n ? row[q + j] : S(0);
+        }
+        if (x1) {
+            const double* row1 = x1 + (size_t)r * n;
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (q + j < n) x[j] = (S)((double)x[j] - row1[q + j]);
+        }
+        float f[4], h[4], l[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) lp_split(x[j], kind == 2, f[j], h[j], l[j]);
+        const size_t e = (size_t)r * ldp + q;
+        if (kind == 1) {
+            __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(hi[b]) + e);
+            o[0] = __floats2bfloat162_rn(f[0], f[1]);
+            o[1] = __floats2bfloat162_rn(f[2], f[3]);
+        } else if (kind == 2) {
+            *reinterpret_cast<float4*>(static_cast<float*>(hi[b]) + e) = make_float4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<float4*>(static_cast<float*>(lo[b]) + e) = make_float4(l[0], l[1], l[2], l[3]);
+        } else {
+            *reinterpret_cast<float4*>(static_cast<float*>(hi[b]) + e) =
+                make_float4(round_tf32(f[0]), round_tf32(f[1]), round_tf32(f[2]), round_tf32(f[3]));
         }
     }
 }
