@@ -239,8 +239,17 @@ __global__ void __launch_bounds__(256) oz_block_slice_kernel(OzOperand o) {
     }
 }
 
+// four doubles' bits at a 32-byte boundary, as one access
+__device__ __forceinline__ void oz_ld4(unsigned long long (&x)[4], const double* p) {
+    asm volatile("ld.global.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3]) : "l"(p));
+}
+__device__ __forceinline__ void oz_st4(unsigned long long* p, const unsigned long long (&x)[4]) {
+    asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};" :: "l"(p), "l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]) : "memory");
+}
+
 // contiguous rows (K <= 128 S): one warp per row takes the row into registers, reduces the
 // exponent field and writes the digits, four k per lane per step (one pass over the operand)
+// Bound by memory: 496 operands of 512^2 (3.1 GB) 636 us with 8-byte loads at a stride of 32, 517 with 32-byte ones.
 template <int S>
 __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
     const int bl = blockIdx.y, b = o.b0 + bl;
@@ -250,15 +259,37 @@ __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
     const double* x = o.X[b] + o.off;
     const double* x2 = o.X2 ? o.X2[b] + o.off : nullptr;
     unsigned long long v[S][4];          // k = 4 lane + 128 s + u
+    const bool wide = (((uintptr_t)x | (uintptr_t)x2 | ((uintptr_t)o.ld * 8)) & 31) == 0;      // rows on 32 bytes
+#pragma unroll
+    for (int s = 0; s < S; s++) {
+        const int k = 128 * s + 4 * lane;
+        if (wide && r < o.rows && k + 3 < o.k) {
+            oz_ld4(v[s], x + (size_t)r * o.ld + k);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                v[s][u] = (r < o.rows && k + u < o.k) ? oz_load(o, x, x2, r, k + u) : 0ull;
+        }
+    }
+    if (wide && x2) {
+#pragma unroll
+        for (int s = 0; s < S; s++) {
+            const int k = 128 * s + 4 * lane;
+            if (r < o.rows && k + 3 < o.k) {
+                unsigned long long w[4];
+                oz_ld4(w, x2 + (size_t)r * o.ld + k);
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    v[s][u] = (unsigned long long)__double_as_longlong(
+                        fma(o.s2, __longlong_as_double((long long)w[u]), __longlong_as_double((long long)v[s][u])));
+            }
+        }
+    }
     int e = 0;
 #pragma unroll
     for (int s = 0; s < S; s++)
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int k = 128 * s + 4 * lane + u;
-            v[s][u] = (r < o.rows && k < o.k) ? oz_load(o, x, x2, r, k) : 0ull;
-            e = max(e, oz_expo_field(v[s][u]));
-        }
+        for (int u = 0; u < 4; u++) e = max(e, oz_expo_field(v[s][u]));
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0 && r < o.rows) o.expo[(size_t)bl * o.rows_pad + r] = e;
 #pragma unroll
@@ -266,14 +297,6 @@ __global__ void __launch_bounds__(256) oz_row_slice_kernel(OzOperand o) {
         const int k = 128 * s + 4 * lane;
         if (k < o.kp) oz_store4(o, bl, r, k, v[s], r < o.rows ? e : 0);
     }
-}
-
-// four doubles' bits at a 32-byte boundary, as one access
-__device__ __forceinline__ void oz_ld4(unsigned long long (&x)[4], const double* p) {
-    asm volatile("ld.global.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3]) : "l"(p));
-}
-__device__ __forceinline__ void oz_st4(unsigned long long* p, const unsigned long long (&x)[4]) {
-    asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};" :: "l"(p), "l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]) : "memory");
 }
 
 struct OzGemm {
