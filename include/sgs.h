@@ -78,7 +78,7 @@ typedef enum {
  *    those maxima is less accurate than the K u sum_k |A_ik||B_kj| of a native
  *    FP64 dot product.
  *  - SGS_FP64_FMA: FP64 fused multiply-adds on the CUDA cores (the error of a
- *    native FP64 dot product), about 8x slower on GB300 at 2N = 512. In SGS_FP64 instances of either
+ *    native FP64 dot product), about 10x slower on GB300 at 2N = 512.  In SGS_FP64 instances of either
  * path, products of few operations (3e6 multiply-adds a launch) run on the FP64
  * pipe: the elementwise bound holds there. */
 typedef enum {
