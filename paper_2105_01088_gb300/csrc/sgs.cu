@@ -897,11 +897,12 @@ int threads_per_row(int ch) {             // the power's exponent
 // below a few hundred matrices and pays one SM's FP64 pipe per column; more CTAs than SMs (152) only
 // share them.  Panels of 16 columns, one-CTA form against the best C, us: n = 64, 6 matrices 53 / 32
 // (C = 8); n = 164, 15: 59 / 36 (8); n = 244, 60: 65 / 47 (4); n = 388, 45: 90 / 53 (8); n = 804, 60:
-// 151 / 90 (4, 8); n = 2000, 14 (12 columns): 237 / 61 (8); at n = 512, 248 in a step, where another
-// stream shares the SMs, the one-CTA form stays ahead.
+// 151 / 90 (4, 8); n = 2000, 14 (12 columns): 237 / 61 (8).  Pairs of CTAs pay up to about 256 matrices (1.6 matrices
+// per SM leave some SMs twice the work of others).  One step, one-CTA form / pairs, us: n = 512, 248 matrices in each half 65310
+// / 64520; 244, 126: 9400 / 9320; 164, 248: 9750 / 9560.  Four or eight CTAs beyond 320 in all lost: n = 244, 60: 5470 / 5590.
 int gj_cluster(int n, int batch, int bb) {
     for (int C = 8; C >= 2; C /= 2)
-        if (batch * C <= 320 && n >= 8 * C && gjc_smem(bb, C, (n + C - 1) / C) <= 200 * 1024) return C;
+        if (batch * C <= (C == 2 ? 512 : 320) && n >= 8 * C && gjc_smem(bb, C, (n + C - 1) / C) <= 200 * 1024) return C;
     return 0;
 }
 // 16 steps on `live` rows, one-CTA form against the best C, us: 64 rows, 3 matrices 153 / 80 (4); 164, 10:

@@ -19,7 +19,7 @@ def skew(rng, b, n, cplx=False):
 
 
 @pytest.mark.parametrize("path", [sgs.FP64_EMULATED, sgs.FP64_FMA])
-@pytest.mark.parametrize("n,batch", [(2, 1), (14, 3), (16, 3), (18, 41), (64, 40), (66, 2), (130, 79), (164, 81), (258, 161),
+@pytest.mark.parametrize("n,batch", [(2, 1), (14, 3), (16, 3), (18, 41), (64, 40), (66, 2), (130, 79), (164, 81), (258, 161), (66, 256), (66, 257),
                                      (330, 3), (1030, 1)])
 def test_inverse(n, batch, path):
     S = skew(np.random.default_rng(n * 1000 + batch), batch, n)
