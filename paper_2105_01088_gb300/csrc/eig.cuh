@@ -415,12 +415,15 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     if (warp == 0) {
         // lo, hi bracket the lowest eigenvalue: Gershgorin below, the smallest diagonal entry above
         double lo = INFINITY, hi = INFINITY, top = 0.0;
+        bool nan = false;
         for (int i = lane; i < M; i += 32) {
             const double r = (i > 0 ? fabs(s_e[i - 1]) : 0.0) + (i + 1 < M ? fabs(s_e[i]) : 0.0);
             lo = fmin(lo, s_d[i] - r);
             hi = fmin(hi, s_d[i]);
             top = fmax(top, fabs(s_d[i]) + r);
+            nan = nan || !isfinite(s_d[i] + r);
         }
+        nan = __any_sync(0xffffffffu, nan);                  // (fmin and fmax drop a NaN)
         for (int o = 16; o > 0; o >>= 1) {
             lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
             hi = fmin(hi, __shfl_xor_sync(0xffffffffu, hi, o));
@@ -441,7 +444,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
         // its factorisation needs no pivoting; each pass cuts the other components by about
         // 16 ulp top / gap
         if (lane == 0) {
-            s_E = 0.5 * (lo + hi);
+            s_E = nan ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (lo + hi);
             const double x = lo - 16.0 * ulp * top, least = ulp * top + 1e-300;
             double* q = reinterpret_cast<double*>(s_part);             // 1 / pivots
             double* l = q + MR;                                        // multipliers
@@ -547,6 +550,7 @@ __global__ void __launch_bounds__(AMP_THREADS) amp_solve_kernel(AmpArgs a) {
     nrm = block_sum(nrm, red);
     if (tid == 0) {
         const double sc = 1.0 / sqrt(nrm);
+        if (!(nrm > 0.0) || !isfinite(nrm)) atomicOr(a.err, SGS_DEV_EIG);
         int jb = 0;
         double best = -1.0;
         for (int i = 0; i < M; i++) {
