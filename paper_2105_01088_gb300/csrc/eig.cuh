@@ -238,7 +238,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // T - x positive definite (T real symmetric tridiagonal: diagonal d, off-diagonal e with squares
 // e2): every leading principal minor positive, by the minors' three-term recurrence; the pair of
-// minors is rescaled by a power of two every four rows, so it neither over- nor underflows
+// minors is rescaled by a power of two every four rows, so it neither over- nor underflows for T of magnitude
+// 2^-150 .. 2^150 (the caller scales others)
 __device__ __forceinline__ bool amp_posdef(const double* d, const double* e2, int M, double x) {
     double p0 = 1.0, p1 = d[0] - x;
     bool ok = p1 > 0.0;
@@ -413,6 +414,25 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     for (int i = tid; i < M; i += AMP_THREADS) s_d[i] = B[i * ld + i].x;
     __syncthreads();
     if (warp == 0) {
+        // T of extreme magnitude (energies in units far from its own): to order one by a power of two, exact
+        int ex = 0;
+        for (int i = lane; i < M; i += 32) {
+            ex = max(ex, (__double2hiint(s_d[i]) >> 20) & 0x7ff);
+            if (i + 1 < M) ex = max(ex, (__double2hiint(s_e[i]) >> 20) & 0x7ff);
+        }
+        ex = __reduce_max_sync(0xffffffffu, ex);
+        const int f = ex > 0 && (ex < 1023 - 150 || ex > 1023 + 150) ? min(max(2046 - ex, 1), 2045) : 1023;
+        if (f != 1023) {
+            const double sc = __hiloint2double(f << 20, 0);
+            for (int i = lane; i < M; i += 32) {
+                s_d[i] *= sc;
+                if (i + 1 < M) {
+                    s_e[i] *= sc;
+                    s_e2[i] = s_e[i] * s_e[i];
+                }
+            }
+            __syncwarp();
+        }
         // lo, hi bracket the lowest eigenvalue: Gershgorin below, the smallest diagonal entry above
         double lo = INFINITY, hi = INFINITY, top = 0.0;
         bool nan = false;
@@ -444,7 +464,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
         // its factorisation needs no pivoting; each pass cuts the other components by about
         // 16 ulp top / gap
         if (lane == 0) {
-            s_E = nan ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (lo + hi);
+            s_E = nan ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (lo + hi) * __hiloint2double((2046 - f) << 20, 0);
             const double x = lo - 16.0 * ulp * top, least = ulp * top + 1e-300;
             double* q = reinterpret_cast<double*>(s_part);             // 1 / pivots
             double* l = q + MR;                                        // multipliers
