@@ -1732,7 +1732,9 @@ cudaError_t update_pass(sgs_ctx* c, Instance& I, cudaStream_t st) {
     c->stage_flops[SGS_STAGE_UPDATE] += (2.0 + 9.0 + 2.0 + 1.0 + 2.0) * n3 * M;
     // Y = Gamma dGamma -> s0 ; R -> p_R
     GemmBatch g = gb_basic(n, n, n, I.p_gamma, n, I.p_dgamma, n, I.p_s[0], n, M);
-    g.b_antisym = 1;    // dGamma, as the assembly stores it
+    // dGamma as the assembly stores it; a pair-sharded instance's comes from the caller, whose sum over the
+    // ranks need not be antisymmetric to the last bit
+    g.b_antisym = I.shard_world == 1;
     if ((e = gemm(c, I, g, st, 2.0 * n3 * M)) != cudaSuccess) return e;
     if ((e = exp_products(c, I, M, I.dtau, st)) != cudaSuccess) return e;
     // T = R Gamma -> s0 ; Gamma' = T R^T -> s2
