@@ -64,8 +64,15 @@ __device__ __forceinline__ void oz_digits4(const double (&v)[4], const bool (&pr
 // Products of many pivots are kept as a mantissa and an exponent of two, so that the logarithm, the
 // square root and the divisions (hundreds of clocks each on this part's FP64 pipe) are taken once per
 // matrix instead of once per pivot.  x scaled by a power of two to magnitude 1 .. 2 by its bits, the
-// exponent added to e; subnormals, zero, infinities and NaN are left as they are
-__device__ __forceinline__ double pow2_split(double x, int f, int& e) {
+// exponent added to e; zero, infinities and NaN are left as they are (a subnormal is scaled up first: a
+// product of two of them would vanish)
+__device__ __forceinline__ double pow2_split(double x, int& e) {
+    int f = (__double2hiint(x) >> 20) & 0x7ff;
+    if (f == 0 && (__double_as_longlong(x) << 1) != 0) {
+        x *= 0x1p54;
+        e -= 54;
+        f = (__double2hiint(x) >> 20) & 0x7ff;
+    }
     const bool ok = f > 0 && f < 2047;
     e += ok ? f - 1023 : 0;
     return ok ? __hiloint2double(__double2hiint(x) - ((f - 1023) << 20), __double2loint(x)) : x;
@@ -79,7 +86,7 @@ __device__ void gj_det(const GJPanelArgs& a, int b, const double* pabs, bool neg
     const int lane = threadIdx.x & 31;
     int e = 0;
     double m = 1.0;
-    for (int j = lane; j < a.bb; j += 32) m = pow2_split(m * pabs[j], expo_field(m * pabs[j]), e);
+    for (int j = lane; j < a.bb; j += 32) m *= pow2_split(pabs[j], e);
     for (int o = 16; o > 0; o >>= 1) {
         m *= __shfl_xor_sync(0xffffffffu, m, o);
         e += __shfl_xor_sync(0xffffffffu, e, o);
@@ -87,7 +94,7 @@ __device__ void gj_det(const GJPanelArgs& a, int b, const double* pabs, bool neg
     if (lane != 0) return;
     const double m0 = a.k0 == 0 ? 1.0 : a.dsign[b];
     double ex = a.k0 == 0 ? 0.0 : a.logdet[b];
-    m = pow2_split(m * m0, expo_field(m * m0), e);
+    m = pow2_split(m * m0, e);
     ex = singular ? -INFINITY : ex + e;
     if (negative) m = -m;
     if (a.k0 + a.bb == a.n) {
