@@ -259,6 +259,141 @@ __device__ __forceinline__ bool amp_posdef(const double* d, const double* e2, in
     return ok;
 }
 
+// a Hermitian matrix reduced to a real symmetric tridiagonal T (diagonal d, off-diagonal e with squares e2)
+struct AmpTri {
+    double d[SGS_MAX_RANK], e[SGS_MAX_RANK], e2[SGS_MAX_RANK];
+    cplx v[SGS_MAX_RANK], w[SGS_MAX_RANK], tau[SGS_MAX_RANK], part[AMP_THREADS / 32][SGS_MAX_RANK];
+};
+
+// The reduction of B (M x M, row stride ld, overwritten) by the whole block; the reflectors' vectors into the columns
+// of V (may be nullptr)
+__device__ __forceinline__ void amp_reduce(cplx* V, cplx* B, int M, int ld, AmpTri& t) {
+    constexpr int NW = AMP_THREADS / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // Householder reduction: reflector k = 1 - tau v v^dag (v_{k+1} = 1) makes column k (beta, 0, ..)
+    // with real beta; A <- A - v w^dag - w v^dag, w = p - (tau/2) (p^dag v) v, p = tau A v
+    for (int k = 0; k + 1 < M; k++) {
+        if (warp == 0) {
+            double xn = 0.0;
+            for (int i = k + 2 + lane; i < M; i += 32) xn += cabs2(B[i * ld + k]);
+            xn = warp_sum(xn);
+            const cplx al = B[(k + 1) * ld + k];
+            cplx tau = cmk(0.0, 0.0), sc = cmk(0.0, 0.0);
+            double beta = al.x;
+            if (xn > 0.0 || al.y != 0.0) {
+                beta = sqrt(cabs2(al) + xn);
+                if (al.x >= 0.0) beta = -beta;
+                const double rb = 1.0 / beta;
+                tau = cmk((beta - al.x) * rb, -al.y * rb);
+                const cplx q = cmk(al.x - beta, al.y);
+                sc = cscale(cconj(q), 1.0 / cabs2(q));
+            }
+            for (int i = k + 1 + lane; i < M; i += 32) {
+                const cplx v = i == k + 1 ? cmk(1.0, 0.0) : cmul(B[i * ld + k], sc);
+                t.v[i] = v;
+                if (V) V[i * ld + k] = v;       // kept for the back transformation
+            }
+            if (lane == 0) { t.tau[k] = tau; t.e[k] = beta; t.e2[k] = beta * beta; }
+        }
+        __syncthreads();
+        // A v: lanes over rows, the columns shared out among the warps
+        for (int i = k + 1 + lane; i < M; i += 32) {
+            cplx p = cmk(0.0, 0.0);
+            for (int j = k + 1 + warp; j < M; j += NW) cfma(p, B[i * ld + j], t.v[j]);
+            t.part[warp][i] = p;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const cplx tau = t.tau[k];
+            double dr = 0.0, di = 0.0;
+            for (int i = k + 1 + lane; i < M; i += 32) {
+                cplx p = t.part[0][i];
+                for (int w = 1; w < NW; w++) p = cadd(p, t.part[w][i]);
+                p = cmul(tau, p);
+                t.w[i] = p;
+                const cplx x = cmul(cconj(p), t.v[i]);
+                dr += x.x;
+                di += x.y;
+            }
+            const cplx f = cscale(cmul(tau, cmk(warp_sum(dr), warp_sum(di))), -0.5);
+            for (int i = k + 1 + lane; i < M; i += 32) {
+                cplx w = t.w[i];
+                cfma(w, f, t.v[i]);
+                t.w[i] = w;
+            }
+        }
+        __syncthreads();
+        for (int i = k + 1 + warp; i < M; i += NW) {
+            const cplx vi = cscale(t.v[i], -1.0), wi = cscale(t.w[i], -1.0);
+            for (int j = k + 1 + lane; j <= i; j += 32) {
+                cplx x = B[i * ld + j];
+                cfma(x, vi, cconj(t.w[j]));
+                cfma(x, wi, cconj(t.v[j]));
+                if (i == j) x.y = 0.0;
+                B[i * ld + j] = x;
+                B[j * ld + i] = cconj(x);
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < M; i += AMP_THREADS) t.d[i] = B[i * ld + i].x;
+    __syncthreads();
+}
+
+// The lowest eigenvalue of T between lo and hi, by one warp: T is scaled to order one first where its magnitude is
+// extreme (by 2^(f - 1023), f returned); top bounds |T|, nan: T is not finite
+__device__ __forceinline__ int amp_lowest(AmpTri& t, int M, double& lo, double& hi, double& top, bool& nan) {
+    const int lane = threadIdx.x & 31;
+    // T of extreme magnitude (energies in units far from its own): to order one by a power of two, exact
+    int ex = 0;
+    for (int i = lane; i < M; i += 32) {
+        ex = max(ex, (__double2hiint(t.d[i]) >> 20) & 0x7ff);
+        if (i + 1 < M) ex = max(ex, (__double2hiint(t.e[i]) >> 20) & 0x7ff);
+    }
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    const int f = ex > 0 && (ex < 1023 - 150 || ex > 1023 + 150) ? min(max(2046 - ex, 1), 2045) : 1023;
+    if (f != 1023) {
+        const double sc = __hiloint2double(f << 20, 0);
+        for (int i = lane; i < M; i += 32) {
+            t.d[i] *= sc;
+            if (i + 1 < M) {
+                t.e[i] *= sc;
+                t.e2[i] = t.e[i] * t.e[i];
+            }
+        }
+        __syncwarp();
+    }
+    // lo, hi bracket the lowest eigenvalue: Gershgorin below, the smallest diagonal entry above
+    lo = hi = INFINITY;
+    top = 0.0;
+    nan = false;
+    for (int i = lane; i < M; i += 32) {
+        const double r = (i > 0 ? fabs(t.e[i - 1]) : 0.0) + (i + 1 < M ? fabs(t.e[i]) : 0.0);
+        lo = fmin(lo, t.d[i] - r);
+        hi = fmin(hi, t.d[i]);
+        top = fmax(top, fabs(t.d[i]) + r);
+        nan = nan || !isfinite(t.d[i] + r);
+    }
+    nan = __any_sync(0xffffffffu, nan);                  // (fmin and fmax drop a NaN)
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmin(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    }
+    const double ulp = 2.220446049250313e-16;
+    lo -= 4.0 * ulp * top;
+    for (int it = 0; it < 14 && hi - lo > ulp * fmax(fabs(lo), fabs(hi)); it++) {
+        const double x = fma(hi - lo, (lane + 1) * (1.0 / 33.0), lo);
+        const unsigned pd = __ballot_sync(0xffffffffu, amp_posdef(t.d, t.e2, M, x));
+        const int n = __ffs(~pd) - 1;                    // shifts 0 .. n - 1 lie below (n = -1: all)
+        const double below = __shfl_sync(0xffffffffu, x, n > 0 ? n - 1 : (n < 0 ? 31 : 0));
+        const double above = __shfl_sync(0xffffffffu, x, n < 0 ? 31 : n);
+        if (n != 0) lo = below;
+        if (n >= 0) hi = above;
+    }
+    return f;
+}
+
 // The direct route: lr and E as amp_jacobi gives them, up to lambda's scale and phase.  Returns false
 // (nothing decided) where a pivot is not positive, tr(G) tr(G^{-1}) >= AMP_COND, or overlaps or amplitudes
 // are small (AMP_SMALL).  M <= SGS_MAX_RANK;
@@ -266,8 +401,8 @@ __device__ __forceinline__ bool amp_posdef(const double* d, const double* e2, in
 // both row and column walks free of bank conflicts.
 __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, double& E) {
     constexpr int NW = AMP_THREADS / 32, MR = SGS_MAX_RANK;
-    __shared__ double s_d[MR], s_rcp[MR], s_e[MR], s_e2[MR], red[32], s_E;
-    __shared__ cplx s_v[MR], s_w[MR], s_tau[MR], s_part[NW][MR];
+    __shared__ AmpTri t;
+    __shared__ double s_rcp[MR], red[32], s_E;
     __shared__ int s_bad;
     const int M = a.M, ld = M + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     cplx* A = sm;                   // G, then U^{-1} h
@@ -290,7 +425,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     if (tid == 0) {
         const double d = a.Gm[0];
         s_bad = !(d > 0.0);
-        s_d[0] = d;
+        t.d[0] = d;
         s_rcp[0] = 1.0 / d;
     }
     if (!__syncthreads_or(overlap)) return false;
@@ -313,7 +448,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
                     A[i * ld + j] = x;
                     if (i == k + 1) {
                         if (!(x.x > 0.0)) s_bad = 1;
-                        s_d[i] = x.x;
+                        t.d[i] = x.x;
                         s_rcp[i] = 1.0 / x.x;
                     }
                 }
@@ -326,7 +461,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
         for (int j = lane; j <= i; j += 32) tri += cabs2(W[i * ld + j]) * s_rcp[i];
     tri = block_sum(tri, red);
     if (s_bad || !(trg * tri < AMP_COND)) return false;
-    if (tid < M) s_rcp[tid] = 1.0 / sqrt(s_d[tid]);          // D^{-1/2}
+    if (tid < M) s_rcp[tid] = 1.0 / sqrt(t.d[tid]);          // D^{-1/2}
     // A <- U^{-1} h, then H' = D^{-1/2} A U^{-dag} D^{-1/2} (lower part, mirrored) into B
     for (int i = warp; i < M; i += NW)
         for (int j = lane; j < M; j += 32) {
@@ -345,135 +480,26 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
             B[j * ld + i] = cconj(x);
         }
     __syncthreads();
-    // Householder reduction: reflector k = 1 - tau v v^dag (v_{k+1} = 1) makes column k (beta, 0, ..)
-    // with real beta; A <- A - v w^dag - w v^dag, w = p - (tau/2) (p^dag v) v, p = tau A v
-    for (int k = 0; k + 1 < M; k++) {
-        if (warp == 0) {
-            double xn = 0.0;
-            for (int i = k + 2 + lane; i < M; i += 32) xn += cabs2(B[i * ld + k]);
-            xn = warp_sum(xn);
-            const cplx al = B[(k + 1) * ld + k];
-            cplx tau = cmk(0.0, 0.0), sc = cmk(0.0, 0.0);
-            double beta = al.x;
-            if (xn > 0.0 || al.y != 0.0) {
-                beta = sqrt(cabs2(al) + xn);
-                if (al.x >= 0.0) beta = -beta;
-                const double rb = 1.0 / beta;
-                tau = cmk((beta - al.x) * rb, -al.y * rb);
-                const cplx q = cmk(al.x - beta, al.y);
-                sc = cscale(cconj(q), 1.0 / cabs2(q));
-            }
-            for (int i = k + 1 + lane; i < M; i += 32) {
-                const cplx v = i == k + 1 ? cmk(1.0, 0.0) : cmul(B[i * ld + k], sc);
-                s_v[i] = v;
-                A[i * ld + k] = v;              // kept for the back transformation
-            }
-            if (lane == 0) { s_tau[k] = tau; s_e[k] = beta; s_e2[k] = beta * beta; }
-        }
-        __syncthreads();
-        // A v: lanes over rows, the columns shared out among the warps
-        for (int i = k + 1 + lane; i < M; i += 32) {
-            cplx p = cmk(0.0, 0.0);
-            for (int j = k + 1 + warp; j < M; j += NW) cfma(p, B[i * ld + j], s_v[j]);
-            s_part[warp][i] = p;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const cplx tau = s_tau[k];
-            double dr = 0.0, di = 0.0;
-            for (int i = k + 1 + lane; i < M; i += 32) {
-                cplx p = s_part[0][i];
-                for (int w = 1; w < NW; w++) p = cadd(p, s_part[w][i]);
-                p = cmul(tau, p);
-                s_w[i] = p;
-                const cplx x = cmul(cconj(p), s_v[i]);
-                dr += x.x;
-                di += x.y;
-            }
-            const cplx f = cscale(cmul(tau, cmk(warp_sum(dr), warp_sum(di))), -0.5);
-            for (int i = k + 1 + lane; i < M; i += 32) {
-                cplx w = s_w[i];
-                cfma(w, f, s_v[i]);
-                s_w[i] = w;
-            }
-        }
-        __syncthreads();
-        for (int i = k + 1 + warp; i < M; i += NW) {
-            const cplx vi = cscale(s_v[i], -1.0), wi = cscale(s_w[i], -1.0);
-            for (int j = k + 1 + lane; j <= i; j += 32) {
-                cplx x = B[i * ld + j];
-                cfma(x, vi, cconj(s_w[j]));
-                cfma(x, wi, cconj(s_v[j]));
-                if (i == j) x.y = 0.0;
-                B[i * ld + j] = x;
-                B[j * ld + i] = cconj(x);
-            }
-        }
-        __syncthreads();
-    }
-    for (int i = tid; i < M; i += AMP_THREADS) s_d[i] = B[i * ld + i].x;
-    __syncthreads();
+    amp_reduce(A, B, M, ld, t);
     if (warp == 0) {
-        // T of extreme magnitude (energies in units far from its own): to order one by a power of two, exact
-        int ex = 0;
-        for (int i = lane; i < M; i += 32) {
-            ex = max(ex, (__double2hiint(s_d[i]) >> 20) & 0x7ff);
-            if (i + 1 < M) ex = max(ex, (__double2hiint(s_e[i]) >> 20) & 0x7ff);
-        }
-        ex = __reduce_max_sync(0xffffffffu, ex);
-        const int f = ex > 0 && (ex < 1023 - 150 || ex > 1023 + 150) ? min(max(2046 - ex, 1), 2045) : 1023;
-        if (f != 1023) {
-            const double sc = __hiloint2double(f << 20, 0);
-            for (int i = lane; i < M; i += 32) {
-                s_d[i] *= sc;
-                if (i + 1 < M) {
-                    s_e[i] *= sc;
-                    s_e2[i] = s_e[i] * s_e[i];
-                }
-            }
-            __syncwarp();
-        }
-        // lo, hi bracket the lowest eigenvalue: Gershgorin below, the smallest diagonal entry above
-        double lo = INFINITY, hi = INFINITY, top = 0.0;
-        bool nan = false;
-        for (int i = lane; i < M; i += 32) {
-            const double r = (i > 0 ? fabs(s_e[i - 1]) : 0.0) + (i + 1 < M ? fabs(s_e[i]) : 0.0);
-            lo = fmin(lo, s_d[i] - r);
-            hi = fmin(hi, s_d[i]);
-            top = fmax(top, fabs(s_d[i]) + r);
-            nan = nan || !isfinite(s_d[i] + r);
-        }
-        nan = __any_sync(0xffffffffu, nan);                  // (fmin and fmax drop a NaN)
-        for (int o = 16; o > 0; o >>= 1) {
-            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = fmin(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-            top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
-        }
+        double lo, hi, top;
+        bool nan;
+        const int f = amp_lowest(t, M, lo, hi, top, nan);
         const double ulp = 2.220446049250313e-16;
-        lo -= 4.0 * ulp * top;
-        for (int it = 0; it < 14 && hi - lo > ulp * fmax(fabs(lo), fabs(hi)); it++) {
-            const double x = fma(hi - lo, (lane + 1) * (1.0 / 33.0), lo);
-            const unsigned pd = __ballot_sync(0xffffffffu, amp_posdef(s_d, s_e2, M, x));
-            const int n = __ffs(~pd) - 1;                    // shifts 0 .. n - 1 lie below (n = -1: all)
-            const double below = __shfl_sync(0xffffffffu, x, n > 0 ? n - 1 : (n < 0 ? 31 : 0));
-            const double above = __shfl_sync(0xffffffffu, x, n < 0 ? 31 : n);
-            if (n != 0) lo = below;
-            if (n >= 0) hi = above;
-        }
         // inverse iteration at a shift just below the eigenvalue, where T - x is positive definite and
         // its factorisation needs no pivoting; each pass cuts the other components by about
         // 16 ulp top / gap
         if (lane == 0) {
             s_E = nan ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (lo + hi) * __hiloint2double((2046 - f) << 20, 0);
             const double x = lo - 16.0 * ulp * top, least = ulp * top + 1e-300;
-            double* q = reinterpret_cast<double*>(s_part);             // 1 / pivots
+            double* q = reinterpret_cast<double*>(t.part);             // 1 / pivots
             double* l = q + MR;                                        // multipliers
             double* z = l + MR;
-            double r = 1.0 / fmax(s_d[0] - x, least);
+            double r = 1.0 / fmax(t.d[0] - x, least);
             q[0] = r;
             for (int i = 1; i < M; i++) {
-                l[i] = s_e[i - 1] * r;
-                r = 1.0 / fmax(fma(-s_e[i - 1], l[i], s_d[i] - x), least);
+                l[i] = t.e[i - 1] * r;
+                r = 1.0 / fmax(fma(-t.e[i - 1], l[i], t.d[i] - x), least);
                 q[i] = r;
             }
             for (int i = 0; i < M; i++) z[i] = 1.0 + 0.125 * (i % 5);
@@ -492,7 +518,7 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
         }
         __syncwarp();
         // y = H_0 H_1 ... H_{M-2} z, then D^{-1/2} y
-        const double* z = reinterpret_cast<double*>(s_part) + 2 * MR;
+        const double* z = reinterpret_cast<double*>(t.part) + 2 * MR;
         cplx y[2];
         for (int u = 0; u < 2; u++) y[u] = cmk(lane + 32 * u < M ? z[lane + 32 * u] : 0.0, 0.0);
         for (int k = M - 2; k >= 0; k--) {
@@ -505,17 +531,17 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
                 dr += x.x;
                 di += x.y;
             }
-            const cplx f = cscale(cmul(s_tau[k], cmk(warp_sum(dr), warp_sum(di))), -1.0);
+            const cplx f = cscale(cmul(t.tau[k], cmk(warp_sum(dr), warp_sum(di))), -1.0);
             for (int u = 0; u < 2; u++) cfma(y[u], f, v[u]);
         }
         for (int u = 0; u < 2; u++)
-            if (lane + 32 * u < M) s_w[lane + 32 * u] = cscale(y[u], s_rcp[lane + 32 * u]);
+            if (lane + 32 * u < M) t.w[lane + 32 * u] = cscale(y[u], s_rcp[lane + 32 * u]);
     }
     __syncthreads();
     // lambda = U^{-dag} D^{-1/2} y
     for (int j = tid; j < M; j += AMP_THREADS) {
         cplx x = cmk(0.0, 0.0);
-        for (int i = j; i < M; i++) cfma(x, cconj(W[i * ld + j]), s_w[i]);
+        for (int i = j; i < M; i++) cfma(x, cconj(W[i * ld + j]), t.w[i]);
         lr[j] = x.x;
         lr[M + j] = x.y;
     }
@@ -534,6 +560,9 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     return !(most - mine > __double2hiint(1.0) - least);
 }
 
+// where in scratch the solve marks its route (1: direct), before the two values of gram_eig_kernel
+__host__ __device__ inline size_t gram_mark(int M) { return 6 * (size_t)(2 * M) * (2 * M) + 2 * M; }
+
 // dynamic shared memory of amp_solve_kernel
 inline size_t amp_smem(int M) { return 3 * (size_t)M * (M + 1) * sizeof(cplx); }
 
@@ -547,13 +576,13 @@ __global__ void __launch_bounds__(AMP_THREADS) amp_solve_kernel(AmpArgs a) {
     const double* h = a.hm;
     double E = 0.0;
     const bool direct = amp_direct(a, reinterpret_cast<cplx*>(amp_sm), lr, E);
+    if (tid == 0) a.scratch[gram_mark(M)] = direct ? 1.0 : 0.0;
     if (direct) {
         amp_embed(G, a.scratch, M);          // for gram_eig_kernel
     } else {
         __syncthreads();
         if (!amp_jacobi(a, lr, E)) return;
     }
-    if (tid == 0) a.scratch[6 * (2 * M) * (2 * M) + 2 * M] = direct ? 1.0 : 0.0;
     // normalisation lambda^dag G lambda = 1 and the phase convention; lambda-tilde = G lambda
     double nrm = 0.0;
     for (int i = warp; i < M; i += AMP_THREADS / 32) {
@@ -609,20 +638,51 @@ __global__ void __launch_bounds__(AMP_THREADS) amp_solve_kernel(AmpArgs a) {
         }
 }
 
-// The eigenvalues of G of the last amplitude solve for the health report: where that solve took the
-// direct route it left the embedding of G in scratch, which is diagonalised here in place
+// dynamic shared memory of gram_eig_kernel
+inline size_t gram_smem(int M) { return (size_t)M * (M + 1) * sizeof(cplx); }
+
+// The smallest and the largest eigenvalue of G of the last amplitude solve, for the health report: after a Jacobi
+// solve they are on its diagonal, after the direct route (which leaves the embedding of G in scratch) they come from
+// the tridiagonal form by multisection, as the energy does.  Jacobi for them took about half of what the direct route
+// saves a step.  They go to scratch behind the route's mark.
 __global__ void __launch_bounds__(AMP_THREADS) gram_eig_kernel(double* scratch, int M) {
-    __shared__ double rc[SGS_MAX_RANK + 1], rs[SGS_MAX_RANK + 1];
-    __shared__ int rp[SGS_MAX_RANK + 1], rq[SGS_MAX_RANK + 1];
-    __shared__ double red[32];
-    const int m = 2 * M;
-    double* flag = scratch + 6 * m * m + 2 * M;
-    if (*flag != 1.0) return;
-    double* V = scratch + m * m;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) V[e] = (e / m == e % m) ? 1.0 : 0.0;
+    extern __shared__ double amp_sm[];
+    __shared__ AmpTri t;
+    cplx* B = reinterpret_cast<cplx*>(amp_sm);
+    const int m = 2 * M, ld = M + 1, tid = threadIdx.x;
+    double* mark = scratch + gram_mark(M);
+    if (*mark != 1.0) {
+        if (tid == 0) {
+            double lo = INFINITY, hi = 0.0;
+            for (int j = 0; j < m; j++) {
+                lo = fmin(lo, scratch[(size_t)j * m + j]);
+                hi = fmax(hi, scratch[(size_t)j * m + j]);
+            }
+            mark[1] = lo;
+            mark[2] = hi;
+        }
+        return;
+    }
+    for (int e = tid; e < M * M; e += AMP_THREADS) {
+        const int i = e / M, j = e % M;
+        B[i * ld + j] = cmk(scratch[(size_t)i * m + j], scratch[(size_t)(i + M) * m + j]);
+    }
     __syncthreads();
-    jacobi_sym(scratch, V, m, m, rc, rs, rp, rq, red);
-    if (threadIdx.x == 0) *flag = 0.0;
+    amp_reduce(nullptr, B, M, ld, t);
+    if (tid < 32) {
+        double lo, hi, top, low;
+        bool nan;
+        amp_lowest(t, M, lo, hi, top, nan);
+        low = 0.5 * (lo + hi);
+        __syncwarp();
+        for (int i = tid; i < M; i += 32) t.d[i] = -t.d[i];         // the largest of T: the lowest of -T
+        __syncwarp();
+        amp_lowest(t, M, lo, hi, top, nan);
+        if (tid == 0) {
+            mark[1] = low;
+            mark[2] = -0.5 * (lo + hi);
+        }
+    }
 }
 
 }  // namespace sgs

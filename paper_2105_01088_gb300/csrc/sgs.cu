@@ -853,6 +853,7 @@ void set_kernel_attributes() {
     raise_smem_limit(renyi_pf_kernel, optin);
     raise_smem_limit(pf_small_kernel, optin);
     raise_smem_limit(amp_solve_kernel, optin);
+    raise_smem_limit(gram_eig_kernel, optin);
     raise_smem_limit(gemm_tma_kernel<TC_TF32>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_BF16>, optin);
     raise_smem_limit(gemm_tma_kernel<TC_3XTF32>, optin);
@@ -2046,7 +2047,7 @@ sgs_status sgs_health(sgs_ctx* c, int instance, double* out) {
     cudaStream_t st = c->stream;
     CUDA_TRY(c, cudaStreamSynchronize(st));
     // Gamma_mu^2 -> s0, then max |Gamma^2 + 1|, non-finite entries of Gamma, and the extreme eigenvalues of G
-    // of the last amplitude solve (the diagonal of a Jacobi result: that solve's, or gram_eig_kernel's)
+    // of the last amplitude solve (gram_eig_kernel)
     GemmBatch g = gb_basic(n, n, n, I.p_gamma, n, I.p_gamma, n, I.p_s[0], n, M);
     const bool prof = c->prof;
     c->prof = false;
@@ -2060,9 +2061,11 @@ sgs_status sgs_health(sgs_ctx* c, int instance, double* out) {
         if (!I.corr_scratch) { c->err = "device allocation failed"; return SGS_ENOMEM; }
         I.corr_cap = 8;
     }
-    gram_eig_kernel<<<1, AMP_THREADS, 0, st>>>(I.eigscratch, M);
+    set_kernel_attributes();
+    gram_eig_kernel<<<1, AMP_THREADS, gram_smem(M), st>>>(I.eigscratch, M);
     counted();
-    health_kernel<<<1, 1024, 0, st>>>(I.s[0], I.gamma, M * nn, n, I.eigscratch, 2 * M, I.Ecur, I.corr_scratch);
+    health_kernel<<<1, 1024, 0, st>>>(I.s[0], I.gamma, M * nn, n, I.eigscratch + gram_mark(M) + 1, I.Ecur,
+                                      I.corr_scratch);
     counted();
     CUDA_TRY(c, cudaMemcpyAsync(out, I.corr_scratch, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(c, cudaStreamSynchronize(st));

@@ -112,10 +112,10 @@ __global__ void __launch_bounds__(256) exp_scale_kernel(double* X, double* X2, d
 
 // health of an instance: out[0] = max |(Gamma^2)_kl + delta_kl| over the states (G2 holds
 // Gamma^2), out[1] = number of non-finite entries of Gamma, out[2] = smallest / largest
-// eigenvalue of G at the last amplitude solve (the diagonal of its Jacobi result, m x m
-// real embedding), out[3] = the energy of that solve
+// eigenvalue of G at the last amplitude solve (gram: the two, from gram_eig_kernel), out[3] =
+// the energy of that solve
 __global__ void __launch_bounds__(1024) health_kernel(const double* G2, const double* gamma, size_t count, int n,
-                                                       const double* eig, int m, const double* E, double* out) {
+                                                       const double* gram, const double* E, double* out) {
     __shared__ double red[32];
     double worst = 0.0, bad = 0.0;
     const size_t nn = (size_t)n * n;
@@ -134,15 +134,9 @@ __global__ void __launch_bounds__(1024) health_kernel(const double* G2, const do
     if (threadIdx.x == 0) {
         double mx = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) mx = fmax(mx, wmax[w]);
-        double lo = INFINITY, hi = 0.0;
-        for (int j = 0; j < m; j++) {
-            const double v = eig[(size_t)j * m + j];
-            lo = fmin(lo, v);
-            hi = fmax(hi, v);
-        }
         out[0] = mx;
         out[1] = bad;
-        out[2] = hi > 0.0 ? lo / hi : 0.0;
+        out[2] = gram[1] > 0.0 ? gram[0] / gram[1] : 0.0;
         out[3] = E[0];
     }
 }
