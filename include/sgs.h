@@ -203,7 +203,8 @@ int sgs_failed_instances(const sgs_ctx* ctx, int* slots, int capacity);
  * and of the blocked complex Pfaffian (8, 12, 16, 24, 32 column pairs) on the new
  * instance's own pairs,
  * with CUDA events, and keeps the fastest.  Choices are cached per (n, rank,
- * precision) for the process, so a shape is timed once; the scratch of tuned
+ * precision, pairs of a launch: all, a chunk or a rank's share) for the process,
+ * so a shape is timed once; the scratch of tuned
  * instances is sized for the widest candidate.  Widths change results only
  * by rounding.  Default: off (fixed widths). */
 sgs_status sgs_set_autotune(sgs_ctx* ctx, int enable);

@@ -1293,14 +1293,16 @@ __global__ void shard_export_gh_kernel(const double* Gm, const double* hm, int M
 // ------------------------------------------------------------------ autotuning
 
 std::mutex g_tune_mu;
-std::map<std::array<int, 3>, std::array<int, 2>> g_tune_cache;   // (n, rank, precision) -> widths
+// (n, rank, precision, pairs and phase Pfaffians a launch holds, chunks) -> widths: the kernels' forms depend on the
+// number of matrices, which a chunked or pair-sharded instance of the same shape has fewer of
+std::map<std::array<int, 6>, std::array<int, 2>> g_tune_cache;
 
 // Time the candidate widths on the instance's own pairs (CUDA events on the context
 // stream, best of two), keep the fastest; a shape already timed in this process reuses
 // its widths.  Results change only by rounding.
 sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     if (I.P == 0) return SGS_OK;
-    const std::array<int, 3> key{I.n, I.M, I.prec};
+    const std::array<int, 6> key{I.n, I.M, I.prec, I.Pc, I.Ppfc, I.nch()};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -1337,10 +1339,8 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     };
     int gj = I.gj_b, pf = I.pf_bs;
     float best = 1e30f;
-    const std::vector<int> gjc = gj_candidates(I.n);
-    const bool extra = std::find(gjc.begin(), gjc.end(), I.gj_def) == gjc.end();    // a width of the cluster form only
-    std::vector<int> tried = gjc;
-    if (extra) tried.push_back(I.gj_def);
+    std::vector<int> tried = gj_candidates(I.n);
+    if (std::find(tried.begin(), tried.end(), I.gj_def) == tried.end()) tried.push_back(I.gj_def);   // cluster form only
     for (int b : tried) {
         if (b > I.gj_cap && b != I.gj_def) continue;
         if ((status = set_panel_pointers(c, I, b, pf)) != SGS_OK) break;
@@ -1369,7 +1369,7 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     CUDA_TRY(c, cudaMemsetAsync(I.err, 0, sizeof(int), st));      // trial runs leave no error state
     CUDA_TRY(c, cudaStreamSynchronize(st));
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    if (!(extra && gj == I.gj_def)) g_tune_cache[key] = {gj, pf};      // that width depends on the number of pairs
+    g_tune_cache[key] = {gj, pf};
     I.tuned_from_cache = 0;
     return SGS_OK;
 }
