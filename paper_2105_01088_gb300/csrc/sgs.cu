@@ -1347,6 +1347,9 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
         const float t = timed([&] { return cudaSuccess; }, [&] { return pair_inverse(c, I, st); });
         if (t < best) { best = t; gj = b; }
     }
+    // the chunk with the most phase Pfaffians (the first pairs, those of state 0, have none)
+    for (int ch = 0; ch < I.nch(); ch++)
+        if (I.ch_pfcnt[ch] > I.cpfcnt()) I.cur = ch;
     if (status == SGS_OK && I.Ppf > 0) {
         status = set_panel_pointers(c, I, gj, pf);
         cudaError_t e = cudaSuccess;
@@ -1361,6 +1364,7 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
             if (t < best) { best = t; pf = b; }
         }
     }
+    I.cur = 0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->prof = prof;

@@ -38,3 +38,16 @@ def test_fewer_pairs_are_timed_on_their_own():
     assert s.tuning(s.admit(model, g, shard=(0, 2)))[2] == 0
     assert s.tuning(s.admit(model, g, pair_chunk=7))[2] == 1
     s.close()
+
+
+@pytest.mark.parametrize("n_bath,chunk", [(16, 5), (30, 3)])     # n = 68 and 124: the chunk of state 0's pairs first
+def test_chunks_without_phase_pfaffians(n_bath, chunk):
+    model = sgs.build_anderson(n_bath, 2.0, -1.0, 0.5)
+    g = states(model, 6)
+    s = sgs.Solver(model, g, None, autotune=True, pair_chunk=chunk)
+    E = s.energy()
+    s.close()
+    s = sgs.Solver(model, g, None)
+    # other panel widths: rounding of well-conditioned (G, h)
+    assert np.abs(s.energy() - E).max() <= 1e-10 * np.abs(E).max()
+    s.close()
