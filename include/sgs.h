@@ -200,9 +200,9 @@ int sgs_failed_instances(const sgs_ctx* ctx, int* slots, int capacity);
 /* Autotuning of the factorisation tile shapes.  With enable = 1, sgs_admit
  * (and sgs_add_state) times the candidate panel widths of the blocked
  * Gauss-Jordan inverse (leaf panels of 8, 12, 16, 20, 24, 32, 48, 64 columns, as shared memory allows)
- * and of the blocked complex Pfaffian (8, 12, 16, 24, 32 column pairs) on the new
- * instance's own pairs,
- * with CUDA events, and keeps the fastest.  Choices are cached per (n, rank,
+ * and of the blocked complex Pfaffian (8, 12, 16, 24, 32 column pairs; not where each
+ * Pfaffian runs in one CTA's shared memory, up to 2N = 152, and has no panels) on the new
+ * instance's own pairs, with CUDA events, and keeps the fastest.  Choices are cached per (n, rank,
  * precision, pairs of a launch: all, a chunk or a rank's share) for the process,
  * so a shape is timed once; the scratch of tuned
  * instances is sized for the widest candidate.  Widths change results only

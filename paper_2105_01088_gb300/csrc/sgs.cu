@@ -1347,10 +1347,11 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
         const float t = timed([&] { return cudaSuccess; }, [&] { return pair_inverse(c, I, st); });
         if (t < best) { best = t; gj = b; }
     }
-    // the chunk with the most phase Pfaffians (the first pairs, those of state 0, have none)
+    // the chunk with the most phase Pfaffians (the first pairs, those of state 0, have none); where a CTA takes
+    // each (pf_small) there is no panel, and the width stays as admitted
     for (int ch = 0; ch < I.nch(); ch++)
         if (I.ch_pfcnt[ch] > I.cpfcnt()) I.cur = ch;
-    if (status == SGS_OK && I.Ppf > 0) {
+    if (status == SGS_OK && I.Ppf > 0 && !pf_small(I.n, I.cpfcnt())) {
         status = set_panel_pointers(c, I, gj, pf);
         cudaError_t e = cudaSuccess;
         if (status == SGS_OK) e = pair_inverse(c, I, st);

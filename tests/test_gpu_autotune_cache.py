@@ -51,3 +51,18 @@ def test_chunks_without_phase_pfaffians(n_bath, chunk):
     # other panel widths: rounding of well-conditioned (G, h)
     assert np.abs(s.energy() - E).max() <= 1e-10 * np.abs(E).max()
     s.close()
+
+
+@pytest.mark.parametrize("n_bath,M", [(7, 3), (9, 4), (15, 4), (21, 5), (26, 6)])       # n = 32 .. 108
+def test_no_width_is_chosen_where_there_is_no_panel(n_bath, M):
+    """Phase Pfaffians of a CTA each: the tuner leaves the width as a solver without tuning has it (timing them told
+    five widths of one kernel apart by noise)."""
+    model = sgs.build_anderson(n_bath, 2.0, -1.0, 0.5)
+    g = states(model, M)
+    s = sgs.Solver(model, g, None)
+    want = s.tuning(0)[1]
+    s.close()
+    for chunk in (0, 2):
+        s = sgs.Solver(model, g, None, autotune=True, pair_chunk=chunk)
+        assert s.tuning(0)[1] == want
+        s.close()
