@@ -153,7 +153,7 @@ __device__ __forceinline__ void gj_panel_copy(double* W, double* panel, int n, i
 __device__ void gj_panel_finish(const GJPanelArgs& a, double* W, int b, double* stage, int cap, const int* s_rows,
                                 const int* s_src, int nr, int c0, int c1) {
     const int n = a.n, k0 = a.k0, bb = a.bb;
-    // a warp per row, lanes along the columns, eight loads in flight per lane
+    // a warp per row, lanes along the columns, four loads in flight per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (nr > 0) {
         const int qc = min(c1 - c0, cap / nr);
@@ -161,14 +161,14 @@ __device__ void gj_panel_finish(const GJPanelArgs& a, double* W, int b, double* 
             const int qn = min(qc, c1 - q0);
             for (int e = warp; e < nr; e += nw) {
                 const double* src = W + (size_t)s_src[e] * n + q0;
-#pragma unroll 8
+#pragma unroll 4
                 for (int x = lane; x < qn; x += 32)
                     if ((unsigned)(q0 + x - k0) >= (unsigned)bb) stage[e * qn + x] = src[x];
             }
             __syncthreads();
             for (int e = warp; e < nr; e += nw) {
                 double* dst = W + (size_t)s_rows[e] * n + q0;
-#pragma unroll 8
+#pragma unroll 4
                 for (int x = lane; x < qn; x += 32)
                     if ((unsigned)(q0 + x - k0) >= (unsigned)bb) dst[x] = stage[e * qn + x];
             }
@@ -196,7 +196,9 @@ __device__ __forceinline__ void warp_argmax(long long& key, int& idx) {
     key = (long long)(((unsigned long long)mh << 32) | ml) - 1;
 }
 
-__global__ void __launch_bounds__(512) gj_panel_kernel(GJPanelArgs a) {
+// One CTA per matrix, for batches that fill the SMs.  Four CTAs fit an SM (32 registers a thread), so that up to 608
+// matrices are one wave: at two (56 registers) 400 inverses of 64 x 64 took 767 us, at four 602.
+__global__ void __launch_bounds__(512, 4) gj_panel_kernel(GJPanelArgs a) {
     extern __shared__ double sm[];
     const int ps = a.bb + 1;                   // odd row stride: column walks hit distinct banks
     double* panel = sm;                        // n x ps
