@@ -393,23 +393,32 @@ std::vector<int> gj_candidates(int n) {
     return v;
 }
 int gj_cluster(int n, int batch, int bb);
-// leaf of the recursive form: 16 columns, or the widest candidate below it whose panel fits one CTA's shared memory
-// (n above about 1700).  In FP64, by the panels' cluster form for `batch` matrices:
-//   * 16 at those n too.  One step, leaf 12 / 16, ms: n = 2000, 28 pairs 151.1 / 142.7; 2000, 6: 61.9 / 59.0;
-//   * 32 where a CTA has at most 128 rows: half the panels and a level of updates less.  Leaf 16 / 32, us: n = 164,
-//     15 pairs 1438 / 1393 (energy); 164, 120: 3774 / 3667; 244, 120: 5740 / 5583; 388, 45: 6350 / 6225; 400, 66:
-//     10508 / 10213; 512, 28: 8711 / 8479; but 512, 120 (256 rows a CTA): 20361 / 20657; 800, 6: 12391 / 12463; 512,
-//     496 (no clusters): 68825 / 73030.
+// Leaf of the recursive form: 16 columns, or the widest candidate below it whose panel fits one CTA's shared memory
+// (n above about 1700).  In FP64, where few pairs leave the panels to clusters of CTAs:
+//   * 16 at those n too, up to 256 pairs (and where the cluster form holds such a panel: it does for every smaller
+//     batch as well).  One step, leaf 12 / 16, ms: n = 2000, 28 pairs 151.1 / 142.7; 2000, 6: 61.9 / 59.0;
+//   * 32 where the panels' time is mostly their columns' latency: half the panels and a level of updates less.  The
+//     line is where the two leaves take the same time.  One step, leaf 16 / 32, us, by pairs:
+//       n      15            45             78             120            171            210            253
+//       64     572 / 552     885 / 864      1072 / 1050    1170 / 1140    1293 / 1276    1365 / 1345    1483 / 1466
+//       100    1188 / 1165   1389 / 1354    1602 / 1559    1704 / 1679    1919 / 1899    2067 / 2049    2222 / 2232
+//       164    1832 / 1830   2456 / 2418    3012 / 2904    3675 / 3595    4585 / 4575    5045 / 4975    5620 / 5555
+//       200    2237 / 2205   2891 / 2829    3693 / 3601    4723 / 4655    5600 / 5587    6368 / 6328    7382 / 7481
+//       256    2558 / 2579   3552 / 3432    4460 / 4309    5550 / 5445    7006 / 7016    7867 / 7905    9245 / 9244
+//       300    3512 / 3495   5027 / 4809    6704 / 6531    8690 / 8653
+//       400    4973 / 5048   7756 / 7592    10700 / 10521  13566 / 13563
+//       512    6717 / 6583   10507 / 10073  13935 / 13816  18961 / 19278
+//     up to 256 pairs at n <= 256, up to 80 at n <= 512; n = 800, 6 pairs: 12391 / 12463.
+// The pairs are those of a chunk, all of them where a step is not chunked (it inverts them in two halves).
 // The mixed forms keep the first: their rounding to tf32 makes a change of S^{-1}'s last bits visible.
-int default_gj_width(int n, int batch, int prec) {
+int default_gj_width(int n, int pairs, int prec) {
     int w = std::min(8, n);
     for (int b : gj_candidates(n))
         if (b <= 16) w = std::max(w, b);
     w = std::min(w, n);
-    if (prec != SGS_FP64 || batch < 1) return w;
-    if (n >= 16 && w < 16 && gj_cluster(n, batch, 16) > 0) return 16;
-    const int C = gj_cluster(n, batch, 32);
-    return n >= 64 && n <= 512 && C > 0 && (n + C - 1) / C <= 128 ? 32 : w;
+    if (prec != SGS_FP64 || pairs < 1) return w;
+    if (n >= 16 && w < 16 && pairs <= 256 && gj_cluster(n, pairs, 16) > 0) return 16;
+    return n >= 64 && pairs <= (n <= 256 ? 256 : n <= 512 ? 80 : 0) ? 32 : w;
 }
 std::vector<int> pf_candidates(int n) {
     std::vector<int> v;
