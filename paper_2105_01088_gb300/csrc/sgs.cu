@@ -907,12 +907,17 @@ int threads_per_row(int ch) {             // the power's exponent
 // below a few hundred matrices and pays one SM's FP64 pipe per column; more CTAs than SMs (152) only
 // share them.  Panels of 16 columns, one-CTA form against the best C, us: n = 64, 6 matrices 53 / 32
 // (C = 8); n = 164, 15: 59 / 36 (8); n = 244, 60: 65 / 47 (4); n = 388, 45: 90 / 53 (8); n = 804, 60:
-// 151 / 90 (4, 8); n = 2000, 14 (12 columns): 237 / 61 (8).  Pairs of CTAs pay up to about 256 matrices (1.6 matrices
-// per SM leave some SMs twice the work of others).  One step, one-CTA form / pairs, us: n = 512, 248 matrices in each half 65310
-// / 64520; 244, 126: 9400 / 9320; 164, 248: 9750 / 9560.  Four or eight CTAs beyond 320 in all lost: n = 244, 60: 5470 / 5590.
+// 151 / 90 (4, 8); n = 2000, 14 (12 columns): 237 / 61 (8).  Four or eight CTAs beyond 320 in all lost: a step at
+// n = 244, 60 matrices in each half, 5470 / 5590.  Pairs of CTAs: a step with one CTA / pairs, us, by matrices in each half:
+//   n      138             163             233             264             298             352             473
+//   64     1508 / 1505     1670 / 1611     1931 / 1888     2113 / 2091     2217 / 2217     2570 / 2476     3115 / 3069
+//   164    6227 / 6212     7238 / 6983     9074 / 8976     9927 / 9856     10716 / 10696   13003 / 12877   16365 / 16472
+//   244    9974 / 9844     11329 / 10901   14795 / 14431   16316 / 16098   17612 / 17548   21400 / 21118   27148 / 27213
+//   512    38722 / 38610   44121 / 43996   59263 / 59060   67382 / 66894   74557 / 74112   87769 / 88262   114787 / 115469
+// They cross at 300 to 420 matrices, the sooner the larger n; the line is at 320.  Both forms give the same bits.
 int gj_cluster(int n, int batch, int bb) {
     for (int C = 8; C >= 2; C /= 2)
-        if (batch * C <= (C == 2 ? 512 : 320) && n >= 8 * C && gjc_smem(bb, C, (n + C - 1) / C) <= 200 * 1024) return C;
+        if (batch * C <= (C == 2 ? 640 : 320) && n >= 8 * C && gjc_smem(bb, C, (n + C - 1) / C) <= 200 * 1024) return C;
     return 0;
 }
 // 16 steps on `live` rows, one-CTA form against the best C, us: 64 rows, 3 matrices 153 / 80 (4); 164, 10:
