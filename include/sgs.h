@@ -215,10 +215,12 @@ sgs_status sgs_set_autotune(sgs_ctx* ctx, int enable);
 sgs_status sgs_get_tuning(const sgs_ctx* ctx, int instance, int* gj_width, int* pf_width, int* from_cache);
 
 /* Fix the panel widths of a live instance (for reproducible timings and
- * profiles): each must be one of the autotuner's candidates and fit the
- * instance's scratch (an instance admitted with autotuning on has room for
- * the widest), or the width the instance was admitted with.  Waits for the context's stream; drops a captured step graph.
- * SGS_EINVAL otherwise. */
+ * profiles): each must be one of the autotuner's candidates and no wider than
+ * the instance was admitted for (with autotuning on, the widest), or the width
+ * the instance was admitted with.  Where each phase Pfaffian runs in one CTA's
+ * shared memory (some batches up to 2N = 152) the second width has no effect.
+ * Waits for the context's stream; drops a captured step graph.  SGS_EINVAL
+ * otherwise. */
 sgs_status sgs_set_panel_widths(sgs_ctx* ctx, int instance, int gj_width, int pf_width);
 
 /* Rank growth (Sec. III C): append to the live instance `slot` the state

@@ -108,7 +108,6 @@ struct Instance {
     int *imp = nullptr, *slot = nullptr;
 
     double *work = nullptr, *si = nullptr, *imd = nullptr, *wr = nullptr, *va = nullptr, *xa = nullptr;
-    double* tbuf = nullptr;
     int *piv = nullptr, *perm = nullptr;
     double *logdet = nullptr, *dsign = nullptr;
     double *pfTU = nullptr, *pfpack = nullptr, *pflog = nullptr, *pfphase = nullptr;
@@ -160,7 +159,7 @@ struct Instance {
 
     // pointer arrays (device)
     double **p_tup = nullptr;           // recursive Gauss-Jordan: pivot rows of an update (second half of work)
-    double **p_work = nullptr, **p_tbuf = nullptr, **p_si = nullptr, **p_imd = nullptr, **p_wr = nullptr,
+    double **p_work = nullptr, **p_si = nullptr, **p_imd = nullptr, **p_wr = nullptr,
            **p_va = nullptr, **p_xa = nullptr, **p_ga = nullptr, **p_gb = nullptr;
     double **p_Y = nullptr, **p_TU = nullptr, **p_pack = nullptr;
     double **p_upA = nullptr, **p_upB = nullptr, **p_upC = nullptr;   // Pfaffian update (2 Ppf)
@@ -360,9 +359,9 @@ size_t oz_scratch_bytes(int n, int M, size_t cap, size_t pair_cap) {
 size_t instance_bytes(int n, int M, int prec, int nimp, bool tune, int fp64_path, size_t oz_cap, int pair_chunk) {
     const size_t Pall = (size_t)M * (M - 1) / 2;
     const size_t nn = (size_t)n * n, P = pair_chunk > 0 ? std::min<size_t>(Pall, pair_chunk) : Pall, Ppf = P;
-    const size_t gj_b = tune ? 64 : 32, bs = tune ? 32 : 16;
+    const size_t bs = tune ? 32 : 16;
     const size_t ni = std::max(nimp, 1);
-    size_t d = 7 * (size_t)M * nn + std::max<size_t>(P, 1) * nn * 7 + P * gj_b * n + Ppf * 20 * n * bs +
+    size_t d = 7 * (size_t)M * nn + std::max<size_t>(P, 1) * nn * 7 + Ppf * 20 * n * bs +
                P * ni * ni * 2 + P * 2 * n * ni + 6 * (size_t)(2 * M) * (2 * M) + 16 * (size_t)M * M;
     size_t bytes = 8 * d + 8 * P * n;   // + pivots and permutations
     if (prec != SGS_FP64 && P > 0) {
@@ -429,19 +428,15 @@ std::vector<int> pf_candidates(int n) {
 
 int default_pf_width(int n) { return (2 * 16 > n) ? n / 2 : 16; }
 
-// Pointer arrays of the Gauss-Jordan panel rows and the Pfaffian panel vectors and
-// packed update operands for panel widths (gj_b, pf_bs); the scratch they point into is
-// sized for the widest candidate the instance may use.
+// Panel widths (gj_b, pf_bs) and the pointer arrays of the Pfaffian panel vectors and packed update
+// operands for them; the scratch they point into is sized for the widest candidate the instance may use.
 sgs_status set_panel_pointers(sgs_ctx* c, Instance& I, int gj_b, int pf_bs) {
-    const int n = I.n, P = I.Pc, Ppf = I.Ppfc;    // one chunk of pairs
+    const int n = I.n, Ppf = I.Ppfc;              // one chunk of pairs
     const size_t nn = (size_t)n * n;
     I.gj_b = gj_b;
     I.pf_bs = pf_bs;
     Instance* prev = c->owner;          // allocations belong to the instance
     c->owner = &I;
-    std::vector<double*> t;
-    for (int p = 0; p < P; p++) t.push_back(I.tbuf + (size_t)p * gj_b * n);
-    if (P > 0 && !(I.p_tbuf = upload_ptrs(c, t))) { c->owner = prev; return SGS_ENOMEM; }
     std::vector<double*> Y, TU, PK, upA, upB, upC;
     const size_t blk = (size_t)n * 4 * pf_bs;
     for (int q = 0; q < Ppf; q++) {
@@ -485,7 +480,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
     I.pf_bs = default_pf_width(n);
     I.gj_cap = default_gj_width(n, 0, I.prec);
     I.pf_cap = I.pf_bs;
-    if (c->autotune) {          // scratch for the widest candidate
+    if (c->autotune) {          // every candidate; scratch for the widest Pfaffian panel
         for (int b : gj_candidates(n)) I.gj_cap = std::max(I.gj_cap, b);
         for (int b : pf_candidates(n)) I.pf_cap = std::max(I.pf_cap, b);
     }
@@ -640,7 +635,6 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
     I.work = c->alloc<double>(Pcm * 2 * nn);
     I.si = c->alloc<double>(Pcm * nn); I.imd = c->alloc<double>(Pcm * nn);
     I.wr = c->alloc<double>(Pcm * nn); I.va = c->alloc<double>(Pcm * nn); I.xa = c->alloc<double>(Pcm * nn);
-    I.tbuf = c->alloc<double>(Pcm * std::max(I.gj_cap, I.gj_def) * n);
     I.piv = c->alloc<int>(Pcm * n); I.perm = c->alloc<int>(Pcm * n);
     I.logdet = c->alloc<double>(Pcm); I.dsign = c->alloc<double>(Pcm);
     I.pfTU = c->alloc<double>(Pfc * 4 * n * I.pf_cap);
@@ -666,7 +660,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
         for (int mu = 0; mu < M; mu++) mask[mu] = (mu % I.shard_world == I.shard_rank) ? 1 : 0;
         CUDA_TRY(c, cudaMemcpyAsync(I.self_mask, mask.data(), M * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     }
-    void* check[] = {I.gamma, I.dgamma, I.work, I.si, I.imd, I.wr, I.va, I.xa, I.tbuf, I.pfTU, I.pfpack, I.s[0],
+    void* check[] = {I.gamma, I.dgamma, I.work, I.si, I.imd, I.wr, I.va, I.xa, I.pfTU, I.pfpack, I.s[0],
                      I.s[1], I.s[2], I.s[3], I.s[4], I.eigscratch, I.err, I.lr, I.fimp};
     for (void* p : check)
         if (!p) { c->err = "device allocation failed"; return SGS_ENOMEM; }
@@ -1098,7 +1092,7 @@ cudaError_t gj_update(sgs_ctx* c, int n, int batch, double** W, double** Tup, in
 // (the panels apply them to every other column); their update by this range is the caller's.
 // Every level updates n x n / 2 elements per matrix, about log2(n / leaf) levels in all,
 // against n / leaf full n x n updates of the one-level blocked form.
-cudaError_t gj_recurse(sgs_ctx* c, int n, int batch, int leaf, int c0, int c1, double** W, double** T, double** Tup,
+cudaError_t gj_recurse(sgs_ctx* c, int n, int batch, int leaf, int c0, int c1, double** W, double** Tup,
                        int* piv, double* logdet, double* dsign, int* err, double tiny, cudaStream_t st,
                        const OzBuf* oz) {
     if (c1 - c0 <= leaf) {
@@ -1107,19 +1101,19 @@ cudaError_t gj_recurse(sgs_ctx* c, int n, int batch, int leaf, int c0, int c1, d
     }
     const int leaves = (c1 - c0 + leaf - 1) / leaf;
     const int m = c0 + ((leaves + 1) / 2) * leaf;
-    cudaError_t e = gj_recurse(c, n, batch, leaf, c0, m, W, T, Tup, piv, logdet, dsign, err, tiny, st, oz);
+    cudaError_t e = gj_recurse(c, n, batch, leaf, c0, m, W, Tup, piv, logdet, dsign, err, tiny, st, oz);
     if (e == cudaSuccess) e = gj_update(c, n, batch, W, Tup, c0, m - c0, m, c1 - m, st, oz, err);
-    if (e == cudaSuccess) e = gj_recurse(c, n, batch, leaf, m, c1, W, T, Tup, piv, logdet, dsign, err, tiny, st, oz);
+    if (e == cudaSuccess) e = gj_recurse(c, n, batch, leaf, m, c1, W, Tup, piv, logdet, dsign, err, tiny, st, oz);
     if (e == cudaSuccess) e = gj_update(c, n, batch, W, Tup, m, c1 - m, c0, m - c0, st, oz, err);
     return e;
 }
 
 // S^{-1} in place in W by the recursive form; Tup: per matrix n * n / 4 doubles of scratch
-cudaError_t launch_gj_recursive(sgs_ctx* c, int n, int batch, int leaf, double** W, double** T, double** Tup,
+cudaError_t launch_gj_recursive(sgs_ctx* c, int n, int batch, int leaf, double** W, double** Tup,
                                 int* piv, double* logdet, double* dsign, int* err, double tiny, cudaStream_t st,
                                 const OzBuf* oz) {
     set_kernel_attributes();
-    return gj_recurse(c, n, batch, leaf, 0, n, W, T, Tup, piv, logdet, dsign, err, tiny, st, oz);
+    return gj_recurse(c, n, batch, leaf, 0, n, W, Tup, piv, logdet, dsign, err, tiny, st, oz);
 }
 
 // upA, upB, upC: 2 batch entries, 2 b and 2 b + 1 the real and imaginary parts of matrix b's update
@@ -1167,7 +1161,7 @@ cudaError_t launch_pf(sgs_ctx* c, int n, int batch, int bsmax, double** Y, doubl
 cudaError_t inverse_range(sgs_ctx* c, Instance& I, int p0, int cnt, cudaStream_t st, const OzBuf* oz) {
     const int n = I.n;
     const size_t nn = (size_t)n * n, po = (size_t)p0 * n;
-    cudaError_t e = launch_gj_recursive(c, n, cnt, I.gj_b, I.p_work + p0, I.p_tbuf + p0, I.p_tup + p0, I.piv + po,
+    cudaError_t e = launch_gj_recursive(c, n, cnt, I.gj_b, I.p_work + p0, I.p_tup + p0, I.piv + po,
                                         I.logdet + p0, I.dsign + p0, I.err, 1e-12, st, oz);
     if (e != cudaSuccess) return e;
     gj_perm_kernel<<<cnt, 128, 2 * (size_t)n * sizeof(int), st>>>(I.piv + po, I.perm + po, n, cnt);
@@ -2118,7 +2112,7 @@ sgs_status sgs_set_panel_widths(sgs_ctx* c, int instance, int gj_width, int pf_w
     const std::vector<int> gj = gj_candidates(I.n), pf = pf_candidates(I.n);
     if ((gj_width != I.gj_def && (std::find(gj.begin(), gj.end(), gj_width) == gj.end() || gj_width > I.gj_cap)) ||
         std::find(pf.begin(), pf.end(), pf_width) == pf.end() || pf_width > I.pf_cap) {
-        c->err = "panel width not a candidate, or wider than the instance's scratch";
+        c->err = "panel width not a candidate, or wider than the instance was admitted for";
         return SGS_EINVAL;
     }
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -2992,24 +2986,23 @@ sgs_status sgs_kernel_inverse(const double* S, int n, int batch, int fp64_path, 
     const size_t nn = (size_t)n * n;
     const int bsz = (n <= 640) ? std::min(32, n) : 16;
     const size_t qn = (size_t)n * n / 4 + n;             // recursive form: pivot rows of the widest update
-    double *W = tmp.alloc<double>(batch * nn), *O = tmp.alloc<double>(batch * nn), *T = tmp.alloc<double>((size_t)batch * bsz * n);
+    double *W = tmp.alloc<double>(batch * nn), *O = tmp.alloc<double>(batch * nn);
     double* U = tmp.alloc<double>(batch * qn);
     int *piv = tmp.alloc<int>((size_t)batch * n), *perm = tmp.alloc<int>((size_t)batch * n), *err = tmp.alloc<int>(1);
     double *ld = tmp.alloc<double>(batch), *ds = tmp.alloc<double>(batch);
     sgs_status st = SGS_OK;
-    if (!W || !O || !T || !U || !piv || !perm || !err || !ld || !ds) st = SGS_ENOMEM;
+    if (!W || !O || !U || !piv || !perm || !err || !ld || !ds) st = SGS_ENOMEM;
     if (st == SGS_OK) {
-        std::vector<double*> pw, pt, po, pu;
+        std::vector<double*> pw, po, pu;
         for (int b = 0; b < batch; b++) {
-            pw.push_back(W + b * nn); pt.push_back(T + (size_t)b * bsz * n); po.push_back(O + b * nn);
-            pu.push_back(U + b * qn);
+            pw.push_back(W + b * nn); po.push_back(O + b * nn); pu.push_back(U + b * qn);
         }
-        double **PW = upload_ptrs(&tmp, pw), **PT = upload_ptrs(&tmp, pt), **PO = upload_ptrs(&tmp, po);
+        double **PW = upload_ptrs(&tmp, pw), **PO = upload_ptrs(&tmp, po);
         double** PU = upload_ptrs(&tmp, pu);
         cudaMemcpyAsync(W, S, batch * nn * sizeof(double), cudaMemcpyHostToDevice, tmp.stream);
         cudaMemsetAsync(err, 0, sizeof(int), tmp.stream);
         const OzBuf oz = tmp_oz(tmp, (size_t)batch * oz_entry_bytes(n, n, std::min(n, n / 2 + bsz)), fp64_path, 0);
-        if (launch_gj_recursive(nullptr, n, batch, bsz, PW, PT, PU, piv, ld, ds, err, 0.0, tmp.stream, &oz) !=
+        if (launch_gj_recursive(nullptr, n, batch, bsz, PW, PU, piv, ld, ds, err, 0.0, tmp.stream, &oz) !=
             cudaSuccess)
             st = SGS_ECUDA;
         gj_perm_kernel<<<batch, 128, 2 * (size_t)n * sizeof(int), tmp.stream>>>(piv, perm, n, batch);
