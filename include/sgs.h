@@ -407,7 +407,9 @@ sgs_status sgs_probe_wait(unsigned long long limit_ns, double* elapsed_ms);
  * so does this call.  For kernel i < n_out (0 Gauss-Jordan panel, 1 Pfaffian
  * panel, 2 Renyi Pfaffian, 3-5 tensor-core product tf32 / bf16 / 3xtf32,
  * 6 emulated FP64 product, 7 block slicer, 8 emulated FP64 product of
- * 16-column tiles; n_out <= 9) it writes the limit
+ * 16-column tiles, 9 Gauss-Jordan panel and 10 Pfaffian panel by clusters,
+ * 11 phase Pfaffian in one CTA, 12 amplitude solve, 13 Gram eigenvalues,
+ * 14 emulated FP64 product of 64-column tiles; n_out <= 15) it writes the limit
  * in force to limit[i] and the device's opt-in maximum less the kernel's
  * static shared memory to expected[i]. */
 sgs_status sgs_kernel_smem_limits(int n_out, int* limit, int* expected);

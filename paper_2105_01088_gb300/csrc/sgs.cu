@@ -2685,7 +2685,9 @@ sgs_status sgs_kernel_smem_limits(int n_out, int* limit, int* expected) {
     const void* k[] = {(const void*)gj_panel_kernel, (const void*)pf_panel_kernel, (const void*)renyi_pf_kernel,
                        (const void*)gemm_tma_kernel<TC_TF32>, (const void*)gemm_tma_kernel<TC_BF16>,
                        (const void*)gemm_tma_kernel<TC_3XTF32>, (const void*)oz_gemm_kernel<OZ_NARROW>,
-                       (const void*)oz_block_slice_kernel, (const void*)oz_gemm_kernel<OZ_NARROW16>};
+                       (const void*)oz_block_slice_kernel, (const void*)oz_gemm_kernel<OZ_NARROW16>,
+                       (const void*)gj_cluster_kernel, (const void*)pf_cluster_kernel, (const void*)pf_small_kernel,
+                       (const void*)amp_solve_kernel, (const void*)gram_eig_kernel, (const void*)oz_gemm_kernel<OZ_WIDE>};
     const int nk = (int)(sizeof(k) / sizeof(k[0]));
     if (!limit || !expected || n_out < 1 || n_out > nk) return SGS_EINVAL;
     set_kernel_attributes();
