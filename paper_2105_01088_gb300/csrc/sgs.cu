@@ -1305,8 +1305,23 @@ std::mutex g_tune_mu;
 // number of matrices, which a chunked or pair-sharded instance of the same shape has fewer of
 std::map<std::array<int, 6>, std::array<int, 2>> g_tune_cache;
 
-// Time the candidate widths on the instance's own pairs (CUDA events on the context
-// stream, best of two), keep the fastest; a shape already timed in this process reuses
+// an instance's side stream and the events of its forks, made on first use
+cudaError_t make_side_stream(Instance& I) {
+    cudaError_t e = cudaSuccess;
+    if (!I.st2) e = cudaStreamCreateWithFlags(&I.st2, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !I.ev_fork) e = cudaEventCreateWithFlags(&I.ev_fork, cudaEventDisableTiming);
+    if (e == cudaSuccess && !I.ev_join) e = cudaEventCreateWithFlags(&I.ev_join, cudaEventDisableTiming);
+    return e;
+}
+void drop_side_stream(Instance& I) {
+    if (I.st2) cudaStreamDestroy(I.st2);
+    if (I.ev_fork) cudaEventDestroy(I.ev_fork);
+    if (I.ev_join) cudaEventDestroy(I.ev_join);
+    I.st2 = nullptr; I.ev_fork = nullptr; I.ev_join = nullptr;
+}
+
+// Time the candidate widths on the instance's own pairs as a step launches them (CUDA events on the
+// context stream, best of two), keep the fastest; a shape already timed in this process reuses
 // its widths.  Results change only by rounding.
 sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     if (I.P == 0) return SGS_OK;
@@ -1345,14 +1360,22 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
         }
         return best;
     };
+    // a step inverts the pairs in two halves on two streams where it is neither chunked nor sharded, and which form
+    // the panels take depends on the matrices of a half
+    const bool split = I.nch() == 1 && I.shard_world == 1, borrowed = I.st2 != nullptr;
+    const std::vector<double> flops(c->stage_flops, c->stage_flops + SGS_N_STAGES);     // the trials are not profiled
+    if (split && make_side_stream(I) != cudaSuccess) {
+        c->err = "autotune: no side stream";
+        status = SGS_ECUDA;
+    }
     int gj = I.gj_b, pf = I.pf_bs;
     float best = 1e30f;
     std::vector<int> tried = gj_candidates(I.n);
     if (std::find(tried.begin(), tried.end(), I.gj_def) == tried.end()) tried.push_back(I.gj_def);   // cluster form only
     for (int b : tried) {
-        if (b > I.gj_cap && b != I.gj_def) continue;
+        if (status != SGS_OK || (b > I.gj_cap && b != I.gj_def)) continue;
         if ((status = set_panel_pointers(c, I, b, pf)) != SGS_OK) break;
-        const float t = timed([&] { return cudaSuccess; }, [&] { return pair_inverse(c, I, st); });
+        const float t = timed([&] { return cudaSuccess; }, [&] { return pair_factors(c, I, st, split); });
         if (t < best) { best = t; gj = b; }
     }
     // the chunk with the most phase Pfaffians (the first pairs, those of state 0, have none); where a CTA takes
@@ -1362,8 +1385,7 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     if (status == SGS_OK && I.Ppf > 0 && !pf_small(I.n, I.cpfcnt())) {
         status = set_panel_pointers(c, I, gj, pf);
         cudaError_t e = cudaSuccess;
-        if (status == SGS_OK) e = pair_inverse(c, I, st);
-        if (e == cudaSuccess) e = delta_range(c, I, 0, I.ccnt(), st, 0);
+        if (status == SGS_OK) e = pair_factors(c, I, st);
         if (e != cudaSuccess) { c->err = std::string("autotune: ") + cudaGetErrorString(e); status = SGS_ECUDA; }
         best = 1e30f;
         for (int b : pf_candidates(I.n)) {
@@ -1376,6 +1398,11 @@ sgs_status autotune_instance(sgs_ctx* c, Instance& I) {
     I.cur = 0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (!borrowed) {             // an instance owns these from its first step on
+        cudaStreamSynchronize(st);
+        drop_side_stream(I);
+    }
+    std::copy(flops.begin(), flops.end(), c->stage_flops);
     c->prof = prof;
     if (status != SGS_OK) return status;
     if ((status = set_panel_pointers(c, I, gj, pf)) != SGS_OK) return status;
@@ -1781,10 +1808,7 @@ cudaError_t step_instance(sgs_ctx* c, Instance& I, cudaStream_t st) {
         if (e == cudaSuccess) e = update_pass(c, I, st);
         return e;
     }
-    cudaError_t e = cudaSuccess;
-    if (!I.st2) e = cudaStreamCreateWithFlags(&I.st2, cudaStreamNonBlocking);
-    if (e == cudaSuccess && !I.ev_fork) e = cudaEventCreateWithFlags(&I.ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess && !I.ev_join) e = cudaEventCreateWithFlags(&I.ev_join, cudaEventDisableTiming);
+    cudaError_t e = make_side_stream(I);
     if (e != cudaSuccess) return e;
     I.cur = 0;
     const int M = I.M, ni = std::max(I.nimp, 1);
@@ -2551,9 +2575,7 @@ void sgs_free(sgs_ctx* c) {
         c->release_instance(I);
         if (I.st) cudaStreamDestroy(I.st);
         if (I.join) cudaEventDestroy(I.join);
-        if (I.st2) cudaStreamDestroy(I.st2);
-        if (I.ev_fork) cudaEventDestroy(I.ev_fork);
-        if (I.ev_join) cudaEventDestroy(I.ev_join);
+        drop_side_stream(I);
     }
     if (c->fork) cudaEventDestroy(c->fork);
     c->release_all();
