@@ -41,7 +41,7 @@
 // over each (a warp per row where the operand's K rows are contiguous and long,
 // else a block of whole rows at a time through shared memory), then the product
 // kernel.  It takes 128 x 32 output tiles with CTAs of 10 warps (256 TMEM
-// columns, 97 KB of shared memory), two to an SM, or, for K > 240, 128 x 64 tiles with
+// columns, 97 KB of shared memory), two to an SM, or, for K > 224, 128 x 64 tiles with
 // one CTA of 18 warps an SM (all of its TMEM, 225 KB), which load 3/5 of the bytes per
 // output.  Each CTA runs over every (grid)-th tile, so that CTAs side by side work on
 // tiles side by side and share their slices in L2 (consecutive tiles per CTA read them
@@ -86,8 +86,7 @@ namespace sgs {
 #define OZ_SLAB_A (OZ_BM * 128)
 
 // Kernel shapes: BN output columns per tile (TMEM: 8 BN columns), EPIW epilogue warps, RING A-ring depth
-// (units), BBUF B buffers, CTAS CTAs per SM.  A 128 x 64 tile takes all of an SM's TMEM and shared memory;
-// with its epilogue serialised after the main loop it measured about half the throughput at K = 512.
+// (units), BBUF B buffers, CTAS CTAs per SM.  A 128 x 64 tile takes all of an SM's TMEM and shared memory.
 template <int BN, int EPIW, int RING, int BBUF, int CTAS> struct OzCfg {
     static constexpr int SLAB_B = BN * 128;
     static constexpr int SMEM = BBUF * OZ_S * SLAB_B + RING * OZ_UNIT * OZ_SLAB_A + 1024;
@@ -921,13 +920,16 @@ inline int oz_sms() {
 
 // Tile width of a product: OZ_NARROW16's, OZ_NARROW's, or OZ_WIDE's for long sums with enough tiles that a last
 // partial round of whole SMs costs less than the wide tile gains.  Narrow / wide, us: 105 antisymmetric products of
-// 804^2 at K = 512 1162 / 945, at 292 1057 / 810; 45 of 388^2 at 388 201 / 164; 120 general of 244^2 at 244 152 / 141;
-// 120 Gauss-Jordan updates of 512 x 128 at K = 128 96 / 131;
-// general 512^2 at K = 512: 160 wide tiles 58 / 64, 192 61 / 64, 256 72 / 65, 320 99 / 90; at K = 256: 160 tiles
-// 37 / 44, 256 45 / 45.
+// 804^2 at K = 512 1162 / 945, at 292 1057 / 810; 45 of 388^2 at 388 201 / 164; general 512^2 at K = 512: 160 wide
+// tiles 58 / 64, 192 61 / 64, 256 72 / 65, 320 99 / 90.  The two cross where a sum has 15 steps of 16 (K > 224).  190
+// pairs' V = D W (general) and X = V D (antisymmetric), n = K, with their slicing:
+//   K    160          192          208          224          228          236          240          256
+//   V    206 / 228    231 / 235    287 / 288    292 / 291    363 / 315    328 / 296    321 / 294    315 / 291
+//   X    201 / 222    222 / 227    261 / 272    266 / 276    319 / 290    289 / 279    286 / 278    282 / 277
+// Gauss-Jordan updates at K = 128 (120 of 512 x 128) 96 / 131; at K = 240 (120 of 472 x 232, the whole inverse) 7062 / 7005.
 inline int oz_width(const GemmBatch& g, int bc) {
     if (g.n <= 16) return 16;
-    return g.k > 240 && (long long)oz_tiles(g, 64) * bc * 2 >= 3 * oz_sms() ? 64 : 32;
+    return g.k > 224 && (long long)oz_tiles(g, 64) * bc * 2 >= 3 * oz_sms() ? 64 : 32;
 }
 
 // the product kernel on slices in place (layout L) for batch entries b0 .. b0 + bc - 1;
