@@ -78,9 +78,11 @@ typedef enum {
  *    those maxima is less accurate than the K u sum_k |A_ik||B_kj| of a native
  *    FP64 dot product.
  *  - SGS_FP64_FMA: FP64 fused multiply-adds on the CUDA cores (the error of a
- *    native FP64 dot product), about 10x slower on GB300 at 2N = 512.  In SGS_FP64 instances of either
- * path, products of few operations (3e6 multiply-adds a launch) run on the FP64
- * pipe: the elementwise bound holds there. */
+ *    native FP64 dot product), about 10x slower on GB300 at 2N = 512.
+ * An instance's products of few operations (3e6 multiply-adds a launch, 4e6 in
+ * the inverse's updates) run on the FP64 pipe on either path, with a native dot
+ * product's error; in the mixed forms (every precision but SGS_FP64) the
+ * products behind S^{-1} and Im Delta stay on the selected path. */
 typedef enum {
     SGS_FP64_EMULATED = 0,
     SGS_FP64_FMA = 1

@@ -810,7 +810,7 @@ sgs_status setup_instance(sgs_ctx* c, Instance& I, const sgs_model& m, const sgs
             I.u_ok = true;
         }
     }
-    I.oz.small_fma = I.oz2.small_fma = true;
+    I.oz.small_fma = I.oz2.small_fma = true;      // in every precision; factor_oz withdraws it in the mixed forms
     if (I.fp64_path == SGS_FP64_EMULATED) {
         // emulated FP64 products: slice scratch for one batch chunk, and one for the side stream
         const size_t b = oz_scratch_bytes(n, M, I.oz_cap, Pc);
@@ -960,7 +960,8 @@ cudaError_t pf_panel(const PfPanelArgs& a, int batch, cudaStream_t st) {
 // (a 64 x 64 x 64 product of 4 states in 3.5 us) before the emulated form's three launches, 25 to 40 us on
 // few tiles, are through.  Measured with the line at 0 (all emulated), 1, 3, 6 and 12 million FMAs: four steps
 // at 2N = 64, M = 4 take 4.71, 3.95, 2.50, 2.49 and 2.51 ms; serving at 2N up to 164 4.20, 4.19, 4.21, 4.24
-// and 4.33.
+// and 4.33.  It rounds every partial sum, where the emulated form sums its digits exactly and rounds once: a native dot
+// product's error, n u instead of u at n <= 144, which against 64 bits moved four steps at 2N = 64 from 1.9e-14 to 4.2e-14.
 constexpr double SMALL_FMAS = 3e6;
 bool small_product(const OzBuf* oz, const GemmBatch& g) { return oz && oz->small_fma && gemm_fmas(g) <= SMALL_FMAS; }
 // the same for a Gauss-Jordan update (one launch against two, 18 us on few tiles): (E, G, h) at 2N = 164, M = 6
