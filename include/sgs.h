@@ -411,9 +411,10 @@ sgs_status sgs_probe_wait(unsigned long long limit_ns, double* elapsed_ms);
  * 6 emulated FP64 product, 7 block slicer, 8 emulated FP64 product of
  * 16-column tiles, 9 Gauss-Jordan panel and 10 Pfaffian panel by clusters,
  * 11 phase Pfaffian in one CTA, 12 amplitude solve, 13 Gram eigenvalues,
- * 14 emulated FP64 product of 64-column tiles; n_out <= 15) it writes the limit
- * in force to limit[i] and the device's opt-in maximum less the kernel's
- * static shared memory to expected[i]. */
+ * 14 emulated FP64 product of 64-column tiles, 15 Gauss-Jordan panel of large
+ * batches; n_out <= 16) it writes the limit in force to limit[i] and the
+ * device's opt-in maximum less the kernel's static shared memory to
+ * expected[i]. */
 sgs_status sgs_kernel_smem_limits(int n_out, int* limit, int* expected);
 
 /* Building blocks with host buffers, for tests and external callers.

@@ -150,10 +150,11 @@ __device__ __forceinline__ void gj_panel_copy(double* W, double* panel, int n, i
 // The end of a Gauss-Jordan panel: its row interchanges (s_rows, s_src, nr) applied to columns c0 .. c1 - 1
 // of W other than the panel's, staged through stage[0 .. cap), a block of columns at a time; the update
 // operand T of those columns (the pivot rows, panel columns zeroed), if asked for.
+template <int LOADS>
 __device__ void gj_panel_finish(const GJPanelArgs& a, double* W, int b, double* stage, int cap, const int* s_rows,
                                 const int* s_src, int nr, int c0, int c1) {
     const int n = a.n, k0 = a.k0, bb = a.bb;
-    // a warp per row, lanes along the columns, four loads in flight per lane
+    // a warp per row, lanes along the columns, LOADS loads in flight per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (nr > 0) {
         const int qc = min(c1 - c0, cap / nr);
@@ -161,14 +162,14 @@ __device__ void gj_panel_finish(const GJPanelArgs& a, double* W, int b, double* 
             const int qn = min(qc, c1 - q0);
             for (int e = warp; e < nr; e += nw) {
                 const double* src = W + (size_t)s_src[e] * n + q0;
-#pragma unroll 4
+#pragma unroll LOADS
                 for (int x = lane; x < qn; x += 32)
                     if ((unsigned)(q0 + x - k0) >= (unsigned)bb) stage[e * qn + x] = src[x];
             }
             __syncthreads();
             for (int e = warp; e < nr; e += nw) {
                 double* dst = W + (size_t)s_rows[e] * n + q0;
-#pragma unroll 4
+#pragma unroll LOADS
                 for (int x = lane; x < qn; x += 32)
                     if ((unsigned)(q0 + x - k0) >= (unsigned)bb) dst[x] = stage[e * qn + x];
             }
@@ -196,9 +197,11 @@ __device__ __forceinline__ void warp_argmax(long long& key, int& idx) {
     key = (long long)(((unsigned long long)mh << 32) | ml) - 1;
 }
 
-// One CTA per matrix, for batches that fill the SMs.  Four CTAs fit an SM (32 registers a thread), so that up to 608
-// matrices are one wave: at two (56 registers) 400 inverses of 64 x 64 took 767 us, at four 602.
-__global__ void __launch_bounds__(512, 4) gj_panel_kernel(GJPanelArgs a) {
+// One CTA per matrix, CTAS of them on an SM.  Four (32 registers a thread) make up to 608 matrices one wave: at two, 400
+// inverses of 64 x 64 took 767 us, at four 602.  Batches of one wave at two take the form with 56 registers: 16 inverses
+// of 64 x 64 379 us against 397, 64 of 200 x 200 2768 against 2831.
+template <int CTAS>
+__global__ void __launch_bounds__(512, CTAS) gj_panel_kernel(GJPanelArgs a) {
     extern __shared__ double sm[];
     const int ps = a.bb + 1;                   // odd row stride: column walks hit distinct banks
     double* panel = sm;                        // n x ps
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(512, 4) gj_panel_kernel(GJPanelArgs a) {
         gj_det(a, b, s_pabs, s_neg != 0, s_sing != 0);
     }
     __syncthreads();
-    gj_panel_finish(a, W, b, panel, n * ps, s_rows, s_src, s_nr, 0, n);
+    gj_panel_finish<CTAS == 2 ? 8 : 4>(a, W, b, panel, n * ps, s_rows, s_src, s_nr, 0, n);
 }
 
 // The panel by a cluster of C CTAs per matrix (grid batch x C): CTA r holds rows r ch .. r ch + ch - 1 of
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(288) gj_cluster_kernel(GJPanelArgs a, int C, i
         gj_det(a, b, s_pabs, neg != 0, singular != 0);
     }
     const int cw = (n + C - 1) / C, c0 = min(n, rank * cw), c1 = min(n, c0 + cw);
-    gj_panel_finish(a, W, b, sm, GJC_STAGE, s_rows, s_src, s_nr, c0, c1);
+    gj_panel_finish<8>(a, W, b, sm, GJC_STAGE, s_rows, s_src, s_nr, c0, c1);
 }
 
 // shared memory of gj_cluster_kernel (bytes)

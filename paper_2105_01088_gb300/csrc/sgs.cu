@@ -382,7 +382,7 @@ std::vector<int> gj_candidates(int n) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, gj_panel_kernel);
+    cudaFuncGetAttributes(&fa, gj_panel_kernel<2>);
     const int limit = optin - (int)fa.sharedSizeBytes;
     std::vector<int> v;
     // between the powers of two: at n = 512 a panel of 12 columns fits four panel CTAs per SM
@@ -849,7 +849,8 @@ void set_kernel_attributes() {
     if (g_attr_done[dev]) return;
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    raise_smem_limit(gj_panel_kernel, optin);
+    raise_smem_limit(gj_panel_kernel<2>, optin);
+    raise_smem_limit(gj_panel_kernel<4>, optin);
     raise_smem_limit(pf_panel_kernel, optin);
     raise_smem_limit(gj_cluster_kernel, optin);
     raise_smem_limit(pf_cluster_kernel, optin);
@@ -930,6 +931,14 @@ int pf_cluster(int live, int batch, int bs) {
 // panels' clusters; n > 152 does not fit.
 bool pf_small(int n, int batch) { return n <= PACKED_PF_MAX && batch >= n - 108; }
 
+// the Gauss-Jordan panel by one CTA per matrix
+cudaError_t gj_panel_one(const GJPanelArgs& a, int batch, cudaStream_t st) {
+    const size_t smem = (size_t)a.n * (a.bb + 1) * sizeof(double) + a.bb * sizeof(double);
+    if (batch > 2 * oz_sms()) gj_panel_kernel<4><<<batch, 512, smem, st>>>(a);
+    else gj_panel_kernel<2><<<batch, 512, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
 // the Gauss-Jordan panel of columns a.k0 .. a.k0 + a.bb - 1
 cudaError_t gj_panel(const GJPanelArgs& a, int batch, cudaStream_t st) {
     counted();
@@ -939,8 +948,7 @@ cudaError_t gj_panel(const GJPanelArgs& a, int batch, cudaStream_t st) {
         return launch_cluster(gj_cluster_kernel, batch * C, cluster_threads(ch), gjc_smem(a.bb, C, ch), C, st, a, C, ch,
                               threads_per_row(ch));
     }
-    gj_panel_kernel<<<batch, 512, (size_t)a.n * (a.bb + 1) * sizeof(double) + a.bb * sizeof(double), st>>>(a);
-    return cudaGetLastError();
+    return gj_panel_one(a, batch, st);
 }
 
 // the Pfaffian panel of elimination steps a.k0 / 2 .. a.k0 / 2 + a.bs - 1
@@ -1027,7 +1035,7 @@ cudaError_t launch_gj(sgs_ctx* c, int n, int batch, int bsz, double** W, double*
     for (int k0 = 0; k0 < n; k0 += bsz) {
         const int bb = std::min(bsz, n - k0);
         GJPanelArgs a{W, T, piv, logdet, dsign, err, n, k0, bb, tiny};
-        gj_panel_kernel<<<batch, 512, (size_t)n * (bb + 1) * sizeof(double) + bb * sizeof(double), st>>>(a);
+        if (const cudaError_t pe = gj_panel_one(a, batch, st); pe != cudaSuccess) return pe;
         counted();
         GemmBatch g = gb_basic(n, n, bb, W, n, T, n, W, n, batch);
         g.offA = k0;
@@ -2705,12 +2713,13 @@ sgs_status sgs_probe_wait(unsigned long long limit_ns, double* elapsed_ms) {
 }
 
 sgs_status sgs_kernel_smem_limits(int n_out, int* limit, int* expected) {
-    const void* k[] = {(const void*)gj_panel_kernel, (const void*)pf_panel_kernel, (const void*)renyi_pf_kernel,
+    const void* k[] = {(const void*)gj_panel_kernel<2>, (const void*)pf_panel_kernel, (const void*)renyi_pf_kernel,
                        (const void*)gemm_tma_kernel<TC_TF32>, (const void*)gemm_tma_kernel<TC_BF16>,
                        (const void*)gemm_tma_kernel<TC_3XTF32>, (const void*)oz_gemm_kernel<OZ_NARROW>,
                        (const void*)oz_block_slice_kernel, (const void*)oz_gemm_kernel<OZ_NARROW16>,
                        (const void*)gj_cluster_kernel, (const void*)pf_cluster_kernel, (const void*)pf_small_kernel,
-                       (const void*)amp_solve_kernel, (const void*)gram_eig_kernel, (const void*)oz_gemm_kernel<OZ_WIDE>};
+                       (const void*)amp_solve_kernel, (const void*)gram_eig_kernel, (const void*)oz_gemm_kernel<OZ_WIDE>,
+                       (const void*)gj_panel_kernel<4>};
     const int nk = (int)(sizeof(k) / sizeof(k[0]));
     if (!limit || !expected || n_out < 1 || n_out > nk) return SGS_EINVAL;
     set_kernel_attributes();

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 def test_limits():
     lim = sgs.smem_limits()
-    assert len(lim) == 15
+    assert len(lim) == 16
     packed = 152 * 151 // 2 * 18 + 4 * 152 * 8 + 16
     need = {2: packed, 9: 200 * 1024, 10: 220 * 1024, 11: packed, 12: 3 * 64 * 65 * 16, 13: 64 * 65 * 16,
             14: 2 * 8 * 64 * 128 + 3 * 2 * 128 * 128 + 1024}
