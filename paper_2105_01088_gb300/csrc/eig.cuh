@@ -560,7 +560,8 @@ __device__ __noinline__ bool amp_direct(const AmpArgs& a, cplx* sm, double* lr, 
     return !(most - mine > __double2hiint(1.0) - least);
 }
 
-// where in scratch the solve marks its route (1: direct), before the two values of gram_eig_kernel
+// where in scratch the solve marks its route (0: Jacobi, 1: direct; 2: gram_eig_kernel has run since), before the two
+// values of gram_eig_kernel
 __host__ __device__ inline size_t gram_mark(int M) { return 6 * (size_t)(2 * M) * (2 * M) + 2 * M; }
 
 // dynamic shared memory of amp_solve_kernel
@@ -644,14 +645,18 @@ inline size_t gram_smem(int M) { return (size_t)M * (M + 1) * sizeof(cplx); }
 // The smallest and the largest eigenvalue of G of the last amplitude solve, for the health report: after a Jacobi
 // solve they are on its diagonal, after the direct route (which leaves the embedding of G in scratch) they come from
 // the tridiagonal form by multisection, as the energy does.  Jacobi for them took about half of what the direct route
-// saves a step.  They go to scratch behind the route's mark.
+// saves a step.  They go to scratch behind the solve's mark, which then says that they are there.
 __global__ void __launch_bounds__(AMP_THREADS) gram_eig_kernel(double* scratch, int M) {
     extern __shared__ double amp_sm[];
     __shared__ AmpTri t;
     cplx* B = reinterpret_cast<cplx*>(amp_sm);
     const int m = 2 * M, ld = M + 1, tid = threadIdx.x;
     double* mark = scratch + gram_mark(M);
-    if (*mark != 1.0) {
+    const double route = *mark;
+    if (route == 2.0) return;
+    __syncthreads();
+    if (tid == 0) *mark = 2.0;
+    if (route != 1.0) {
         if (tid == 0) {
             double lo = INFINITY, hi = 0.0;
             for (int j = 0; j < m; j++) {
